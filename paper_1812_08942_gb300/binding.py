@@ -127,13 +127,15 @@ def _prec_of(dtype):
 
 
 class Graph:
-    """Owns a gr_ctx handle; destroyed with the object."""
+    """Owns a gr_ctx handle; destroyed with the object.  stream: the CUDA
+    stream its work runs on (the current one when it was created)."""
 
-    def __init__(self, handle, n, m, device):
+    def __init__(self, handle, n, m, device, stream=None):
         self.handle = ctypes.c_void_p(handle)
         self.n = int(n)
         self.m = int(m)
         self.device = device
+        self.stream = stream
 
     def __del__(self):
         h = getattr(self, "handle", None)
@@ -143,6 +145,13 @@ class Graph:
 
     def close(self):
         self.__del__()
+
+
+def _join(g):
+    """Calls that queue their last kernels without waiting: a caller on another
+    stream than g's gets its results, and may free its inputs, as after a wait."""
+    if g.stream != torch.cuda.current_stream(g.device).cuda_stream:
+        torch.cuda.synchronize(g.device)
 
 
 # ---------------------------------------------------------------------------
@@ -165,10 +174,11 @@ def graph_reduce_create(n, u, v, w, device=None) -> Graph:
     assert u.dtype == torch.int32 and v.dtype == torch.int32 and w.dtype == torch.float64
     h = ctypes.c_void_p()
     with torch.cuda.device(dev):
+        stream = _stream(dev)
         st = lib.graph_reduce_create(ctypes.byref(h), int(n), int(u.numel()), _ptr(u), _ptr(v), _ptr(w),
-                                     1 if on_host else 0, _stream(dev))
+                                     1 if on_host else 0, stream)
     _check(st, None)
-    return Graph(h.value, n, u.numel(), dev)
+    return Graph(h.value, n, u.numel(), dev, stream.value or 0)
 
 
 def graph_reduce_smooth(g: Graph, X, sweeps, omega=0.7, seed=0, level=0):
@@ -259,7 +269,7 @@ def graph_reduce_coarsen(g: Graph, agg, nc) -> Graph:
     n = ctypes.c_int64()
     m = ctypes.c_int64()
     load().graph_reduce_get_info(h, ctypes.byref(n), ctypes.byref(m))
-    return Graph(h.value, n.value, m.value, g.device)
+    return Graph(h.value, n.value, m.value, g.device, g.stream)
 
 
 def graph_reduce_get_edges(g: Graph, on_host=False, out=None):
@@ -325,7 +335,7 @@ def graph_reduce_multilevel(g: Graph, params: ReduceParams, want_stats=True):
         n = ctypes.c_int64()
         m = ctypes.c_int64()
         load().graph_reduce_get_info(arr[i], ctypes.byref(n), ctypes.byref(m))
-        levels.append(Graph(arr[i], n.value, m.value, g.device))
+        levels.append(Graph(arr[i], n.value, m.value, g.device, g.stream))
     _check(st, g.handle)
     out = []
     if want_stats:
@@ -366,6 +376,7 @@ def graph_reduce_reduce_data(levels, F, mean=False):
     st = load().graph_reduce_reduce_data(arr, len(levels), _ptr(F), int(F.shape[1]),
                                          1 if F.dtype == torch.float64 else 0, 1 if mean else 0, _ptr(out))
     _check(st, levels[0].handle)
+    _join(levels[0])
     return out
 
 

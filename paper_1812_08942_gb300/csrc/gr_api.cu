@@ -423,6 +423,7 @@ void graph_reduce_destroy(gr_ctx* c) {
     for (void* p : ptrs)
         if (p) cudaFreeAsync(p, s);
     c->ws.release();
+    if (c->event) cudaEventDestroy(c->event);
     delete c;
 }
 

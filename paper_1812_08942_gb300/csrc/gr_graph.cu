@@ -721,11 +721,6 @@ gr_status coarsen_impl(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx** out) 
 // ---------------------------------------------------------------------------
 // Map composition (fine -> coarsest)
 // ---------------------------------------------------------------------------
-struct MapChain {
-    const int32_t* map[64];
-    int count;
-};
-
 __global__ void k_compose(MapChain chain, int64_t n, int32_t* __restrict__ out) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -734,10 +729,10 @@ __global__ void k_compose(MapChain chain, int64_t n, int32_t* __restrict__ out) 
     out[i] = x;
 }
 
-gr_status compose_impl(gr_ctx* const* levels, int nlevels, int32_t* out) {
+gr_status map_chain(gr_ctx* const* levels, int nlevels, MapChain* out) {
     gr_ctx* c0 = levels[0];
     if (nlevels > 64) return set_error(c0, GR_EINVAL, "compose: at most 64 levels");
-    MapChain ch;
+    MapChain& ch = *out;
     ch.count = nlevels;
     for (int l = 0; l < nlevels; ++l) {
         if (!levels[l] || !levels[l]->parent_map)
@@ -746,6 +741,14 @@ gr_status compose_impl(gr_ctx* const* levels, int nlevels, int32_t* out) {
             return set_error(c0, GR_EINVAL, "compose: levels do not chain");
         ch.map[l] = levels[l]->parent_map;
     }
+    return GR_OK;
+}
+
+gr_status compose_impl(gr_ctx* const* levels, int nlevels, int32_t* out) {
+    gr_ctx* c0 = levels[0];
+    MapChain ch;
+    const gr_status st = map_chain(levels, nlevels, &ch);
+    if (st != GR_OK) return st;
     int64_t n = c0->parent_n;
     if (n > 0) {
         k_compose<<<(unsigned)ceil_div(n, TB), TB, 0, c0->stream>>>(ch, n, out);

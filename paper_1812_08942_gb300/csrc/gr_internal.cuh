@@ -113,6 +113,7 @@ struct gr_ctx {
     // mapping from the parent level (coarse contexts only)
     int32_t* parent_map = nullptr;
     int64_t parent_n = 0;
+    cudaEvent_t event = nullptr;  // marks a readback the host waits for while later work is queued
     gr::Workspace ws;
     std::string last_error;
 };
@@ -190,6 +191,29 @@ cudaError_t degree_scale(gr_ctx* c);
 // for per-row sorting, sets *too_long and leaves cc untouched.
 gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, bool* too_long);
 
+// Composition of up to 64 node maps: label = map[count-1][... map[0][i]]
+struct MapChain {
+    const int32_t* map[64];
+    int count;
+};
+
+// The members of every label of a node map in ascending node id (gr_group.cu).
+// group_begin counts the labels of n nodes in [0, nc) and starts the readback
+// of what group_finish decides by; work queued on the stream between the two
+// runs while the host waits.  After group_finish without *bad (a label out of
+// range; nothing more was launched) members[start[A] .. start[A + 1]) are
+// label A's nodes.  Scratch: workspace slot `slot` of c (kept until the
+// next job there) and, when a group is large, the sort slots.
+struct GroupJob {
+    int64_t n = 0, nc = 0;
+    int32_t* start = nullptr;      // nc + 1
+    uint32_t* members = nullptr;   // n
+    int2* place = nullptr;         // n: (label, place among the label's claims)
+    int32_t* host = nullptr;       // pinned: [0] bad label, [1] largest group
+};
+gr_status group_begin(gr_ctx* c, int slot, const MapChain& map, int64_t n, int64_t nc, GroupJob* job);
+gr_status group_finish(gr_ctx* c, GroupJob* job, bool* bad);
+
 // Slot of the calling thread in a list that grows by one entry per thread
 // with `keep` set: one atomic per block, entries in thread order within the
 // block; -1 if !keep.  Every thread of the block must call it (it holds
@@ -255,6 +279,8 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
                          int64_t max_proposals, int32_t* agg, int64_t* nc_out, int64_t* proposals_out);
 gr_status coarsen_impl(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx** out);
 gr_status compose_impl(gr_ctx* const* levels, int nlevels, int32_t* out);
+// the parent maps of a chain of coarse contexts, checked to chain
+gr_status map_chain(gr_ctx* const* levels, int nlevels, MapChain* ch);
 gr_status reduce_data_impl(gr_ctx* const* levels, int nlevels, const void* F, int d, int f64, int mean,
                            void* F_out);
 gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normalized, int galerkin_mass,
