@@ -408,6 +408,7 @@ def graph_reduce_loss_fwd(fine: Graph, coarse: Graph, agg, X, w_c, sweeps_c, ome
     st = load().graph_reduce_loss_fwd(fine.handle, coarse.handle, _ptr(agg), _ptr(X), K, _ptr(w_c), int(sweeps_c),
                                       float(omega), _ptr(loss), _ptr(saved))
     _check(st, fine.handle)
+    _join(fine)
     return loss, saved
 
 

@@ -9,473 +9,850 @@
 //   y_{s+1} = (1-w) y_s + w D_c^-1 A_c y_s          (isolated node: unchanged)
 //   R_c[k]  = y^T L_c y / sum_A M_A (y_A - mu_k)^2,  mu_k = sum M y / sum M
 //   loss    = (1/K) sum_k (R_c[k]/R_f[k] - 1)^2
-// Vectors are FP32; every global sum is reduced in FP64 in a fixed order.
-#include "gr_internal.cuh"
+// Vectors are FP32; sums are FP32 per lane and FP64 from the warp level up, in
+// a fixed order.
+//
+// Layout.  Every pass over vectors is a pass over rows in which G = K / 4
+// lanes hold one row, a 16-byte chunk each (short rows: 32 / G rows a warp),
+// or a warp holds one row, its sub-groups taking slots in turn (long rows).
+// A thread per entry or per edge, reading K scalars 4 bytes at a time, took
+// 17 us for a sweep of the 32,768-node reduced mesh (K = 24) and 200 us for
+// the fine quotients of the 128^3 mesh.  The weights are put in slot order
+// once per call, so that a sweep reads them with the columns instead of
+// through the edge ids.  Column sums end in the kernel that makes them (last
+// block); one-block kernels adding 304 rows of partials took 49 us each,
+// eight per loss and gradient.
+#include "gr_loss.cuh"
+#include "gr_sweep.cuh"
+#include "gr_vec.cuh"
 
 namespace gr {
 
-constexpr int LS_THREADS = 256;
+namespace {
 
-__global__ void k_i32_to_i64_n(const int32_t* a, int64_t n, int64_t* b) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = a[i];
-    else if (i == n) b[i] = 0;
-}
+constexpr int LT = 256;
+constexpr int LW = LT / 32;
+// Blocks per SM of the row passes, which is also their grid: a larger grid
+// would leave its later blocks to a second wave over rows that have left L2
+// (the fine pass read 427 MB for 301 in 181 us).
+constexpr int ROW_BLOCKS = 6;
 
-// one block: FP64 sum of n floats in a fixed order
-__global__ void k_sum_f32(const float* a, int64_t n, double* out) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)a[i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int j = 0; j < (int)blockDim.x; ++j) t += sh[j];
-        *out = t;
+// lanes of a warp over rows and 16-byte chunks of a row
+template <int K, bool LONG>
+struct RowLanes {
+    static constexpr int G = K / 4, GP = next_pow2_c(G);
+    static constexpr int RPW = LONG ? 1 : 32 / G;   // rows per warp
+    static constexpr int TS = LONG ? 32 / GP : 1;   // sub-groups sharing a row's slots
+    int seg, q, t;
+    bool ok;
+    __device__ RowLanes() {
+        const int lane = threadIdx.x & 31;
+        seg = LONG ? 0 : lane / G;
+        q = LONG ? lane % GP : lane % G;
+        t = LONG ? lane / GP : 0;
+        ok = LONG ? q < G : seg < RPW;
+    }
+    __device__ bool writes() const { return ok && t == 0; }
+};
+
+__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+
+// f(w, x) for every slot of the lane's share of [b, e): x the chunk of the
+// slot's column in src; eight slots in flight (a reduced mesh's row of 14 in
+// two round trips), in slot order per lane
+template <int K, bool LONG, typename F>
+__device__ __forceinline__ void for_slots(const RowLanes<K, LONG>& m, int64_t b, int64_t e,
+                                          const int2* __restrict__ cw, const float* __restrict__ src, F f) {
+    constexpr int U = 8, TS = RowLanes<K, LONG>::TS;
+    if (!m.ok) return;
+    for (int64_t j = b + m.t; j < e; j += U * TS) {
+        int2 v[U];
+        float4 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + u * TS < e) v[u] = __ldg(cw + j + u * TS);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + u * TS < e) x[u] = ld4(src + (int64_t)v[u].x * K + m.q * 4);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + u * TS < e) f(__int_as_float(v[u].y), x[u]);
     }
 }
 
+// sum over a long row's sub-groups (every lane of the warp calls it)
+template <int K, bool LONG>
+__device__ __forceinline__ void join_row(float4& a) {
+    if constexpr (LONG) {
+#pragma unroll
+        for (int o = RowLanes<K, true>::GP; o < 32; o <<= 1) {
+            a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+            a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+            a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
+            a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
+        }
+    }
+}
 
-// Reduce K per-thread FP32 values over the block; write an FP64 partial.
-template <int K>
-__device__ void block_colsum(float (&v)[K], double* __restrict__ part) {
-    __shared__ double ws[LS_THREADS / 32][K];
+// Two column sums per lane (chunks s1, s2) into the block's partial row:
+// lanes of one chunk added in FP32, warps in FP64.  True in the last block,
+// with the totals in red (K of s1, then K of s2).
+template <int K, bool LONG>
+__device__ bool finish_cols(const RowLanes<K, LONG>& m, float4 s1, float4 s2, double* part, unsigned* counter,
+                            double* red) {
+    using L = RowLanes<K, LONG>;
+    __shared__ double ws[LW][2 * K];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float a[8] = {s1.x, s1.y, s1.z, s1.w, s2.x, s2.y, s2.z, s2.w};
+    constexpr int STEP = LONG ? L::GP : L::G, CNT = LONG ? L::TS : L::RPW;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float x = v[k];
+    for (int i = 0; i < 8; ++i) {
+        float t = m.ok ? a[i] : 0.f;
+        float acc = t;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) ws[warp][k] = (double)x;
+        for (int r = 1; r < CNT; ++r) acc += __shfl_sync(0xffffffffu, t, (lane + r * STEP) & 31);
+        a[i] = acc;
+    }
+    if (lane < L::G) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ws[warp][lane * 4 + i] = (double)a[i];
+            ws[warp][K + lane * 4 + i] = (double)a[4 + i];
+        }
     }
     __syncthreads();
-    if (threadIdx.x < K) {
-        double s = 0.0;
-        for (int w = 0; w < LS_THREADS / 32; ++w) s += ws[w][threadIdx.x];
-        part[(int64_t)blockIdx.x * K + threadIdx.x] = s;
+    if (threadIdx.x < 2 * K) {
+        double t = 0.0;
+        for (int w = 0; w < LW; ++w) t += ws[w][threadIdx.x];
+        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = t;
     }
+    __threadfence();
+    __syncthreads();
+    return finish_partials<K, LT>(part, gridDim.x, counter, red);
 }
 
-// out[j] = sum over blocks of part[b*NS + j]
-__global__ void k_finish_sums(const double* __restrict__ part, int nblocks, int NS,
-                              double* __restrict__ out) {
-    int j = threadIdx.x;
-    if (j >= NS) return;
-    // eight interleaved accumulators keep eight loads in flight (fixed order)
-    double a[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) a[u] = 0.0;
-    int b = 0;
-    for (; b + 7 < nblocks; b += 8) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] += part[(int64_t)(b + u) * NS + j];
+// R_f: per column sum_e w (x_u - x_v)^2 over the edges (p, v) of row p and
+// sum_p x_p^2, in one pass over the rows.
+template <int K, bool LONG>
+__global__ void __launch_bounds__(LT, ROW_BLOCKS) k_fine_quotients(int64_t n, const int64_t* __restrict__ eptr,
+                                                       const int32_t* __restrict__ ev, const double* __restrict__ ew,
+                                                       const float* __restrict__ X, double* part, unsigned* counter,
+                                                       float* __restrict__ Rf) {
+    __shared__ double red[LT];
+    const RowLanes<K, LONG> m;
+    constexpr int U = 2, TS = RowLanes<K, LONG>::TS, RPW = RowLanes<K, LONG>::RPW;
+    float4 num = make_float4(0.f, 0.f, 0.f, 0.f), den = num;
+    // 32-bit row and edge numbers (n, m < 2^31) keep the kernel at 4 blocks per SM or more
+    const unsigned rows = (unsigned)n, stride = ((gridDim.x * LT) >> 5) * RPW;
+    unsigned p = ((blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg;
+    if (!m.ok) p = rows;
+    unsigned b1 = 0, e1 = 0;  // the next row's edges, read one row ahead
+    if (p < rows) {
+        b1 = (unsigned)__ldg(eptr + p);
+        e1 = (unsigned)__ldg(eptr + p + 1);
     }
-    for (; b < nblocks; ++b) a[0] += part[(int64_t)b * NS + j];
-    out[j] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-}
-
-// sum_e w_e (x_u - x_v)^2 per column, over a canonical edge list
-template <int K>
-__global__ void __launch_bounds__(LS_THREADS) k_edge_quad(int64_t m, const int32_t* __restrict__ eu,
-                                                          const int32_t* __restrict__ ev,
-                                                          const double* __restrict__ w64,
-                                                          const float* __restrict__ w32,
-                                                          const float* __restrict__ X,
-                                                          double* __restrict__ part) {
-    float v[K];
+    const float* Xq = X + m.q * 4;
+    while (p < rows) {
+        const unsigned b = b1, e = e1;
+        const float4 x = ld4(Xq + (size_t)p * K);
+        p += stride;
+        if (p < rows) {
+            b1 = (unsigned)__ldg(eptr + p);
+            e1 = (unsigned)__ldg(eptr + p + 1);
+            if (m.q == 0 && m.t == 0 && b1 < e1) {
+                // the next row's edges into L1: no register waits for them
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(ev + b1));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(ew + b1));
+            }
+        }
+        if (m.t == 0) {
+            den.x = fmaf(x.x, x.x, den.x);
+            den.y = fmaf(x.y, x.y, den.y);
+            den.z = fmaf(x.z, x.z, den.z);
+            den.w = fmaf(x.w, x.w, den.w);
+        }
+        for (unsigned j = b + m.t; j < e; j += U * TS) {
+            float w[U];
+            float4 y[U];
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = 0.f;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t a = eu[e], b = ev[e];
-        const float w = w64 ? (float)w64[e] : w32[e];
+            for (int u = 0; u < U; ++u)
+                if (j + u * TS < e) {
+                    y[u] = ld4(Xq + (size_t)__ldg(ev + j + u * TS) * K);
+                    w[u] = f64_to_f32(__ldg(ew + j + u * TS));
+                }
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            float t = X[a * K + k] - X[b * K + k];
-            v[k] = fmaf(w * t, t, v[k]);
+            for (int u = 0; u < U; ++u)
+                if (j + u * TS < e) {
+                    float t = x.x - y[u].x;
+                    num.x = fmaf(w[u] * t, t, num.x);
+                    t = x.y - y[u].y;
+                    num.y = fmaf(w[u] * t, t, num.y);
+                    t = x.z - y[u].z;
+                    num.z = fmaf(w[u] * t, t, num.z);
+                    t = x.w - y[u].w;
+                    num.w = fmaf(w[u] * t, t, num.w);
+                }
         }
     }
-    block_colsum<K>(v, part);
+    if (finish_cols<K, LONG>(m, num, den, part, counter, red) && threadIdx.x < K)
+        Rf[threadIdx.x] = (float)(red[threadIdx.x] / red[K + threadIdx.x]);
 }
 
-// sum_i mass_i * (x_i - mu)^2 per column (mass NULL: 1, mu NULL: 0)
+// y0[A] = mean of the member rows, M_A = size.  A warp per aggregate: its
+// sub-groups take members in turn, four in flight each.
 template <int K>
-__global__ void __launch_bounds__(LS_THREADS) k_row_quad(int64_t n, const float* __restrict__ X,
-                                                         const float* __restrict__ mass,
-                                                         const double* __restrict__ mu,
-                                                         double* __restrict__ part) {
-    float v[K];
+__global__ void __launch_bounds__(LT) k_aggregate_means(int64_t nc, const int32_t* __restrict__ start,
+                                                        const uint32_t* __restrict__ members,
+                                                        const float* __restrict__ X, float* __restrict__ y0,
+                                                        float* __restrict__ mass) {
+    const RowLanes<K, true> m;
+    constexpr int U = 4, TS = RowLanes<K, true>::TS;
+    const int64_t A = ((int64_t)blockIdx.x * LT + threadIdx.x) >> 5;
+    if (A >= nc) return;
+    const int32_t b = start[A], e = start[A + 1];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (m.ok)
+        for (int32_t i = b + m.t; i < e; i += U * TS) {
+            float4 x[U];
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float mi = mass ? mass[i] : 1.f;
+            for (int u = 0; u < U; ++u)
+                if (i + u * TS < e) x[u] = ld4(X + (int64_t)__ldg(members + i + u * TS) * K + m.q * 4);
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            float t = X[i * K + k] - (mu ? (float)mu[k] : 0.f);
-            v[k] = fmaf(mi * t, t, v[k]);
+            for (int u = 0; u < U; ++u)
+                if (i + u * TS < e) {
+                    s.x += x[u].x;
+                    s.y += x[u].y;
+                    s.z += x[u].z;
+                    s.w += x[u].w;
+                }
+        }
+    join_row<K, true>(s);
+    const float c = (float)(e - b);
+    if (m.writes())
+        st4(y0 + A * K + m.q * 4, e > b ? make_float4(s.x / c, s.y / c, s.z / c, s.w / c) : s);
+    if ((threadIdx.x & 31) == 0) mass[A] = c;
+}
+
+// Weights in slot order beside their columns, and the row sums D; SCALE: also
+// the FP64 row sums dP and the smallest dG / dP over rows with dP > 0 (positive
+// doubles order like their bit patterns, so an integer minimum is exact).
+// P lanes per row, lane sums in slot order, combined by a fixed butterfly.
+template <int P, bool SCALE>
+__global__ void __launch_bounds__(LT) k_param_slots(int64_t nc, const int64_t* __restrict__ rowptr,
+                                                    const int32_t* __restrict__ col, const int32_t* __restrict__ eid,
+                                                    const float* __restrict__ w, int2* __restrict__ cw,
+                                                    float* __restrict__ D, double* __restrict__ dP,
+                                                    const double* __restrict__ dG,
+                                                    unsigned long long* __restrict__ lam) {
+    const int l = threadIdx.x % P;
+    const int64_t A = ((int64_t)blockIdx.x * LT + threadIdx.x) / P;
+    float s = 0.f;
+    double sd = 0.0;
+    if (A < nc) {
+        const int64_t e = rowptr[A + 1];
+        for (int64_t j = rowptr[A] + l; j < e; j += P) {
+            const float x = w[eid[j]];
+            cw[j] = make_int2(col[j], __float_as_int(x));
+            s += x;
+            if (SCALE) sd += f32_to_f64(x);
         }
     }
-    block_colsum<K>(v, part);
-}
-
-// sum_i mass_i x_i per column
-template <int K>
-__global__ void __launch_bounds__(LS_THREADS) k_row_sum(int64_t n, const float* __restrict__ X,
-                                                        const float* __restrict__ mass,
-                                                        double* __restrict__ part) {
-    float v[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float mi = mass[i];
+    for (int o = P / 2; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (SCALE) sd += __shfl_xor_sync(0xffffffffu, sd, o);
+    }
+    if (A < nc && l == 0) {
+        D[A] = s;
+        if (SCALE) dP[A] = sd;
+    }
+    if constexpr (SCALE) {
+        if (!lam) return;  // uniform
+        unsigned long long v = ~0ull;
+        if (A < nc && l == 0 && sd > 0.0) v = (unsigned long long)__double_as_longlong(dG[A] / sd);
 #pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = fmaf(mi, X[i * K + k], v[k]);
+        for (int o = 16; o >= P; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, v, o);
+            v = x < v ? x : v;
+        }
+        if ((threadIdx.x & 31) == 0 && v != ~0ull) atomicMin(lam, v);
     }
-    block_colsum<K>(v, part);
 }
 
-__global__ void k_agg_keys(int64_t n, const int32_t* __restrict__ agg, int64_t nc,
-                           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                           int32_t* __restrict__ cnt, int32_t* __restrict__ bad) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int32_t a = agg[i];
-    if (a < 0 || a >= nc) {
-        atomicExch(bad, 1);
-        a = 0;
+// One forward sweep: z = D^-1 A y (or y where D is not positive),
+// y1 = (1-w) y + w z.  SWEEP false: y1 = y, nothing written.  MEAN: the
+// mass-weighted column means of y1 end in mu.
+template <int K, bool LONG, bool SWEEP, bool MEAN>
+__global__ void __launch_bounds__(LT) k_param_sweep(int64_t n, const int64_t* __restrict__ rowptr,
+                                                    const int2* __restrict__ cw, const float* __restrict__ D,
+                                                    const float* __restrict__ y, float omega,
+                                                    float* __restrict__ z_out, float* __restrict__ y1,
+                                                    const float* __restrict__ mass, double* part, unsigned* counter,
+                                                    double* __restrict__ mu) {
+    __shared__ double red[LT];
+    const RowLanes<K, LONG> m;
+    constexpr int RPW = RowLanes<K, LONG>::RPW;
+    const float zero = 0.f, one_m = 1.f - omega;
+    float4 sy = make_float4(zero, zero, zero, zero), sm = sy;
+    const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
+    for (int64_t A = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg; A < n; A += stride) {
+        float4 yi = make_float4(zero, zero, zero, zero);
+        if (m.ok) yi = ld4(y + A * K + m.q * 4);
+        if constexpr (SWEEP) {
+            float4 s = make_float4(zero, zero, zero, zero);
+            for_slots<K, LONG>(m, rowptr[A], rowptr[A + 1], cw, y, [&](float w, const float4& x) {
+                s.x = fmaf(w, x.x, s.x);
+                s.y = fmaf(w, x.y, s.y);
+                s.z = fmaf(w, x.z, s.z);
+                s.w = fmaf(w, x.w, s.w);
+            });
+            join_row<K, LONG>(s);
+            if (m.writes()) {
+                const float d = D[A];
+                const float4 z = d > 0.f ? make_float4(s.x / d, s.y / d, s.z / d, s.w / d) : yi;
+                if (z_out) st4(z_out + A * K + m.q * 4, z);
+                yi.x = one_m * yi.x + omega * z.x;
+                yi.y = one_m * yi.y + omega * z.y;
+                yi.z = one_m * yi.z + omega * z.z;
+                yi.w = one_m * yi.w + omega * z.w;
+                st4(y1 + A * K + m.q * 4, yi);
+            }
+        }
+        if constexpr (MEAN) {
+            if (m.writes()) {
+                const float M = mass[A];
+                sy.x = fmaf(M, yi.x, sy.x);
+                sy.y = fmaf(M, yi.y, sy.y);
+                sy.z = fmaf(M, yi.z, sy.z);
+                sy.w = fmaf(M, yi.w, sy.w);
+                sm.x += M;
+            }
+        }
     }
-    keys[i] = (uint32_t)a;
-    vals[i] = (uint32_t)i;
-    atomicAdd(&cnt[a], 1);
+    if constexpr (MEAN) {
+        if (finish_cols<K, LONG>(m, sy, sm, part, counter, red) && threadIdx.x < K)
+            mu[threadIdx.x] = red[threadIdx.x] / red[K];  // chunk 0's first sum is the total mass
+    }
 }
 
-// y0[A] = mean of the member rows (members in ascending fine id), M_A = size
-template <int K>
-__global__ void k_aggregate_means(int64_t nc, const int64_t* __restrict__ start,
-                                  const int32_t* __restrict__ cnt, const uint32_t* __restrict__ members,
-                                  const float* __restrict__ X, float* __restrict__ y0,
-                                  float* __restrict__ mass) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nc * K) return;
-    int64_t A = idx / K;
-    int k = (int)(idx % K);
-    int64_t b = start[A];
-    int32_t c = cnt[A];
-    float s = 0.f;
-    for (int32_t t = 0; t < c; ++t) s += X[(int64_t)members[b + t] * K + k];
-    y0[idx] = c > 0 ? s / (float)c : 0.f;
-    if (k == 0) mass[A] = (float)c;
+// Loop control of the edge scaling, from this iteration's loss: convergence
+// test, step size from the loss ratio, lambda_1 after the last update.
+__device__ __forceinline__ void scale_control(const ScaleStep& st, float loss) {
+    ScaleState& S = *st.state;
+    if (S.stop) return;
+    const double L = (double)loss;
+    if (!st.lam_prev) {
+        S.L0 = L;
+        S.lam1 = 1.0;
+        S.eta = st.eta_max;
+    } else {
+        if ((S.L_prev - L) / L < st.eps) {
+            S.stop = 1;
+            return;
+        }
+        if (*st.lam_prev != ~0ull) S.lam1 = __longlong_as_double((long long)*st.lam_prev);
+        S.eta = (S.L_prev / S.L0) * st.eta_max;
+    }
+    S.inv_bound = 1.0 / (S.lam1 * st.bound_step);
+    *st.loss_hist = loss;
+    S.L_prev = L;
+    S.it += 1;
 }
 
-// D_c[A] = sum of the parameter weights on A's row (warp per row, fixed order)
-__global__ void k_param_degree(int64_t n, const int64_t* __restrict__ rowptr,
-                               const int32_t* __restrict__ eid, const float* __restrict__ w,
-                               float* __restrict__ D) {
-    const int lane = threadIdx.x & 31;
-    int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (p >= n) return;
-    float s = 0.f;
-    for (int64_t j = rowptr[p] + lane; j < rowptr[p + 1]; j += 32) s += w[eid[j]];
+// Quotients of the smoothed block: y^T L y from the squared differences over
+// every row's slots (each edge twice), sum M (y - mu)^2; in the last block
+// the loss and the adjoint's coefficients
+//   coef[0..K) = 2 g / Q, [K..2K) = 2 g N / Q^2, [2K..3K) = g / Q, [3K..4K) = mu,
+// g = d loss / d R_c.  LY: L y is stored.
+template <int K, bool LONG, bool LY>
+__global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __restrict__ rowptr,
+                                                  const int2* __restrict__ cw, const float* __restrict__ y,
+                                                  const float* __restrict__ mass, const double* __restrict__ mu,
+                                                  double* part, unsigned* counter, const float* __restrict__ Rf,
+                                                  const float* __restrict__ grad_loss, float* __restrict__ loss_out,
+                                                  float* __restrict__ ly_out, float* __restrict__ coef, ScaleStep st) {
+    __shared__ double red[LT];
+    const RowLanes<K, LONG> m;
+    constexpr int RPW = RowLanes<K, LONG>::RPW;
+    const float zero = 0.f;
+    float4 N = make_float4(zero, zero, zero, zero), Q = N, mk = N;
+    if (m.ok) {
+        const double* u = mu + m.q * 4;
+        mk = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
+    }
+    const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
+    for (int64_t A = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg; A < n; A += stride) {
+        float4 ya = make_float4(zero, zero, zero, zero), l = ya;
+        if (m.ok) ya = ld4(y + A * K + m.q * 4);
+        for_slots<K, LONG>(m, rowptr[A], rowptr[A + 1], cw, y, [&](float w, const float4& x) {
+            float d = ya.x - x.x, wd = w * d;
+            N.x = fmaf(wd, d, N.x);
+            l.x += wd;
+            d = ya.y - x.y, wd = w * d;
+            N.y = fmaf(wd, d, N.y);
+            l.y += wd;
+            d = ya.z - x.z, wd = w * d;
+            N.z = fmaf(wd, d, N.z);
+            l.z += wd;
+            d = ya.w - x.w, wd = w * d;
+            N.w = fmaf(wd, d, N.w);
+            l.w += wd;
+        });
+        if constexpr (LY) {
+            join_row<K, LONG>(l);
+            if (m.writes()) st4(ly_out + A * K + m.q * 4, l);
+        }
+        if (m.writes()) {
+            const float M = mass[A];
+            float t = ya.x - mk.x;
+            Q.x = fmaf(M * t, t, Q.x);
+            t = ya.y - mk.y;
+            Q.y = fmaf(M * t, t, Q.y);
+            t = ya.z - mk.z;
+            Q.z = fmaf(M * t, t, Q.z);
+            t = ya.w - mk.w;
+            Q.w = fmaf(M * t, t, Q.w);
+        }
+    }
+    if (!finish_cols<K, LONG>(m, N, Q, part, counter, red)) return;
+    const int k = threadIdx.x;
+    if (k >= 32) return;  // the first warp: a column per lane
+    double s = 0.0;
+    if (k < K) {
+        const double Ns = 0.5 * red[k], Qs = red[K + k], f = (double)Rf[k];
+        const double Rc = Ns / Qs, r = Rc / f - 1.0;
+        s = r * r;
+        if (coef) {
+            const double gq = (grad_loss ? (double)*grad_loss : 1.0) * (2.0 / K) * r / (f * Qs);
+            coef[k] = (float)(2.0 * gq);
+            coef[K + k] = (float)(2.0 * gq * Rc);
+            coef[2 * K + k] = (float)gq;
+            coef[3 * K + k] = (float)mu[k];
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) D[p] = s;
-}
-
-// forward sweep: z = D^-1 A y (or y when isolated), y1 = (1-w) y + w z
-template <int K>
-__global__ void k_param_sweep(int64_t n, const int64_t* __restrict__ rowptr,
-                              const int32_t* __restrict__ col, const int32_t* __restrict__ eid,
-                              const float* __restrict__ w, const float* __restrict__ D,
-                              const float* __restrict__ y, float omega, float* __restrict__ z_out,
-                              float* __restrict__ y1) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * K) return;
-    int64_t A = idx / K;
-    int k = (int)(idx % K);
-    float s = 0.f;
-    for (int64_t j = rowptr[A]; j < rowptr[A + 1]; ++j) s = fmaf(w[eid[j]], y[(int64_t)col[j] * K + k], s);
-    float z = D[A] > 0.f ? s / D[A] : y[idx];
-    if (z_out) z_out[idx] = z;
-    y1[idx] = (1.f - omega) * y[idx] + omega * z;
-}
-
-// adjoint sweep: yb_s = (1-w) yb + w A D^-1 yb   (isolated: yb_s = yb)
-template <int K>
-__global__ void k_param_sweep_adj(int64_t n, const int64_t* __restrict__ rowptr,
-                                  const int32_t* __restrict__ col, const int32_t* __restrict__ eid,
-                                  const float* __restrict__ w, const float* __restrict__ D,
-                                  const float* __restrict__ yb, float omega,
-                                  float* __restrict__ yb_out) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * K) return;
-    int64_t A = idx / K;
-    int k = (int)(idx % K);
-    if (!(D[A] > 0.f)) {
-        yb_out[idx] = yb[idx];
-        return;
+    if (k == 0) {
+        const float loss = (float)(s * (1.0 / K));
+        if (loss_out) *loss_out = loss;
+        if (st.state) scale_control(st, loss);
     }
-    float s = 0.f;
-    for (int64_t j = rowptr[A]; j < rowptr[A + 1]; ++j) {
-        int64_t B = col[j];
-        s = fmaf(w[eid[j]], yb[B * K + k] / D[B], s);
-    }
-    yb_out[idx] = (1.f - omega) * yb[idx] + omega * s;
 }
 
-// scalars: mu, Q, N, R_c, gRc from the FP64 sums
-__global__ void k_loss_scalars(int K, const double* __restrict__ Nsum, const double* __restrict__ Qsum,
-                               const float* __restrict__ Rf, const float* __restrict__ grad_loss,
-                               float* __restrict__ loss_out, float* __restrict__ gRc,
-                               float* __restrict__ Qf, float* __restrict__ Nf) {
-    if (threadIdx.x != 0) return;
-    double loss = 0.0;
-    const double g = grad_loss ? (double)*grad_loss : 1.0;
-    for (int k = 0; k < K; ++k) {
-        double Rc = Nsum[k] / Qsum[k];
-        double r = Rc / (double)Rf[k] - 1.0;
-        loss += r * r;
-        if (gRc) gRc[k] = (float)(g * 2.0 * r / (double)Rf[k] / (double)K);
-        if (Qf) Qf[k] = (float)Qsum[k];
-        if (Nf) Nf[k] = (float)Nsum[k];
-    }
-    if (loss_out) *loss_out = (float)(loss / (double)K);
-}
-
-__global__ void k_rf(int K, const double* __restrict__ num, const double* __restrict__ den,
-                     float* __restrict__ Rf) {
-    int k = threadIdx.x;
-    if (k < K) Rf[k] = (float)(num[k] / den[k]);
-}
-
-__global__ void k_mu(int K, const double* __restrict__ s, const double* __restrict__ msum,
-                     double* __restrict__ mu) {
-    int k = threadIdx.x;
-    if (k < K) mu[k] = s[k] / *msum;
-}
-
-// ybar_S = gRc (2 L y / Q - 2 N M (y - mu) / Q^2)
+// Adjoint of the quotients: yb = 2 g / Q (L y) - 2 g N / Q^2 M (y - mu), and
+// T = yb / D, which the reverse sweeps gather
 template <int K>
-__global__ void k_adj_final(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                            const int32_t* __restrict__ eid, const float* __restrict__ w,
-                            const float* __restrict__ y, const float* __restrict__ mass,
-                            const double* __restrict__ mu, const float* __restrict__ Q,
-                            const float* __restrict__ N, const float* __restrict__ gRc,
-                            float* __restrict__ yb) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * K) return;
-    int64_t A = idx / K;
-    int k = (int)(idx % K);
-    const float ya = y[idx];
-    float ly = 0.f;
-    for (int64_t j = rowptr[A]; j < rowptr[A + 1]; ++j) ly = fmaf(w[eid[j]], ya - y[(int64_t)col[j] * K + k], ly);
-    const float q = Q[k];
-    yb[idx] = gRc[k] * (2.f * ly / q - 2.f * N[k] * mass[A] * (ya - (float)mu[k]) / (q * q));
-}
-
-// per coarse edge: direct term + sum over sweeps of the weight adjoint
-template <int K>
-__global__ void k_edge_grad(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                            int S, int64_t nK, const float* __restrict__ Y, const float* __restrict__ Z,
-                            const float* __restrict__ YB, const float* __restrict__ D, float omega,
-                            const float* __restrict__ Q, const float* __restrict__ gRc,
-                            float* __restrict__ grad) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m) return;
-    const int64_t A = eu[e], B = ev[e];
-    const float* yS = Y + (int64_t)S * nK;
-    float g = 0.f;
+__global__ void __launch_bounds__(LT) k_adj_start(int64_t n, const float* __restrict__ ly, const float* __restrict__ y,
+                                                  const float* __restrict__ mass, const float* __restrict__ D,
+                                                  const float* __restrict__ coef, float* __restrict__ yb,
+                                                  float* __restrict__ T) {
+    const int64_t idx = (int64_t)blockIdx.x * LT + threadIdx.x;  // 16-byte chunk
+    if (idx >= n * (K / 4)) return;
+    const int64_t A = idx / (K / 4);
+    const int q = (int)(idx % (K / 4)) * 4;
+    const float4 l = ld4(ly + idx * 4), v = ld4(y + idx * 4);
+    const float M = mass[A], d = D[A];
+    const float li[4] = {l.x, l.y, l.z, l.w}, vi[4] = {v.x, v.y, v.z, v.w};
+    float o[4];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float t = yS[A * K + k] - yS[B * K + k];
-        g = fmaf(gRc[k] * t / Q[k], t, g);
-    }
-    const float iDA = 1.f / D[A], iDB = 1.f / D[B];
-    for (int s = 0; s < S; ++s) {
-        const float* y = Y + (int64_t)s * nK;
-        const float* z = Z + (int64_t)s * nK;
-        const float* yb = YB + (int64_t)(s + 1) * nK;
-        float ga = 0.f, gb = 0.f;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            ga = fmaf(yb[A * K + k], y[B * K + k] - z[A * K + k], ga);
-            gb = fmaf(yb[B * K + k], y[A * K + k] - z[B * K + k], gb);
+    for (int i = 0; i < 4; ++i)
+        o[i] = coef[q + i] * li[i] - coef[K + q + i] * M * (vi[i] - coef[3 * K + q + i]);
+    st4(yb + idx * 4, make_float4(o[0], o[1], o[2], o[3]));
+    st4(T + idx * 4, make_float4(o[0] / d, o[1] / d, o[2] / d, o[3] / d));
+}
+
+// reverse sweep: yb_s = (1-w) yb + w A T (isolated: yb_s = yb), T_s = yb_s / D
+template <int K, bool LONG>
+__global__ void __launch_bounds__(LT) k_param_sweep_adj(int64_t n, const int64_t* __restrict__ rowptr,
+                                                        const int2* __restrict__ cw, const float* __restrict__ D,
+                                                        const float* __restrict__ yb, const float* __restrict__ T,
+                                                        float omega, float* __restrict__ yb_out,
+                                                        float* __restrict__ T_out) {
+    const RowLanes<K, LONG> m;
+    constexpr int RPW = RowLanes<K, LONG>::RPW;
+    const float zero = 0.f, one_m = 1.f - omega;
+    const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
+    for (int64_t A = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg; A < n; A += stride) {
+        float4 s = make_float4(zero, zero, zero, zero);
+        for_slots<K, LONG>(m, rowptr[A], rowptr[A + 1], cw, T, [&](float w, const float4& x) {
+            s.x = fmaf(w, x.x, s.x);
+            s.y = fmaf(w, x.y, s.y);
+            s.z = fmaf(w, x.z, s.z);
+            s.w = fmaf(w, x.w, s.w);
+        });
+        join_row<K, LONG>(s);
+        if (!m.writes()) continue;
+        const float d = D[A];
+        float4 b = ld4(yb + A * K + m.q * 4);
+        if (d > 0.f) {
+            b.x = one_m * b.x + omega * s.x;
+            b.y = one_m * b.y + omega * s.y;
+            b.z = one_m * b.z + omega * s.z;
+            b.w = one_m * b.w + omega * s.w;
         }
-        g += omega * (ga * iDA + gb * iDB);
+        st4(yb_out + A * K + m.q * 4, b);
+        st4(T_out + A * K + m.q * 4, make_float4(b.x / d, b.y / d, b.z / d, b.w / d));
     }
-    grad[e] = g;
+}
+
+// Alg. 1's update of edge e = (A, B) with gradient g: momentum, the lambda_1
+// guard, never below zero
+__device__ __forceinline__ void update_edge(int64_t e, int32_t A, int32_t B, float g, const ScaleStep& st) {
+    const double inv = st.state->inv_bound, eta = st.state->eta;
+    double d = st.alpha * (double)st.dw[e] - eta * (double)g;
+    d = d > 0.0 ? d : 0.0;
+    // min(dG / (dP + d)) <= bound at either end <=> d >= min(dG / bound - dP)
+    const double cp = st.dG[A] * inv - st.dP[A], cq = st.dG[B] * inv - st.dP[B];
+    const double cap = cp < cq ? cp : cq;
+    if (d >= cap) d = cap > 0.0 ? cap : 0.0;
+    st.dw[e] = (float)d;
+    st.w[e] = (float)((double)st.w[e] + d);
+}
+
+// Per reduced edge (A, B): the direct term g / Q (y_A - y_B)^2 plus, over the
+// sweeps, w [T_A (y_B - z_A) + T_B (y_A - z_B)]; G lanes per edge, a 16-byte
+// chunk of the columns each.  SCALE: the edge's scaling update in place of
+// its gradient; the sweeps read the slot-order copy of the weights, so w may
+// change here.
+template <int K, bool SCALE>
+__global__ void __launch_bounds__(LT) k_edge_grad(int64_t m, const int32_t* __restrict__ eu,
+                                                  const int32_t* __restrict__ ev, int S, int64_t nK,
+                                                  const float* __restrict__ Y, const float* __restrict__ Z,
+                                                  const float* __restrict__ T, float omega,
+                                                  const float* __restrict__ coef, float* __restrict__ grad,
+                                                  ScaleStep st) {
+    constexpr int G = K / 4, EPW = 32 / G;  // edges per warp
+    const int lane = threadIdx.x & 31, seg = lane / G, q = lane % G;
+    const int64_t e = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * EPW + seg;
+    const bool ok = seg < EPW && e < m;
+    float g = 0.f, gs = 0.f;
+    if (ok) {
+        const int32_t A = eu[e], B = ev[e];
+        const int64_t a = (int64_t)A * K + q * 4, b = (int64_t)B * K + q * 4;
+        const float4 c = ld4(coef + 2 * K + q * 4);
+        const float4 ya = ld4(Y + (int64_t)S * nK + a), yb = ld4(Y + (int64_t)S * nK + b);
+        float t = ya.x - yb.x;
+        g = c.x * t * t;
+        t = ya.y - yb.y;
+        g = fmaf(c.y * t, t, g);
+        t = ya.z - yb.z;
+        g = fmaf(c.z * t, t, g);
+        t = ya.w - yb.w;
+        g = fmaf(c.w * t, t, g);
+#pragma unroll 2
+        for (int s = 0; s < S; ++s) {
+            const int64_t o = (int64_t)s * nK;
+            const float4 ta = ld4(T + o + a), tb = ld4(T + o + b);  // T_{s+1}
+            const float4 y0 = ld4(Y + o + a), y1 = ld4(Y + o + b);
+            const float4 z0 = ld4(Z + o + a), z1 = ld4(Z + o + b);
+            gs = fmaf(ta.x, y1.x - z0.x, gs);
+            gs = fmaf(ta.y, y1.y - z0.y, gs);
+            gs = fmaf(ta.z, y1.z - z0.z, gs);
+            gs = fmaf(ta.w, y1.w - z0.w, gs);
+            gs = fmaf(tb.x, y0.x - z1.x, gs);
+            gs = fmaf(tb.y, y0.y - z1.y, gs);
+            gs = fmaf(tb.z, y0.z - z1.z, gs);
+            gs = fmaf(tb.w, y0.w - z1.w, gs);
+        }
+    }
+    g = fmaf(omega, gs, g);
+    float tot = g;
+#pragma unroll
+    for (int i = 1; i < G; ++i) tot += __shfl_down_sync(0xffffffffu, g, i);
+    if constexpr (!SCALE) {
+        if (ok && q == 0) grad[e] = tot;
+    } else {
+        // the update is FP64 work (four divisions an edge): the block's edges
+        // are handed to full warps, one lane in G would pay the pipe for all
+        constexpr int EPB = EPW * LW;
+        __shared__ float s_g[EPB];
+        if (seg < EPW && q == 0) s_g[(threadIdx.x >> 5) * EPW + seg] = tot;
+        __syncthreads();
+        const int64_t f = (int64_t)blockIdx.x * EPB + threadIdx.x;
+        if (threadIdx.x >= EPB || f >= m || st.state->stop) return;
+        update_edge(f, eu[f], ev[f], s_g[threadIdx.x], st);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-static int red_grid(const gr_ctx* c) { return c->num_sms > 0 ? 2 * c->num_sms : 64; }
+// A warp per row from a mean of 32 slots on; below, G lanes hold a row's
+// slots in flight by themselves and the other rows of the warp hide them
+// (a warp per row on 7,680 rows of 13 slots, K = 16: 9 us a sweep against 6).
+bool long_rows(const gr_ctx* c, int64_t slots) { return slots >= 32 * c->n; }
 
-template <int K>
-static cudaError_t coarse_rc_parts(gr_ctx* cc, const float* y, const float* w_c, const float* mass,
-                                   const double* msum, double* part, double* Nsum, double* musum,
-                                   double* mu, double* Qsum) {
-    cudaStream_t s = cc->stream;
-    const int rg = red_grid(cc);
-    // N: sum over reduced edges with the parameter weights
-    k_edge_quad<K><<<rg, LS_THREADS, 0, s>>>(cc->m, cc->eu, cc->ev, nullptr, w_c, y, part); count_launch();
-    k_finish_sums<<<1, 64, 0, s>>>(part, rg, K, Nsum); count_launch();
-    k_row_sum<K><<<rg, LS_THREADS, 0, s>>>(cc->n, y, mass, part); count_launch();
-    k_finish_sums<<<1, 64, 0, s>>>(part, rg, K, musum); count_launch();
-    k_mu<<<1, 64, 0, s>>>(K, musum, msum, mu); count_launch();
-    k_row_quad<K><<<rg, LS_THREADS, 0, s>>>(cc->n, y, mass, mu, part); count_launch();
-    k_finish_sums<<<1, 64, 0, s>>>(part, rg, K, Qsum); count_launch();
-    return cudaGetLastError();
+// blocks of a row pass: one wave, and what the statistics tickets can count
+template <int K, bool LONG>
+unsigned row_grid(const gr_ctx* c, int64_t n) {
+    const int64_t want = ceil_div(n > 0 ? n : 1, (int64_t)RowLanes<K, LONG>::RPW * LW);
+    int64_t cap = (int64_t)c->num_sms * ROW_BLOCKS;
+    if (cap > STATS_GROUP * STATS_MAX_GROUPS) cap = STATS_GROUP * STATS_MAX_GROUPS;
+    return (unsigned)(want < cap ? want : cap);
+}
+constexpr size_t PART_ROWS = (size_t)STATS_GROUP * STATS_MAX_GROUPS;
+
+template <int K, bool LONG>
+gr_status fine_quotients(gr_ctx* f, const float* X, double* part, unsigned* counter, float* Rf) {
+    k_fine_quotients<K, LONG><<<row_grid<K, LONG>(f, f->n), LT, 0, f->stream>>>(f->n, f->eptr, f->ev, f->ew, X, part,
+                                                                               counter, Rf);
+    count_launch();
+    GR_TRY_CUDA(f, cudaGetLastError(), "fine quotients");
+    return GR_OK;
 }
 
+bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
 template <int K>
-static gr_status loss_fwd_k(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X,
-                            const float* w_c, int S, double omega, float* loss, float* saved) {
+gr_status fine_k(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, float* y0, float* Rf, float* mass,
+                 bool* bad) {
     cudaStream_t s = f->stream;
     const int64_t n = f->n, nc = cc->n;
-    const int rg = red_grid(f);
-    float* y0 = saved;
-    float* Rf = saved + nc * K;
-    float* mass = Rf + K;
-    // scratch on the coarse context
-    void *pa, *pb, *pc;
-    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_A, sizeof(double) * (size_t)(rg * K + 8 * K) + 256, &pa), "ws");
-    double* part = (double*)pa;
-    double* Nsum = part + rg * K;
-    double* den = Nsum + K;
-    double* musum = den + K;
-    double* mu = musum + K;
-    double* Qsum = mu + K;
-    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_B, sizeof(float) * (size_t)nc * K * 2 + sizeof(float) * nc + 256, &pb), "ws");
-    float* ya = (float*)pb;
-    float* yb = ya + nc * K;
-    float* D = yb + nc * K;
-    // fine Rayleigh quotients
-    k_edge_quad<K><<<rg, LS_THREADS, 0, s>>>(f->m, f->eu, f->ev, f->ew, nullptr, X, part); count_launch();
-    k_finish_sums<<<1, 64, 0, s>>>(part, rg, K, Nsum); count_launch();
-    k_row_quad<K><<<rg, LS_THREADS, 0, s>>>(n, X, nullptr, nullptr, part); count_launch();
-    k_finish_sums<<<1, 64, 0, s>>>(part, rg, K, den); count_launch();
-    k_rf<<<1, 64, 0, s>>>(K, Nsum, den, Rf); count_launch();
-    // aggregate means: stable sort of fine ids by label
-    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_C, sizeof(uint32_t) * (size_t)n * 4 + sizeof(int64_t) * (nc + 1) * 2 +
-                                              sizeof(int32_t) * (nc + 2) + 1024, &pc), "ws");
-    uint32_t* k0 = (uint32_t*)pc;
-    uint32_t* v0 = k0 + n;
-    uint32_t* k1 = v0 + n;
-    uint32_t* v1 = k1 + n;
-    int64_t* cnt64 = (int64_t*)(v1 + n + (n & 1));
-    int64_t* start = cnt64 + (nc + 1);
-    int32_t* cnt = (int32_t*)(start + (nc + 1));
-    int32_t* bad = cnt + nc;
-    GR_TRY_CUDA(cc, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)(nc + 1), s), "memset");
-    k_agg_keys<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(n, agg, nc, k0, v0, cnt, bad); count_launch();
-    int alt = 0;
-    GR_TRY_CUDA(cc, radix_sort_u32(k0, v0, k1, v1, n, bits_for((uint64_t)(nc - 1)), cc->ws, s, &alt), "sort");
-    const uint32_t* members = alt ? v1 : v0;
-    k_i32_to_i64_n<<<(unsigned)ceil_div(nc + 1, 256), 256, 0, s>>>(cnt, nc, cnt64); count_launch();
-    GR_TRY_CUDA(cc, scan_exclusive_i64(cnt64, start, nc + 1, cc->ws, s), "scan");
-    k_aggregate_means<K><<<(unsigned)ceil_div(nc * K, 256), 256, 0, s>>>(nc, start, cnt, members, X, y0, mass); count_launch();
-    // sweeps on the reduced graph with the parameter weights
-    k_param_degree<<<(unsigned)ceil_div(nc * 32, 256), 256, 0, s>>>(nc, cc->rowptr, cc->eid, w_c, D); count_launch();
+    // rows are moved in 16-byte chunks: a block or result that does not start
+    // on such a boundary goes through an aligned copy
+    const bool cx = !aligned16(X), cy = !aligned16(y0);
+    const size_t b_part = sizeof(double) * 2 * K * PART_ROWS, b_y = cy ? sizeof(float) * (size_t)nc * K : 0;
+    void* p;
+    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_A, b_part + STATS_COUNTER_BYTES + 256 + b_y +
+                                              (cx ? sizeof(float) * (size_t)n * K : 0), &p), "ws");
+    double* part = (double*)p;
+    unsigned* counter = (unsigned*)((char*)p + b_part);
+    float* ytmp = (float*)((char*)p + ((b_part + STATS_COUNTER_BYTES + 255) & ~size_t(255)));
+    float* yout = cy ? ytmp : y0;
+    if (cx) {
+        float* t = (float*)((char*)ytmp + b_y);
+        GR_TRY_CUDA(cc, cudaMemcpyAsync(t, X, sizeof(float) * (size_t)n * K, cudaMemcpyDeviceToDevice, s), "copy");
+        X = t;
+    }
+    GR_TRY_CUDA(cc, cudaMemsetAsync(counter, 0, STATS_COUNTER_BYTES, s), "memset");
+    MapChain ch;
+    ch.map[0] = agg;
+    ch.count = 1;
+    GroupJob job;
+    gr_status st = group_begin(cc, WS_LOSS_C, ch, n, nc, &job);
+    if (st != GR_OK) return st;
+    // upper edges per row: half the slots
+    st = long_rows(f, f->m) ? fine_quotients<K, true>(f, X, part, counter, Rf)
+                            : fine_quotients<K, false>(f, X, part, counter, Rf);
+    if (st != GR_OK) return st;
+    st = group_finish(cc, &job, bad);
+    if (st != GR_OK || *bad) return st;
+    k_aggregate_means<K><<<(unsigned)ceil_div(nc * 32, LT), LT, 0, s>>>(nc, job.start, job.members, X, yout, mass);
+    count_launch();
+    if (cy) GR_TRY_CUDA(cc, cudaMemcpyAsync(y0, yout, b_y, cudaMemcpyDeviceToDevice, s), "copy");
+    GR_TRY_CUDA(cc, cudaGetLastError(), "aggregate means");
+    return GR_OK;
+}
+
+template <int K, bool LONG>
+gr_status coarse_k(gr_ctx* cc, int S, double omega, const float* y0, const float* Rf, const float* mass,
+                   const LossWork& W, bool adjoint, const float* grad_loss, float* loss_out, const ScaleStep& st) {
+    cudaStream_t s = cc->stream;
+    const int64_t nc = cc->n, nK = nc * K;
+    const unsigned grid = row_grid<K, LONG>(cc, nc);
+    const float om = (float)omega;
     const float* y = y0;
+    if (S == 0) {
+        k_param_sweep<K, LONG, false, true><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, W.D, y, om, nullptr, nullptr,
+                                                                 mass, W.part, W.counter, W.mu);
+        count_launch();
+    }
     for (int it = 0; it < S; ++it) {
-        float* out = (it & 1) ? yb : ya;
-        k_param_sweep<K><<<(unsigned)ceil_div(nc * K, 256), 256, 0, s>>>(nc, cc->rowptr, cc->col, cc->eid, w_c,
-                                                                         D, y, (float)omega, nullptr, out); count_launch();
+        // without the adjoint two buffers take turns
+        float* out = adjoint ? W.Y + (size_t)(it + 1) * nK : W.Y + (size_t)(it & 1) * nK;
+        float* z = adjoint ? W.Z + (size_t)it * nK : nullptr;
+        if (it + 1 < S)
+            k_param_sweep<K, LONG, true, false><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, W.D, y, om, z, out, nullptr,
+                                                                     nullptr, nullptr, nullptr);
+        else
+            k_param_sweep<K, LONG, true, true><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, W.D, y, om, z, out, mass,
+                                                                    W.part, W.counter, W.mu);
+        count_launch();
         y = out;
     }
-    k_sum_f32<<<1, 256, 0, s>>>(mass, nc, den); count_launch();
-    GR_TRY_CUDA(cc, coarse_rc_parts<K>(cc, y, w_c, mass, den, part, Nsum, musum, mu, Qsum), "rc");
-    k_loss_scalars<<<1, 32, 0, s>>>(K, Nsum, Qsum, Rf, nullptr, loss, nullptr, nullptr, nullptr); count_launch();
-    GR_TRY_CUDA(cc, cudaGetLastError(), "loss fwd");
-    // label check
-    int32_t hbad = 0;
-    GR_TRY_CUDA(cc, cudaMemcpyAsync(&hbad, bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy");
-    GR_TRY_CUDA(cc, cudaStreamSynchronize(s), "sync");
-    if (hbad) return set_error(f, GR_EINVAL, "loss_fwd: agg labels must lie in [0, coarse n)");
+    if (adjoint)
+        k_quotients<K, LONG, true><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, y, mass, W.mu, W.part, W.counter, Rf,
+                                                        grad_loss, loss_out, W.yb1, W.coef, st);
+    else
+        k_quotients<K, LONG, false><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, y, mass, W.mu, W.part, W.counter, Rf,
+                                                         nullptr, loss_out, nullptr, nullptr, st);
+    count_launch();
+    GR_TRY_CUDA(cc, cudaGetLastError(), "loss");
+    return GR_OK;
+}
+
+template <int K, bool LONG>
+gr_status adjoint_k(gr_ctx* cc, int S, double omega, const float* mass, const LossWork& W, float* grad,
+                    const ScaleStep& st) {
+    cudaStream_t s = cc->stream;
+    const int64_t nc = cc->n, nK = nc * K;
+    const unsigned grid = row_grid<K, LONG>(cc, nc);
+    const float om = (float)omega;
+    if (S > 0) {
+        float *yb = W.yb0, *yn = W.yb1;  // yb1 held L y
+        k_adj_start<K><<<(unsigned)ceil_div(nc * (K / 4), LT), LT, 0, s>>>(nc, W.yb1, W.Y + (size_t)S * nK, mass, W.D,
+                                                                          W.coef, yb, W.T + (size_t)(S - 1) * nK);
+        count_launch();
+        // T_S .. T_1; the adjoint of y_0 itself enters no gradient
+        for (int it = S - 1; it >= 1; --it) {
+            k_param_sweep_adj<K, LONG><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, W.D, yb, W.T + (size_t)it * nK, om, yn,
+                                                            W.T + (size_t)(it - 1) * nK);
+            count_launch();
+            float* t = yb;
+            yb = yn;
+            yn = t;
+        }
+    }
+    if (cc->m > 0) {
+        constexpr int EPB = (32 / (K / 4)) * LW;
+        const unsigned ge = (unsigned)ceil_div(cc->m, EPB);
+        if (st.state)
+            k_edge_grad<K, true><<<ge, LT, 0, s>>>(cc->m, cc->eu, cc->ev, S, nK, W.Y, W.Z, W.T, om, W.coef, nullptr, st);
+        else
+            k_edge_grad<K, false><<<ge, LT, 0, s>>>(cc->m, cc->eu, cc->ev, S, nK, W.Y, W.Z, W.T, om, W.coef, grad, st);
+        count_launch();
+    }
+    GR_TRY_CUDA(cc, cudaGetLastError(), "loss adjoint");
     return GR_OK;
 }
 
 template <int K>
-static gr_status loss_bwd_k(gr_ctx* cc, const float* saved, const float* w_c, int S, double omega,
-                            const float* grad_loss, float* grad) {
+gr_status coarse_pick(gr_ctx* cc, int S, double omega, const float* y0, const float* Rf, const float* mass,
+                      const LossWork& W, bool adjoint, const float* grad_loss, float* loss_out, const ScaleStep& st) {
+    return long_rows(cc, 2 * cc->m) ? coarse_k<K, true>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st)
+                                       : coarse_k<K, false>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+}
+
+template <int K>
+gr_status adjoint_pick(gr_ctx* cc, int S, double omega, const float* mass, const LossWork& W, float* grad,
+                       const ScaleStep& st) {
+    return long_rows(cc, 2 * cc->m) ? adjoint_k<K, true>(cc, S, omega, mass, W, grad, st)
+                                       : adjoint_k<K, false>(cc, S, omega, mass, W, grad, st);
+}
+
+}  // namespace
+
+gr_status loss_fine(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, int K, float* y0, float* Rf,
+                    float* mass, bool* bad) {
+    switch (K) {
+        case 4: return fine_k<4>(f, cc, agg, X, y0, Rf, mass, bad);
+        case 8: return fine_k<8>(f, cc, agg, X, y0, Rf, mass, bad);
+        case 16: return fine_k<16>(f, cc, agg, X, y0, Rf, mass, bad);
+        case 24: return fine_k<24>(f, cc, agg, X, y0, Rf, mass, bad);
+        case 32: return fine_k<32>(f, cc, agg, X, y0, Rf, mass, bad);
+    }
+    return set_error(f, GR_EINVAL, "loss: K must be 4, 8, 16, 24 or 32");
+}
+
+gr_status loss_work(gr_ctx* cc, int K, int S, bool adjoint, LossWork* W) {
+    const size_t nc = (size_t)cc->n, nK = nc * (size_t)K;
+    size_t need = 0;
+    auto add = [&](size_t bytes) {
+        size_t off = need;
+        need += (bytes + 255) & ~size_t(255);
+        return off;
+    };
+    const size_t o_cw = add(sizeof(int2) * (size_t)(cc->m > 0 ? 2 * cc->m : 1)), o_D = add(4 * nc),
+                 o_part = add(sizeof(double) * 2 * (size_t)K * PART_ROWS), o_ctr = add(STATS_COUNTER_BYTES),
+                 o_coef = add(sizeof(float) * 4 * (size_t)K), o_mu = add(sizeof(double) * (size_t)K),
+                 o_Y = add(4 * nK * (adjoint ? (size_t)S + 1 : 2)), o_Z = add(adjoint ? 4 * nK * (size_t)S : 0),
+                 o_T = add(adjoint ? 4 * nK * (size_t)S : 0), o_b0 = add(adjoint ? 4 * nK : 0),
+                 o_b1 = add(adjoint ? 4 * nK : 0);
+    void* base;
+    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_B, need, &base), "ws");
+    char* B = (char*)base;
+    W->cw = (int2*)(B + o_cw);
+    W->D = (float*)(B + o_D);
+    W->part = (double*)(B + o_part);
+    W->counter = (unsigned*)(B + o_ctr);
+    W->coef = (float*)(B + o_coef);
+    W->mu = (double*)(B + o_mu);
+    W->Y = (float*)(B + o_Y);
+    W->Z = (float*)(B + o_Z);
+    W->T = (float*)(B + o_T);
+    W->yb0 = (float*)(B + o_b0);
+    W->yb1 = (float*)(B + o_b1);
+    GR_TRY_CUDA(cc, cudaMemsetAsync(W->counter, 0, STATS_COUNTER_BYTES, cc->stream), "memset");
+    return GR_OK;
+}
+
+gr_status loss_weights(gr_ctx* cc, const float* w, const LossWork& W, double* dP, const double* dG,
+                       unsigned long long* lam) {
     cudaStream_t s = cc->stream;
     const int64_t nc = cc->n;
-    const int64_t nK = nc * K;
-    const float* y0 = saved;
-    const float* Rf = saved + nK;
-    const float* mass = Rf + K;
-    const int rg = red_grid(cc);
-    void *pa, *pb;
-    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_A, sizeof(double) * (size_t)(rg * K + 8 * K) + 256, &pa), "ws");
-    double* part = (double*)pa;
-    double* Nsum = part + rg * K;
-    double* den = Nsum + K;
-    double* musum = den + K;
-    double* mu = musum + K;
-    double* Qsum = mu + K;
-    // Y[0..S], Z[0..S-1], YB[0..S], D, gRc, Q, N
-    size_t floats = (size_t)nK * (3 * S + 2) + nc + 4 * K + 64;
-    GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_B, sizeof(float) * floats, &pb), "ws");
-    float* Y = (float*)pb;
-    float* Z = Y + (size_t)(S + 1) * nK;
-    float* YB = Z + (size_t)(S > 0 ? S : 0) * nK;
-    float* D = YB + (size_t)(S + 1) * nK;
-    float* gRc = D + nc;
-    float* Qf = gRc + K;
-    float* Nf = Qf + K;
-    GR_TRY_CUDA(cc, cudaMemcpyAsync(Y, y0, sizeof(float) * nK, cudaMemcpyDeviceToDevice, s), "copy");
-    k_param_degree<<<(unsigned)ceil_div(nc * 32, 256), 256, 0, s>>>(nc, cc->rowptr, cc->eid, w_c, D); count_launch();
-    for (int it = 0; it < S; ++it) {
-        k_param_sweep<K><<<(unsigned)ceil_div(nK, 256), 256, 0, s>>>(nc, cc->rowptr, cc->col, cc->eid, w_c, D,
-                                                                     Y + it * nK, (float)omega, Z + it * nK,
-                                                                     Y + (it + 1) * nK);
+    auto run = [&](auto kern, int lanes) {
+        kern<<<(unsigned)ceil_div(nc * lanes, LT), LT, 0, s>>>(nc, cc->rowptr, cc->col, cc->eid, w, W.cw, W.D, dP, dG,
+                                                                lam);
         count_launch();
-    }
-    k_sum_f32<<<1, 256, 0, s>>>(mass, nc, den); count_launch();  // total mass, FP64
-    const float* yS = Y + (size_t)S * nK;
-    GR_TRY_CUDA(cc, coarse_rc_parts<K>(cc, yS, w_c, mass, den, part, Nsum, musum, mu, Qsum), "rc");
-    k_loss_scalars<<<1, 32, 0, s>>>(K, Nsum, Qsum, Rf, grad_loss, nullptr, gRc, Qf, Nf); count_launch();
-    k_adj_final<K><<<(unsigned)ceil_div(nK, 256), 256, 0, s>>>(nc, cc->rowptr, cc->col, cc->eid, w_c, yS, mass,
-                                                               mu, Qf, Nf, gRc, YB + (size_t)S * nK); count_launch();
-    for (int it = S - 1; it >= 0; --it) {
-        k_param_sweep_adj<K><<<(unsigned)ceil_div(nK, 256), 256, 0, s>>>(
-            nc, cc->rowptr, cc->col, cc->eid, w_c, D, YB + (size_t)(it + 1) * nK, (float)omega, YB + (size_t)it * nK);
-        count_launch();
-    }
-    if (cc->m > 0) {
-        k_edge_grad<K><<<(unsigned)ceil_div(cc->m, 256), 256, 0, s>>>(cc->m, cc->eu, cc->ev, S, nK, Y, Z, YB, D,
-                                                                      (float)omega, Qf, gRc, grad);
-        count_launch();
-    }
-    GR_TRY_CUDA(cc, cudaGetLastError(), "loss bwd");
+    };
+    const bool lng = long_rows(cc, 2 * cc->m);
+    if (dP) lng ? run(k_param_slots<32, true>, 32) : run(k_param_slots<8, true>, 8);
+    else lng ? run(k_param_slots<32, false>, 32) : run(k_param_slots<8, false>, 8);
+    GR_TRY_CUDA(cc, cudaGetLastError(), "parameter weights");
     return GR_OK;
+}
+
+gr_status loss_coarse(gr_ctx* cc, int K, int S, double omega, const float* y0, const float* Rf, const float* mass,
+                      const LossWork& W, bool adjoint, const float* grad_loss, float* loss_out, const ScaleStep& st) {
+    switch (K) {
+        case 4: return coarse_pick<4>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+        case 8: return coarse_pick<8>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+        case 16: return coarse_pick<16>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+        case 24: return coarse_pick<24>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+        case 32: return coarse_pick<32>(cc, S, omega, y0, Rf, mass, W, adjoint, grad_loss, loss_out, st);
+    }
+    return set_error(cc, GR_EINVAL, "loss: K must be 4, 8, 16, 24 or 32");
+}
+
+gr_status loss_adjoint(gr_ctx* cc, int K, int S, double omega, const float* mass, const LossWork& W, float* grad,
+                       const ScaleStep& st) {
+    switch (K) {
+        case 4: return adjoint_pick<4>(cc, S, omega, mass, W, grad, st);
+        case 8: return adjoint_pick<8>(cc, S, omega, mass, W, grad, st);
+        case 16: return adjoint_pick<16>(cc, S, omega, mass, W, grad, st);
+        case 24: return adjoint_pick<24>(cc, S, omega, mass, W, grad, st);
+        case 32: return adjoint_pick<32>(cc, S, omega, mass, W, grad, st);
+    }
+    return set_error(cc, GR_EINVAL, "loss: K must be 4, 8, 16, 24 or 32");
 }
 
 gr_status loss_fwd_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, const float* X, int K,
                         const float* w_c, int sweeps, double omega, float* loss, float* saved) {
-    switch (K) {
-        case 4: return loss_fwd_k<4>(fine, coarse, agg, X, w_c, sweeps, omega, loss, saved);
-        case 8: return loss_fwd_k<8>(fine, coarse, agg, X, w_c, sweeps, omega, loss, saved);
-        case 16: return loss_fwd_k<16>(fine, coarse, agg, X, w_c, sweeps, omega, loss, saved);
-        case 24: return loss_fwd_k<24>(fine, coarse, agg, X, w_c, sweeps, omega, loss, saved);
-        case 32: return loss_fwd_k<32>(fine, coarse, agg, X, w_c, sweeps, omega, loss, saved);
+    const int64_t nK = coarse->n * K;
+    float *y0 = saved, *Rf = saved + nK, *mass = Rf + K;
+    bool bad = false;
+    gr_status st = loss_fine(fine, coarse, agg, X, K, y0, Rf, mass, &bad);
+    if (st != GR_OK) return st;
+    if (bad) return set_error(fine, GR_EINVAL, "loss_fwd: agg labels must lie in [0, coarse n)");
+    LossWork W;
+    st = loss_work(coarse, K, sweeps, false, &W);
+    if (st != GR_OK) return st;
+    const float* y = y0;
+    if (!aligned16(y0)) {  // the sweeps read 16-byte chunks
+        GR_TRY_CUDA(coarse, cudaMemcpyAsync(W.Y + nK, y0, sizeof(float) * nK, cudaMemcpyDeviceToDevice, coarse->stream),
+                    "copy");
+        y = W.Y + nK;
     }
-    return set_error(fine, GR_EINVAL, "loss_fwd: K must be 4, 8, 16, 24 or 32");
+    st = loss_weights(coarse, w_c, W, nullptr, nullptr, nullptr);
+    if (st != GR_OK) return st;
+    return loss_coarse(coarse, K, sweeps, omega, y, Rf, mass, W, false, nullptr, loss, ScaleStep());
 }
 
 gr_status loss_bwd_impl(gr_ctx* coarse, const float* saved, int K, const float* w_c, int sweeps,
                         double omega, const float* grad_loss, float* grad_w) {
-    switch (K) {
-        case 4: return loss_bwd_k<4>(coarse, saved, w_c, sweeps, omega, grad_loss, grad_w);
-        case 8: return loss_bwd_k<8>(coarse, saved, w_c, sweeps, omega, grad_loss, grad_w);
-        case 16: return loss_bwd_k<16>(coarse, saved, w_c, sweeps, omega, grad_loss, grad_w);
-        case 24: return loss_bwd_k<24>(coarse, saved, w_c, sweeps, omega, grad_loss, grad_w);
-        case 32: return loss_bwd_k<32>(coarse, saved, w_c, sweeps, omega, grad_loss, grad_w);
-    }
-    return set_error(coarse, GR_EINVAL, "loss_bwd: K must be 4, 8, 16, 24 or 32");
+    const int64_t nK = coarse->n * K;
+    const float *Rf = saved + nK, *mass = Rf + K;
+    LossWork W;
+    gr_status st = loss_work(coarse, K, sweeps, true, &W);
+    if (st != GR_OK) return st;
+    GR_TRY_CUDA(coarse, cudaMemcpyAsync(W.Y, saved, sizeof(float) * nK, cudaMemcpyDeviceToDevice, coarse->stream),
+                "copy");
+    st = loss_weights(coarse, w_c, W, nullptr, nullptr, nullptr);
+    if (st != GR_OK) return st;
+    st = loss_coarse(coarse, K, sweeps, omega, W.Y, Rf, mass, W, true, grad_loss, nullptr, ScaleStep());
+    if (st != GR_OK) return st;
+    return loss_adjoint(coarse, K, sweeps, omega, mass, W, grad_w, ScaleStep());
 }
 
 }  // namespace gr

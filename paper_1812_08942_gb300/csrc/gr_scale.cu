@@ -9,62 +9,14 @@
 // Every edge of an iteration updates from the degrees at the iteration's start
 // (the paper gives no edge order, and this order parallelises); updates never
 // go below zero, as the scheme only scales weights up.
-#include "gr_internal.cuh"
+#include <math.h>
+#include <string.h>
+
+#include <vector>
+
+#include "gr_loss.cuh"
 
 namespace gr {
-
-namespace {
-
-constexpr int ST = 256;
-
-// for every edge: momentum step, the lambda_1 guard, the update
-__global__ void k_sgd_edges(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                            const float* __restrict__ grad, const double* __restrict__ dG,
-                            const double* __restrict__ dP, double bound, double alpha, double eta,
-                            float* __restrict__ dw, float* __restrict__ w) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m) return;
-    const int32_t p = eu[e], q = ev[e];
-    double d = alpha * (double)dw[e] - eta * (double)grad[e];
-    d = d > 0.0 ? d : 0.0;
-    const double phi_p = dG[p] / (dP[p] + d), phi_q = dG[q] / (dP[q] + d);
-    if ((phi_p < phi_q ? phi_p : phi_q) <= bound) {
-        const double cp = dG[p] / bound - dP[p], cq = dG[q] / bound - dP[q];
-        const double cap = cp < cq ? cp : cq;
-        d = cap > 0.0 ? cap : 0.0;
-    }
-    dw[e] = (float)d;
-    w[e] = (float)((double)w[e] + d);
-}
-
-// d_P(p) = sum of the row's current weights in slot order (= ascending edge id)
-__global__ void k_row_weight_sums(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ eid,
-                                  const float* __restrict__ w, double* __restrict__ d) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    double s = 0.0;
-    for (int64_t j = rowptr[p]; j < rowptr[p + 1]; ++j) s += (double)w[eid[j]];
-    d[p] = s;
-}
-
-// lambda_1 estimate: min over nodes with d_P > 0 of d_G / d_P (positive
-// doubles order like their bit patterns, so an integer minimum is exact)
-__global__ void k_min_ratio(int64_t n, const double* __restrict__ dG, const double* __restrict__ dP,
-                            unsigned long long* __restrict__ out) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long v = ~0ull;
-    if (p < n && dP[p] > 0.0) v = (unsigned long long)__double_as_longlong(dG[p] / dP[p]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long x = __shfl_xor_sync(0xffffffffu, v, o);
-        v = x < v ? x : v;
-    }
-    if ((threadIdx.x & 31) == 0 && v != ~0ull) atomicMin(out, v);
-}
-
-__global__ void k_set_f32(float* __restrict__ p, float v) { *p = v; }
-
-}  // namespace
 
 gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, const float* X, int K, int sweeps,
                            double omega, double alpha, double eta_max, double delta_bar, double eps, int kmax,
@@ -78,68 +30,99 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
         return off;
     };
     const size_t o_dG = add(8 * (size_t)nc), o_dP = add(8 * (size_t)nc), o_dw = add(4 * (size_t)mc),
-                 o_g = add(4 * (size_t)mc), o_saved = add(4 * ((size_t)nc * (K + 1) + K)), o_sc = add(64);
+                 o_y0 = add(4 * (size_t)nc * K), o_Rf = add(4 * (size_t)K), o_mass = add(4 * (size_t)nc),
+                 o_state = add(sizeof(ScaleState)), o_loss = add(4 * (size_t)kmax), o_lam = add(8 * (size_t)kmax);
     void* base;
     GR_TRY_CUDA(fine, fine->ws.get(WS_SCALE, need, &base), "scaling scratch");
     char* B = (char*)base;
     double* dG = (double*)(B + o_dG);
     double* dP = (double*)(B + o_dP);
     float* dw = (float*)(B + o_dw);
-    float* grad = (float*)(B + o_g);
-    float* saved = (float*)(B + o_saved);
-    float* loss = (float*)(B + o_sc);
-    float* one = loss + 1;
-    unsigned long long* lmin = (unsigned long long*)(B + o_sc + 8);
+    float* y0 = (float*)(B + o_y0);
+    float* Rf = (float*)(B + o_Rf);
+    float* mass = (float*)(B + o_mass);
+    ScaleState* state = (ScaleState*)(B + o_state);
+    float* lossd = (float*)(B + o_loss);
+    unsigned long long* lam = (unsigned long long*)(B + o_lam);  // per update: bits of the smallest d_G / d_P after it
     int64_t* hs = host_scratch();
     if (!hs) return set_error(fine, GR_ENOMEM, "scale_edges: pinned scratch unavailable");
-    const unsigned gn = (unsigned)ceil_div(nc > 0 ? nc : 1, ST), gm = (unsigned)ceil_div(mc > 0 ? mc : 1, ST);
 
+    bool bad = false;
+    gr_status st = loss_fine(fine, coarse, agg, X, K, y0, Rf, mass, &bad);
+    if (st != GR_OK) return st;
+    if (bad) return set_error(fine, GR_EINVAL, "scale_edges: agg labels must lie in [0, coarse n)");
+    LossWork W;
+    st = loss_work(coarse, K, sweeps, true, &W);
+    if (st != GR_OK) return st;
+    GR_TRY_CUDA(fine, cudaMemcpyAsync(W.Y, y0, 4 * (size_t)nc * K, cudaMemcpyDeviceToDevice, s), "copy");
     GR_TRY_CUDA(fine, cudaMemsetAsync(dw, 0, 4 * (size_t)mc, s), "memset");
-    k_set_f32<<<1, 1, 0, s>>>(one, 1.0f);
-    count_launch();
-    k_row_weight_sums<<<gn, ST, 0, s>>>(nc, coarse->rowptr, coarse->eid, w, dG);
-    count_launch();
-    GR_TRY_CUDA(fine, cudaMemcpyAsync(dP, dG, 8 * (size_t)nc, cudaMemcpyDeviceToDevice, s), "copy");
-    const double step_delta = pow(delta_bar, 1.0 / kmax);  // per-iteration share of the bound
-    double lam1 = 1.0, eta = eta_max, L0 = 0.0, L_prev = 0.0;
-    int it = 0;
+    GR_TRY_CUDA(fine, cudaMemsetAsync(state, 0, sizeof(ScaleState), s), "memset");
+    GR_TRY_CUDA(fine, cudaMemsetAsync(lam, 0xff, 8 * (size_t)kmax, s), "memset");
+
+    ScaleStep step;
+    step.state = state;
+    step.eta_max = eta_max;
+    step.eps = eps;
+    step.bound_step = pow(delta_bar, 1.0 / kmax);  // per-iteration share of the bound
+    step.alpha = alpha;
+    step.dG = dG;
+    step.dP = dP;
+    step.dw = dw;
+    step.w = w;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    auto done = [&](gr_status r) {
+        for (cudaEvent_t e : ev)
+            if (e) cudaEventDestroy(e);
+        return r;
+    };
+    for (cudaEvent_t& e : ev)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
+            return done(set_error(fine, GR_ECUDA, "scale_edges: event"));
+    auto cuda = [&](cudaError_t e) { return e == cudaSuccess ? GR_OK : cuda_error(fine, e, "scale_edges"); };
+    bool stopped = false;
     for (int k = 1; k <= kmax; ++k) {
-        gr_status st = loss_fwd_impl(fine, coarse, agg, X, K, w, sweeps, omega, loss, saved);
-        if (st != GR_OK) return st;
-        GR_TRY_CUDA(fine, cudaMemcpyAsync(hs, loss, 4, cudaMemcpyDeviceToHost, s), "readback");
-        GR_TRY_CUDA(fine, cudaStreamSynchronize(s), "sync");
-        const double L = (double)((const float*)hs)[0];
-        if (k == 1) L0 = L;
-        if (k > 1 && (L_prev - L) / L < eps) break;  // convergence test
-        st = loss_bwd_impl(coarse, saved, K, w, sweeps, omega, one, grad);
-        if (st != GR_OK) return st;
-        if (mc > 0) {
-            k_sgd_edges<<<gm, ST, 0, s>>>(mc, coarse->eu, coarse->ev, grad, dG, dP, lam1 * step_delta, alpha, eta,
-                                         dw, w);
-            count_launch();
+        const int slot = k & 1;
+        if (k > 2) {  // has iteration k - 2 ended the loop?
+            if ((st = cuda(cudaEventSynchronize(ev[slot]))) != GR_OK) return done(st);
+            if (((const int32_t*)hs)[slot]) {
+                stopped = true;
+                break;
+            }
         }
-        k_row_weight_sums<<<gn, ST, 0, s>>>(nc, coarse->rowptr, coarse->eid, w, dP);
-        count_launch();
-        GR_TRY_CUDA(fine, cudaMemsetAsync(lmin, 0xff, 8, s), "memset");
-        k_min_ratio<<<gn, ST, 0, s>>>(nc, dG, dP, lmin);
-        count_launch();
-        GR_TRY_CUDA(fine, cudaMemcpyAsync(hs, lmin, 8, cudaMemcpyDeviceToHost, s), "readback");
-        GR_TRY_CUDA(fine, cudaStreamSynchronize(s), "sync");
-        const unsigned long long bits = ((const unsigned long long*)hs)[0];
-        if (bits != ~0ull) {
-            double r;
-            memcpy(&r, &bits, 8);
-            lam1 = r;  // new lambda_1 estimate
+        if (k == 1) {
+            st = loss_weights(coarse, w, W, dG, nullptr, nullptr);
+            if (st == GR_OK) st = cuda(cudaMemcpyAsync(dP, dG, 8 * (size_t)nc, cudaMemcpyDeviceToDevice, s));
+        } else {
+            st = loss_weights(coarse, w, W, dP, dG, lam + (k - 2));
         }
-        eta = (L / L0) * eta_max;  // step size from the loss ratio
-        if (loss_hist) loss_hist[it] = L;
-        if (lam1_hist) lam1_hist[it] = lam1;
-        ++it;
-        L_prev = L;
+        if (st != GR_OK) return done(st);
+        step.lam_prev = k > 1 ? lam + (k - 2) : nullptr;
+        step.loss_hist = lossd + (k - 1);
+        st = loss_coarse(coarse, K, sweeps, omega, W.Y, Rf, mass, W, true, nullptr, nullptr, step);
+        if (st == GR_OK) st = loss_adjoint(coarse, K, sweeps, omega, mass, W, nullptr, step);
+        if (st == GR_OK) st = cuda(cudaMemcpyAsync((int32_t*)hs + slot, &state->stop, 4, cudaMemcpyDeviceToHost, s));
+        if (st == GR_OK) st = cuda(cudaEventRecord(ev[slot], s));
+        if (st != GR_OK) return done(st);
     }
-    if (iters_out) *iters_out = it;
-    GR_TRY_CUDA(fine, cudaGetLastError(), "scale_edges kernels");
-    return GR_OK;
+    // lambda_1 after the last update
+    if (!stopped) st = loss_weights(coarse, w, W, dP, dG, lam + (kmax - 1));
+    ScaleState end;
+    std::vector<float> hl((size_t)kmax);
+    std::vector<unsigned long long> hm((size_t)kmax);
+    if (st == GR_OK) st = cuda(cudaMemcpyAsync(&end, state, sizeof(end), cudaMemcpyDeviceToHost, s));
+    if (st == GR_OK) st = cuda(cudaMemcpyAsync(hl.data(), lossd, 4 * (size_t)kmax, cudaMemcpyDeviceToHost, s));
+    if (st == GR_OK) st = cuda(cudaMemcpyAsync(hm.data(), lam, 8 * (size_t)kmax, cudaMemcpyDeviceToHost, s));
+    const gr_status sync = cuda(cudaStreamSynchronize(s));
+    if (st == GR_OK) st = sync;
+    if (st != GR_OK) return done(st);
+    double lam1 = 1.0;
+    for (int i = 0; i < end.it; ++i) {
+        if (hm[i] != ~0ull) memcpy(&lam1, &hm[i], 8);
+        if (loss_hist) loss_hist[i] = (double)hl[i];
+        if (lam1_hist) lam1_hist[i] = lam1;
+    }
+    if (iters_out) *iters_out = end.it;
+    return done(cuda(cudaGetLastError()));
 }
 
 }  // namespace gr

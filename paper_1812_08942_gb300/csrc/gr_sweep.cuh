@@ -68,14 +68,13 @@ __device__ __forceinline__ void sum_partial_rows(const double* base, int nrows, 
 }
 
 // Called by every thread of a block once its partial row part[blockIdx.x]
-// (2K doubles: the K column sums, then the K sums of squares) is written and
-// fenced.  The last block overall writes mu = s1 / n and 1 / s with
-// s^2 = s2 - n mu^2 into stats_out.  NT >= 2K threads take part in the sums.
+// (2K doubles) is written and fenced.  True in the last block overall, with
+// the totals of the 2K columns in red (NT doubles of shared memory, visible
+// to the whole block); the tickets are zero again.  NT >= 2K threads take
+// part in the sums.
 template <int K, int NT>
-__device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64_t n,
-                             double* __restrict__ stats_out) {
+__device__ bool finish_partials(double* part, int nblocks, unsigned* counter, double* red) {
     constexpr int NS = 2 * K;
-    __shared__ double red[NT];
     __shared__ int s_go;
     const int t = threadIdx.x;
     const int g = blockIdx.x / STATS_GROUP, g0 = g * STATS_GROUP;
@@ -84,7 +83,7 @@ __device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64
     unsigned* gcount = counter + STATS_GCOUNT_OFF;
     if (t == 0) s_go = atomicAdd(gcount + g, 1u) == (unsigned)(gs - 1);
     __syncthreads();
-    if (!s_go) return;
+    if (!s_go) return false;
     __threadfence();
     sum_partial_rows<K, NT>(part + (int64_t)g0 * NS, gs, NS, red);
     // every row of the group has been read (barrier above): the group sum
@@ -95,9 +94,21 @@ __device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64
     __syncthreads();
     if (t == 0) s_go = atomicAdd(counter, 1u) == (unsigned)(ngroups - 1);
     __syncthreads();
-    if (!s_go) return;
+    if (!s_go) return false;
     __threadfence();
     sum_partial_rows<K, NT>(part, ngroups, (int64_t)STATS_GROUP * NS, red);
+    if (t == 0) *counter = 0u;
+    return true;
+}
+
+// The last block writes mu = s1 / n and 1 / s with s^2 = s2 - n mu^2 into
+// stats_out, from partial rows of K column sums, then K sums of squares.
+template <int K, int NT>
+__device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64_t n,
+                             double* __restrict__ stats_out) {
+    __shared__ double red[NT];
+    if (!finish_partials<K, NT>(part, nblocks, counter, red)) return;
+    const int t = threadIdx.x;
     if (t < K) {
         double s1 = red[t], s2 = red[K + t];
         double mu = s1 / (double)n;
@@ -106,7 +117,6 @@ __device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64
         stats_out[t] = mu;
         stats_out[K + t] = sd > 0.0 ? 1.0 / sd : 1.0;
     }
-    if (t == 0) *counter = 0u;
 }
 
 }  // namespace gr
