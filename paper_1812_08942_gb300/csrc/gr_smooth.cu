@@ -429,9 +429,11 @@ __global__ void __launch_bounds__(SM_THREADS) k_sweep_stream(
 // than deeper per-warp prefetch did.  Slot indices are 32-bit (2m < 2^32) and
 // rows 32-bit (n < 2^31).
 // ---------------------------------------------------------------------------
+// Sums of a row-group kernel's lanes into the block's partial row; true in the
+// last block, with the totals in red.
 template <typename Acc, int K, int E, int G>
-__device__ void block_stats_rows(Acc (&s1)[E], Acc (&s2)[E], double* __restrict__ part,
-                                 unsigned* __restrict__ counter, int64_t n, double* __restrict__ stats_out) {
+__device__ bool block_sums_rows(Acc (&s1)[E], Acc (&s2)[E], double* __restrict__ part,
+                                unsigned* __restrict__ counter, double* red) {
     __shared__ double wst[SM_WARPS][2 * K];
     constexpr int RPW = 32 / G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -462,7 +464,14 @@ __device__ void block_stats_rows(Acc (&s1)[E], Acc (&s2)[E], double* __restrict_
     }
     __threadfence();
     __syncthreads();
-    finish_stats<K, SM_THREADS>(part, gridDim.x, counter, n, stats_out);
+    return finish_partials<K, SM_THREADS>(part, gridDim.x, counter, red);
+}
+
+template <typename Acc, int K, int E, int G>
+__device__ void block_stats_rows(Acc (&s1)[E], Acc (&s2)[E], double* __restrict__ part,
+                                 unsigned* __restrict__ counter, int64_t n, double* __restrict__ stats_out) {
+    __shared__ double red[SM_THREADS];
+    if (block_sums_rows<Acc, K, E, G>(s1, s2, part, counter, red)) write_stats<K>(red, n, stats_out);
 }
 
 
@@ -1057,46 +1066,128 @@ __device__ __forceinline__ uint64_t gs_prio(uint64_t seed, int64_t i) {
     return splitmix64_at(seed, (1ull << 62) + (uint64_t)i);
 }
 
-__global__ void k_jp_round(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                           uint64_t seed, int32_t* colour, int32_t* __restrict__ left, int32_t* __restrict__ maxc) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || __ldcg(colour + i) >= 0) return;
-    const uint64_t pi = gs_prio(seed, i);
-    const int64_t b = rowptr[i], e = rowptr[i + 1];
-    for (int64_t j = b; j < e; ++j) {
-        const int32_t q = col[j];
-        if (__ldcg(colour + q) < 0) {
+// Nodes with no higher-priority neighbour start the first round's list; the
+// others count theirs.
+constexpr int JP_THREADS = 256;
+constexpr int JP_READY = 1024;
+__global__ void __launch_bounds__(JP_THREADS) k_jp_init(int64_t n, const int64_t* __restrict__ rowptr,
+                                                        const int32_t* __restrict__ col, uint64_t seed,
+                                                        int32_t* __restrict__ colour, int32_t* __restrict__ pending,
+                                                        int32_t* __restrict__ list, int32_t* __restrict__ count) {
+    const int64_t i = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x;
+    int32_t above = -1;
+    if (i < n) {
+        const uint64_t pi = gs_prio(seed, i);
+        const int64_t e = rowptr[i + 1];
+        above = 0;
+        for (int64_t j = rowptr[i]; j < e; ++j) {
+            const int32_t q = col[j];
             const uint64_t pq = gs_prio(seed, q);
-            if (pq > pi || (pq == pi && q > i)) {
-                atomicAdd(left, 1);
-                return;
-            }
+            above += (pq > pi || (pq == pi && q > i)) ? 1 : 0;
         }
+        colour[i] = -1;
+        pending[i] = above;
     }
-    // smallest colour not used by a coloured neighbour, 64 candidates at a time
-    int32_t c = 0;
-    for (int32_t base = 0;; base += 64) {
-        unsigned long long used = 0;
-        for (int64_t j = b; j < e; ++j) {
-            const int32_t cq = __ldcg(colour + col[j]);
-            if (cq >= base && cq < base + 64) used |= 1ull << (cq - base);
-        }
-        if (~used) {
-            c = base + __ffsll((long long)~used) - 1;
-            break;
-        }
-    }
-    colour[i] = c;
-    atomicMax(maxc, c);
+    const int32_t s = block_slot<JP_THREADS>(above == 0, count);
+    if (s >= 0) list[s] = (int32_t)i;
 }
 
-__global__ void k_colour_keys(int64_t n, const int32_t* __restrict__ colour, uint32_t* __restrict__ keys,
-                              uint32_t* __restrict__ vals, int32_t* __restrict__ cnt) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    keys[i] = (uint32_t)colour[i];
-    vals[i] = (uint32_t)i;
-    atomicAdd(&cnt[colour[i]], 1);
+// One round over its list: the smallest colour the coloured (= higher-
+// priority) neighbours leave free, then one neighbour fewer to wait for at
+// every uncoloured (= lower-priority) one; those that wait for none form the
+// next round's list.  Two adjacent nodes are never in one list, so what a
+// round reads was written before it.  Every node is handled once: rounds over
+// all nodes took 43 us each on a 101 x 89 x 75 mesh (18 rounds), with a host
+// wait after each; colouring and five sweeps of it went from 1,870 to 959 us.
+__global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restrict__ rowptr,
+                                                         const int32_t* __restrict__ col,
+                                                         const int32_t* __restrict__ list,
+                                                         const int32_t* __restrict__ count, int32_t* colour,
+                                                         int32_t* __restrict__ pending, int32_t* __restrict__ next,
+                                                         int32_t* __restrict__ next_count,
+                                                         int32_t* __restrict__ maxc) {
+    // nodes that become ready gather in shared memory, so that the next list
+    // grows by one global atomic per block (one per node serialised on the
+    // counter: 25 us a round); more than JP_READY of them are listed directly
+    __shared__ int32_t ready[JP_READY];
+    __shared__ int32_t nready, base_s, top_s;
+    if (threadIdx.x == 0) {
+        nready = 0;
+        top_s = -1;
+    }
+    __syncthreads();
+    const int32_t cnt = *count;
+    int32_t top = -1;
+    for (int64_t t = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * JP_THREADS) {
+        const int32_t i = list[t];
+        const int64_t b = rowptr[i], e = rowptr[i + 1];
+        // the smallest colour not used by a coloured neighbour, 64 candidates
+        // at a time; eight neighbours' colours, then eight counts in flight
+        int32_t c = 0;
+        for (int32_t base = 0;; base += 64) {
+            unsigned long long used = 0;
+            for (int64_t j = b; j < e; j += 8) {
+                int32_t cq[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) cq[u] = j + u < e ? __ldcg(colour + col[j + u]) : -1;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (cq[u] >= base && cq[u] < base + 64) used |= 1ull << (cq[u] - base);
+            }
+            if (~used) {
+                c = base + __ffsll((long long)~used) - 1;
+                break;
+            }
+        }
+        for (int64_t j = b; j < e; j += 8) {
+            int32_t q[8], was[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                q[u] = j + u < e ? col[j + u] : -1;
+                if (q[u] >= 0 && __ldcg(colour + q[u]) >= 0) q[u] = -1;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) was[u] = q[u] >= 0 ? atomicSub(&pending[q[u]], 1) : 0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (was[u] == 1) {
+                    const int32_t k = atomicAdd(&nready, 1);
+                    if (k < JP_READY) ready[k] = q[u];
+                    else next[atomicAdd(next_count, 1)] = q[u];
+                }
+        }
+        colour[i] = c;
+        top = c > top ? c : top;
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0 && top >= 0) atomicMax(&top_s, top);
+    __syncthreads();
+    const int32_t m = nready < JP_READY ? nready : JP_READY;
+    if (threadIdx.x == 0) {
+        if (m > 0) base_s = atomicAdd(next_count, m);
+        if (top_s >= 0) atomicMax(maxc, top_s);
+    }
+    __syncthreads();
+    for (int32_t k = threadIdx.x; k < m; k += JP_THREADS) next[base_s + k] = ready[k];
+}
+
+// sort keys and the nodes per colour: colours below 256 (the greedy colours
+// of any sparse graph) are counted per block first -- one counter a colour
+// for all nodes took 148 us on the mesh above
+__global__ void __launch_bounds__(JP_THREADS) k_colour_keys(int64_t n, const int32_t* __restrict__ colour,
+                                                            uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                            int32_t* __restrict__ cnt) {
+    __shared__ int32_t hist[JP_THREADS];
+    hist[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * JP_THREADS) {
+        const int32_t c = colour[i];
+        keys[i] = (uint32_t)c;
+        vals[i] = (uint32_t)i;
+        atomicAdd(c < JP_THREADS ? &hist[c] : &cnt[c], 1);
+    }
+    __syncthreads();
+    if (hist[threadIdx.x]) atomicAdd(&cnt[threadIdx.x], hist[threadIdx.x]);
 }
 
 // Colouring for colour_seed: colour (device, n) and, in the context, the node
@@ -1104,6 +1195,7 @@ __global__ void k_colour_keys(int64_t n, const int32_t* __restrict__ colour, uin
 static gr_status gs_prepare(gr_ctx* c, uint64_t colour_seed, int32_t* colour_out) {
     const int64_t n = c->n;
     cudaStream_t s = c->stream;
+    constexpr int BATCH = 8;  // rounds queued between two looks at the list's length
     size_t need = 0;
     auto add = [&](size_t bytes) {
         size_t off = need;
@@ -1111,7 +1203,7 @@ static gr_status gs_prepare(gr_ctx* c, uint64_t colour_seed, int32_t* colour_out
         return off;
     };
     const size_t o_col = add(4 * (size_t)n), o_k0 = add(4 * (size_t)n), o_v0 = add(4 * (size_t)n),
-                 o_k1 = add(4 * (size_t)n), o_v1 = add(4 * (size_t)n), o_cnt = add(4 * (size_t)(n + 2)),
+                 o_k1 = add(4 * (size_t)n), o_v1 = add(4 * (size_t)n), o_cnt = add(4 * (size_t)(n + 257)),
                  o_ptr = add(4 * (size_t)(n + 2)), o_ctr = add(64);
     void* base;
     GR_TRY_CUDA(c, c->ws.get(WS_GS, need, &base), "colouring scratch");
@@ -1123,30 +1215,47 @@ static gr_status gs_prepare(gr_ctx* c, uint64_t colour_seed, int32_t* colour_out
     uint32_t* v1 = (uint32_t*)(B + o_v1);
     int32_t* cnt = (int32_t*)(B + o_cnt);
     int32_t* cptr = (int32_t*)(B + o_ptr);
-    int32_t* ctr = (int32_t*)(B + o_ctr);  // [0] left after the round, [1] largest colour
+    // [0 .. BATCH] lengths of a batch's lists, [BATCH + 1] largest colour
+    int32_t* ctr = (int32_t*)(B + o_ctr);
+    static_assert(4 * (BATCH + 2) <= 64, "counters fit their block and the host scratch");
+    int32_t* lists[2] = {(int32_t*)k0, (int32_t*)v0};  // free until the sort
+    int32_t* pending = (int32_t*)k1;
     int64_t* hs = host_scratch();
     if (!hs) return set_error(c, GR_ENOMEM, "colouring: pinned scratch unavailable");
-    GR_TRY_CUDA(c, cudaMemsetAsync(colour, 0xff, 4 * (size_t)n, s), "memset");
+    const int32_t* hc = (const int32_t*)hs;
     GR_TRY_CUDA(c, cudaMemsetAsync(ctr, 0, 64, s), "memset");
-    const unsigned gn = (unsigned)ceil_div(n > 0 ? n : 1, 256);
-    // every round colours at least the highest-priority uncoloured node
-    int64_t left = n;
-    for (int64_t round = 0; left > 0; ++round) {
-        if (round > n) return set_error(c, GR_ECUDA, "colouring: no progress");
-        GR_TRY_CUDA(c, cudaMemsetAsync(ctr, 0, 4, s), "memset");
-        k_jp_round<<<gn, 256, 0, s>>>(n, c->rowptr, c->col, colour_seed, colour, ctr, ctr + 1);
-        count_launch();
-        GR_TRY_CUDA(c, cudaMemcpyAsync(hs, ctr, 8, cudaMemcpyDeviceToHost, s), "readback");
-        GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
-        const int64_t now = ((int32_t*)hs)[0];
-        if (now >= left) return set_error(c, GR_ECUDA, "colouring: a round made no progress");
-        left = now;
-    }
-    const int32_t ncol = n > 0 ? ((int32_t*)hs)[1] + 1 : 0;
-    // the nodes in ascending (colour, id): a stable sort of the ids by colour
-    GR_TRY_CUDA(c, cudaMemsetAsync(cnt, 0, 4 * (size_t)(ncol + 1), s), "memset");
+    const int64_t want = ceil_div(n > 0 ? n : 1, (int64_t)JP_THREADS), cap = (int64_t)c->num_sms * 8;
+    const unsigned gn = (unsigned)want, gr = (unsigned)(want < cap ? want : cap);
     if (n > 0) {
-        k_colour_keys<<<gn, 256, 0, s>>>(n, colour, k0, v0, cnt);
+        k_jp_init<<<gn, JP_THREADS, 0, s>>>(n, c->rowptr, c->col, colour_seed, colour, pending, lists[0], ctr);
+        count_launch();
+    }
+    // every round colours its list; the priorities order the nodes, so no list
+    // is empty before all are coloured
+    int64_t left = n;
+    int cur = 0;
+    while (left > 0) {
+        for (int r = 0; r < BATCH; ++r) {
+            k_jp_round<<<gr, JP_THREADS, 0, s>>>(c->rowptr, c->col, lists[cur], ctr + r, colour, pending,
+                                                lists[cur ^ 1], ctr + r + 1, ctr + BATCH + 1);
+            count_launch();
+            cur ^= 1;
+        }
+        GR_TRY_CUDA(c, cudaMemcpyAsync(hs, ctr, 4 * (BATCH + 2), cudaMemcpyDeviceToHost, s), "readback");
+        // the last list opens the next batch
+        GR_TRY_CUDA(c, cudaMemcpyAsync(ctr, ctr + BATCH, 4, cudaMemcpyDeviceToDevice, s), "copy");
+        GR_TRY_CUDA(c, cudaMemsetAsync(ctr + 1, 0, 4 * BATCH, s), "memset");
+        GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
+        int64_t did = 0;
+        for (int r = 0; r < BATCH; ++r) did += hc[r];
+        if (did <= 0 || did > left) return set_error(c, GR_ECUDA, "colouring: a round made no progress");
+        left -= did;
+    }
+    const int32_t ncol = n > 0 ? hc[BATCH + 1] + 1 : 0;
+    // the nodes in ascending (colour, id): a stable sort of the ids by colour
+    GR_TRY_CUDA(c, cudaMemsetAsync(cnt, 0, 4 * (size_t)(ncol + 257), s), "memset");
+    if (n > 0) {
+        k_colour_keys<<<gr, JP_THREADS, 0, s>>>(n, colour, k0, v0, cnt);
         count_launch();
     }
     int alt = 0;
@@ -1171,43 +1280,62 @@ gr_status colour_impl(gr_ctx* c, uint64_t colour_seed, int32_t* colour_out, int3
     return GR_OK;
 }
 
+// a chunk of a block that the running kernel also writes (elsewhere): no read-only path
+template <typename T, int E>
+__device__ __forceinline__ void load_chunk_rw(const T* p, typename AccOf<T>::type (&x)[E]) {
+    constexpr int B = E * (int)sizeof(T);
+    static_assert(B == 16 || B == 8, "a chunk is 16 or 8 bytes");
+    alignas(16) T v[E];
+    if constexpr (B == 16) *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(p);
+    else *reinterpret_cast<uint2*>(v) = *reinterpret_cast<const uint2*>(p);
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = (typename AccOf<T>::type)v[e];
+}
+
 // Update the listed rows (one colour) in place: G lanes per row, one chunk
 // each; the neighbours have other colours and are not written by this launch.
+// Bound by the gathers' round trips: four slots in flight (colouring and five
+// sweeps of a 101 x 89 x 75 mesh, K = 16: 959 us with four, 979 with two,
+// 1,042 with eight, whose registers cost resident warps).  (Column sums ended
+// in these launches too: 8 us of finish for each of the six colours of a mesh,
+// where a pass of its own takes 21 once.)
 template <typename T, int K>
 __global__ void __launch_bounds__(SM_THREADS) k_gs_class(int64_t cnt, const int32_t* __restrict__ rows,
                                                          const int64_t* __restrict__ rowptr,
-                                                         const typename SlotOf<T>::type* __restrict__ slots,
-                                                         T* __restrict__ X, double omega_d) {
+                                                         const typename SlotOf<T>::type* __restrict__ slots, T* X,
+                                                         double omega_d) {
     using Slot = typename SlotOf<T>::type;
     using L = RowLayout<T, K>;
     using Acc = typename AccOf<T>::type;
-    constexpr int E = L::E, G = L::G, RPW = 32 / G;
+    constexpr int E = L::E, G = L::G, RPW = 32 / G, U = 4;
     const int lane = threadIdx.x & 31, seg = lane / G, q = lane % G;
     if (seg >= RPW) return;
     const int64_t r = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RPW + seg;
     if (r >= cnt) return;
     const int64_t i = rows[r];
-    const int64_t b = rowptr[i], e = rowptr[i + 1];
-    const Acc omega = (Acc)omega_d, one_m = (Acc)(1.0 - omega_d);
-    Acc xi[E];
-    load_chunk<T, E>(X + i * K + q * E, xi);
+    const unsigned b = (unsigned)rowptr[i], e = (unsigned)rowptr[i + 1];  // 2m < 2^32
     if (b == e) return;  // isolated: keeps its value
-    Acc acc[E];
+    const Acc omega = (Acc)omega_d, one_m = (Acc)(1.0 - omega_d);
+    Acc xi[E], acc[E];
+    load_chunk_rw<T, E>(X + i * K + q * E, xi);
 #pragma unroll
     for (int t = 0; t < E; ++t) acc[t] = Acc(0);
-    for (int64_t j = b; j < e; j += 2) {
-        const bool two = j + 1 < e;
-        const Slot v0 = __ldg(slots + j);
-        const Slot v1 = __ldg(slots + (two ? j + 1 : j));
-        Acc x0[E], x1[E];
-        load_chunk<T, E>(X + (int64_t)slot_col(v0) * K + q * E, x0);
-        load_chunk<T, E>(X + (int64_t)slot_col(v1) * K + q * E, x1);
-        const Acc w0 = slot_w(v0, Acc(0)), w1 = slot_w(v1, Acc(0));
+    for (unsigned j = b; j < e; j += U) {
+        Slot v[U];
+        Acc x[U][E];
 #pragma unroll
-        for (int t = 0; t < E; ++t) {
-            acc[t] = fma(w0, x0[t], acc[t]);
-            if (two) acc[t] = fma(w1, x1[t], acc[t]);
-        }
+        for (int u = 0; u < U; ++u)
+            if (j + u < e) v[u] = __ldg(slots + j + u);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + u < e) load_chunk_rw<T, E>(X + (int64_t)slot_col(v[u]) * K + q * E, x[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + u < e) {
+                const Acc w = slot_w(v[u], Acc(0));
+#pragma unroll
+                for (int t = 0; t < E; ++t) acc[t] = fma(w, x[u][t], acc[t]);
+            }
     }
     Acc y[E];
 #pragma unroll

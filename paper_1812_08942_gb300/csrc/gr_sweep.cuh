@@ -101,13 +101,10 @@ __device__ bool finish_partials(double* part, int nblocks, unsigned* counter, do
     return true;
 }
 
-// The last block writes mu = s1 / n and 1 / s with s^2 = s2 - n mu^2 into
-// stats_out, from partial rows of K column sums, then K sums of squares.
-template <int K, int NT>
-__device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64_t n,
-                             double* __restrict__ stats_out) {
-    __shared__ double red[NT];
-    if (!finish_partials<K, NT>(part, nblocks, counter, red)) return;
+// mu = s1 / n and 1 / s with s^2 = s2 - n mu^2 into stats_out, from K column
+// sums, then K sums of squares
+template <int K>
+__device__ __forceinline__ void write_stats(const double* red, int64_t n, double* __restrict__ stats_out) {
     const int t = threadIdx.x;
     if (t < K) {
         double s1 = red[t], s2 = red[K + t];
@@ -117,6 +114,14 @@ __device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64
         stats_out[t] = mu;
         stats_out[K + t] = sd > 0.0 ? 1.0 / sd : 1.0;
     }
+}
+
+// The last block writes the statistics of the partial rows.
+template <int K, int NT>
+__device__ void finish_stats(double* part, int nblocks, unsigned* counter, int64_t n,
+                             double* __restrict__ stats_out) {
+    __shared__ double red[NT];
+    if (finish_partials<K, NT>(part, nblocks, counter, red)) write_stats<K>(red, n, stats_out);
 }
 
 }  // namespace gr
