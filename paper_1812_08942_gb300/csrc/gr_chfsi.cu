@@ -122,22 +122,39 @@ __global__ void k_cf_values(int64_t n, const int64_t* __restrict__ rowptr, const
 }
 
 // Out = c1 (A Y) + c2 Y + c3 Yp (Yp may be NULL), n x p row-major, A from
-// its slot values av and diagonal ad.  Short rows: warp per row, lanes over
-// columns, the row's products in slot order.
+// its slot values av and diagonal ad.  Short rows: W lanes per row (16 for
+// p <= 16, else a warp), lanes over columns, the row's products in slot order.
+// A filter step on a thousand rows is bound by its round trips: eight slots'
+// neighbour rows are fetched together (1,000 rows of 13 slots, p = 16: 5.9 us a
+// step; one slot at a time and a warp per row of 16 columns 6.8).
+template <int W>
 __global__ void k_cf_apply(int64_t n, int p, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                            const double* __restrict__ av, const double* __restrict__ ad, double c1, double c2,
                            double c3, const double* __restrict__ Y, const double* __restrict__ Yp,
                            double* __restrict__ Out) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
-         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    constexpr int U = 8;
+    const int lane = threadIdx.x % W;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W; i < n;
+         i += ((int64_t)gridDim.x * blockDim.x) / W) {
         const int64_t j0 = rowptr[i], j1 = rowptr[i + 1];
-        for (int q = lane; q < p; q += 32) {
+        for (int q = lane; q < p; q += W) {
             const double yi = Y[i * p + q];
+            const double yp = Yp ? Yp[i * p + q] : 0.0;
             double acc = ad[i] * yi;
-            for (int64_t j = j0; j < j1; ++j) acc += av[j] * Y[(int64_t)col[j] * p + q];
+            for (int64_t j = j0; j < j1; j += U) {
+                double a[U], y[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (j + u < j1) {
+                        a[u] = av[j + u];
+                        y[u] = Y[(int64_t)col[j + u] * p + q];
+                    }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (j + u < j1) acc += a[u] * y[u];
+            }
             double o = c1 * acc + c2 * yi;
-            if (Yp) o += c3 * Yp[i * p + q];
+            if (Yp) o += c3 * yp;
             Out[i * p + q] = o;
         }
     }
@@ -260,9 +277,21 @@ __global__ void k_cf_resid(int64_t n, int p, int k, const double* __restrict__ A
     const int64_t r0 = (int64_t)blockIdx.x * chunk, r1 = r0 + chunk < n ? r0 + chunk : n;
     const double th = theta[c];
     double t = 0.0;
-    for (int64_t i = r0; i < r1; ++i) {
-        const double r = AX[i * p + c] - th * X[i * p + c];
-        t += r * r;
+    constexpr int U = 8;  // rows in flight (a row's loads at a time: 33 us)
+    for (int64_t i = r0; i < r1; i += U) {
+        double a[U], x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < r1) {
+                a[u] = AX[(i + u) * p + c];
+                x[u] = X[(i + u) * p + c];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < r1) {
+                const double r = a[u] - th * x[u];
+                t += r * r;
+            }
     }
     part[(int64_t)blockIdx.x * k + c] = t;
 }
@@ -491,7 +520,8 @@ gr_status coarsest_eigenpairs(gr_ctx* c, const double* b, int k, Workspace& ws, 
         if (long_rows)
             k_cf_apply_long<<<wgrid, CT, 0, s>>>(n, p, c->rowptr, c->col, av, ad, c1, c2, c3, Y, Yp, Out);
         else
-            k_cf_apply<<<wgrid, CT, 0, s>>>(n, p, c->rowptr, c->col, av, ad, c1, c2, c3, Y, Yp, Out);
+            p <= 16 ? k_cf_apply<16><<<wgrid, CT, 0, s>>>(n, p, c->rowptr, c->col, av, ad, c1, c2, c3, Y, Yp, Out)
+                    : k_cf_apply<32><<<wgrid, CT, 0, s>>>(n, p, c->rowptr, c->col, av, ad, c1, c2, c3, Y, Yp, Out);
         count_launch();
     };
     auto gram = [&](const double* Y1, const double* Y2) {

@@ -12,6 +12,8 @@
 #include <vector>
 
 #include "gr_internal.cuh"
+#include "gr_sweep.cuh"
+#include "gr_vec.cuh"
 
 namespace gr {
 
@@ -41,6 +43,19 @@ __global__ void k_prolong(int64_t n, int k, const int32_t* __restrict__ map, con
 // division, taken per entry and iteration, cost more than the row's
 // products.  The keep test reads the sign bit of g with an integer compare
 // (a floating compare would take the FP64 pipe too).
+// a / b for b > 0 to within an ulp or so: an FP32 reciprocal refined by one
+// Newton step, and the quotient corrected by its residual -- five FP64
+// operations where the division takes about ten (388 -> 251 us over the
+// hierarchy of a 128^3 mesh, k = 8); b outside FP32's range divides.  The range test is on the exponent: a floating compare is an FP64
+// operation too.
+__device__ __forceinline__ double quotient(double a, double b) {
+    if ((unsigned)((__double2hiint(b) >> 20) - 923) > 200u) return a / b;  // b in [2^-100, 2^101)
+    double y = f32_to_f64(1.0f / f64_to_f32(b));
+    y = fma(y, fma(-b, y, 1.0), y);
+    const double q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+
 __global__ void k_shift_gain(int64_t n, int k, const double* __restrict__ deg, const double* __restrict__ lam,
                              const double* __restrict__ b, double omega, double* __restrict__ g) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -49,7 +64,7 @@ __global__ void k_shift_gain(int64_t n, int k, const double* __restrict__ deg, c
     const int c = (int)(idx % k);
     const double D = deg[r];
     const double diag = D - lam[c] * (b ? b[r] : 1.0);
-    g[idx] = diag > 0.0 ? omega * D / diag : -1.0;
+    g[idx] = __double2hiint(diag) > 0 ? quotient(omega * D, diag) : (diag > 0.0 ? omega * D / diag : -1.0);
 }
 
 // One iteration, thread per (row, column).
@@ -129,99 +144,139 @@ __global__ void k_base_mass(int64_t n, const double* __restrict__ deg, int norma
     if (i < n) b[i] = normalized ? (deg[i] > 0.0 ? deg[i] : 1.0) : 1.0;
 }
 
-// row-major n x k <-> column-major
-__global__ void k_to_colmajor(int64_t n, int k, const double* __restrict__ U, double* __restrict__ V) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * k) return;
-    V[(idx % k) * n + idx / k] = U[idx];
-}
-__global__ void k_to_rowmajor(int64_t n, int k, const double* __restrict__ V, double* __restrict__ U) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * k) return;
-    U[idx] = V[(idx % k) * n + idx / k];
-}
+// ---------------------------------------------------------------------------
+// Modified Gram-Schmidt in column order, right-looking: step j finishes
+// column j, whose products with the columns after it are then known, and step
+// j + 1 subtracts its share from all of them in the same pass that makes the
+// next products.  The same operations on the same numbers as column-by-column
+// MGS (each column loses its parts along 0, 1, ... in that order), in k passes
+// instead of k (k + 1) / 2 pairs of them.  A thread holds a row, columns are
+// stored one after the other (coalesced; the first pass reads the row-major
+// block and the last writes it), and only the columns that are left are
+// touched.  Bound by the FP64 pipe, k (k + 1) multiply-adds a row (2,097,152 x
+// 8: 285 us at 530 G a second): dots, axpys, divisions and transposes apart
+// took 1,450 us, the passes and the final scaling take 550.
+// ---------------------------------------------------------------------------
+constexpr int MG_BLOCKS = 4;  // per SM
 
-// Sum of one double per thread over the block, in a fixed order.
-__device__ __forceinline__ double block_sum(double s, double* red) {
+// Step with R columns left, of which `left` (<= R) exist: V points at the first
+// of them, prev (NULL: step 0, the columns come from row-major Y) holds the
+// products of the column before it, prev[0] its squared norm.  R is the
+// register width: a column guarded at run time would still take its turn on
+// the FP64 pipe.
+template <int R>
+__global__ void __launch_bounds__(ET, R <= 8 ? MG_BLOCKS : 1) k_mgs_step(int64_t n, int left,
+                                                                        const double* __restrict__ Y, double* V,
+                                                                        const double* __restrict__ prev,
+                                                                        double* part, unsigned* counter,
+                                                                        double* __restrict__ sums) {
+    constexpr int NS = R <= 2 ? 2 : (R + 1) / 2 * 2;
+    __shared__ double red[ET];
+    __shared__ double ws[ET / 32][NS];
+    double acc[R], f[R];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < ET / 32; ++w) t += red[w];
-    __syncthreads();
-    return t;  // valid in thread 0
-}
-
-// Per-block partial of a grid reduction; the last block to arrive adds the
-// partials (thread t takes blocks t, t + ET, ... in order, then block_sum).
-__device__ __forceinline__ void grid_finish(double s, double* __restrict__ part, unsigned* __restrict__ counter,
-                                            double* __restrict__ out) {
-    __shared__ double red[ET / 32];
-    __shared__ bool last;
-    const double t = block_sum(s, red);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = t;
-        __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    for (int i = 0; i < R; ++i) {
+        acc[i] = 0.0;
+        f[i] = prev && i < left ? prev[i + 1] / prev[0] : 0.0;
     }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        double a = 0.0;
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += ET) a += __ldcg(part + b);
-        const double total = block_sum(a, red);
-        if (threadIdx.x == 0) {
-            *out = total;
-            *counter = 0u;
+    for (int64_t r = (int64_t)blockIdx.x * ET + threadIdx.x; r < n; r += (int64_t)gridDim.x * ET) {
+        double v[R];
+        if (!prev) {
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[i] = i < left ? Y[r * left + i] : 0.0;
+        } else {
+            const double p = V[r - n];
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[i] = i < left ? V[(int64_t)i * n + r] : 0.0;
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[i] = fma(-f[i], p, v[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            if (i < left) V[(int64_t)i * n + r] = v[i];
+            acc[i] = fma(v[0], v[i], acc[i]);
         }
     }
-}
-
-// out = a . b over n entries: per-block partials, the last block to finish
-// adds them in block order (one atomic ticket, no wait)
-__global__ void __launch_bounds__(ET) k_dot(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
-                                            double* __restrict__ part, unsigned* __restrict__ counter,
-                                            double* __restrict__ out) {
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += a[i] * b[i];
-    grid_finish(s, part, counter, out);
-}
-
-// y -= r x  (r = *rp)
-__global__ void k_axpy(int64_t n, const double* __restrict__ rp, const double* __restrict__ x,
-                       double* __restrict__ y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] -= (*rp) * x[i];
-}
-
-// y /= sqrt(*nrm2)
-__global__ void k_unit(int64_t n, const double* __restrict__ nrm2, double* __restrict__ y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] /= sqrt(*nrm2);
-}
-
-// per-edge sum over the canonical list of w (x_u - x_v)^2 for column x (= x' L x),
-// with the same block-partial / last-block finish
-__global__ void __launch_bounds__(ET) k_edge_quad(int64_t m, const int32_t* __restrict__ eu,
-                                                  const int32_t* __restrict__ ev, const double* __restrict__ ew,
-                                                  const double* __restrict__ x, double* __restrict__ part,
-                                                  unsigned* __restrict__ counter, double* __restrict__ out) {
-    double s = 0.0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const double d = x[eu[e]] - x[ev[e]];
-        s += ew[e] * d * d;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        double t = acc[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) ws[warp][i] = t;
     }
-    grid_finish(s, part, counter, out);
+    __syncthreads();
+    if (threadIdx.x < NS) {
+        double t = 0.0;
+        if (threadIdx.x < R)
+            for (int w = 0; w < ET / 32; ++w) t += ws[w][threadIdx.x];
+        part[(int64_t)blockIdx.x * NS + threadIdx.x] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (finish_partials<NS / 2, ET>(part, gridDim.x, counter, red) && (int)threadIdx.x < left)
+        sums[threadIdx.x] = red[threadIdx.x];
 }
 
-// x' B x for B = D (x' x for B = I uses k_dot)
-__global__ void k_scale_by(int64_t n, const double* __restrict__ x, const double* __restrict__ deg,
-                           double* __restrict__ y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = x[i] * deg[i];
+// U (row-major) = the finished columns over their norms: the first sum of a
+// column's step is its squared norm
+__global__ void __launch_bounds__(ET) k_mgs_take(int64_t n, int k, const double* __restrict__ V,
+                                                 const double* __restrict__ sums, int ld, double* __restrict__ U) {
+    __shared__ double inv[32];
+    if ((int)threadIdx.x < k) inv[threadIdx.x] = 1.0 / sqrt(sums[threadIdx.x * ld]);
+    __syncthreads();
+    for (int64_t r = (int64_t)blockIdx.x * ET + threadIdx.x; r < n; r += (int64_t)gridDim.x * ET)
+        for (int i = 0; i < k; ++i) U[r * k + i] = V[(int64_t)i * n + r] * inv[i];
+}
+
+// x' L x and x' B x of every column: thread per (row, column) over the row's
+// upper edges, w (x_u - x_v)^2, and b x^2 (b NULL: 1).  Column-wise passes
+// over the edge list gathered 8 bytes at a time.  Bound by the FP64 pipe
+// (three operations per edge and column).  out[2 c] and out[2 c + 1].
+__global__ void __launch_bounds__(ET) k_rayleigh(int64_t n, int k, const int64_t* __restrict__ eptr,
+                                                 const int32_t* __restrict__ ev, const double* __restrict__ ew,
+                                                 const double* __restrict__ b, const double* __restrict__ U,
+                                                 double* part, unsigned* counter, double* __restrict__ out) {
+    __shared__ double red[ET], s1[ET], s2[ET];
+    const int rpb = ET / k, c = threadIdx.x % k, rt = threadIdx.x / k;
+    double num = 0.0, den = 0.0;
+    if (rt < rpb)
+        for (int64_t r = (int64_t)blockIdx.x * rpb + rt; r < n; r += (int64_t)gridDim.x * rpb) {
+            const double x = U[r * k + c];
+            const int64_t e1 = eptr[r + 1];
+            constexpr int W = 4;
+            for (int64_t e = eptr[r]; e < e1; e += W) {
+                double y[W], w[W];
+#pragma unroll
+                for (int u = 0; u < W; ++u)
+                    if (e + u < e1) {
+                        y[u] = U[(int64_t)__ldg(ev + e + u) * k + c];
+                        w[u] = __ldg(ew + e + u);
+                    }
+#pragma unroll
+                for (int u = 0; u < W; ++u)
+                    if (e + u < e1) {
+                        const double d = x - y[u];
+                        num = fma(w[u] * d, d, num);
+                    }
+            }
+            den = fma(b ? b[r] * x : x, x, den);
+        }
+    s1[threadIdx.x] = num;
+    s2[threadIdx.x] = den;
+    __syncthreads();
+    if (threadIdx.x < 64) {  // sum 2 q + 0 / 1 of column q
+        const int q = threadIdx.x >> 1;
+        const double* s = (threadIdx.x & 1) ? s2 : s1;
+        double t = 0.0;
+        if (q < k)
+            for (int i = 0; i < rpb; ++i) t += s[i * k + q];
+        part[(int64_t)blockIdx.x * 64 + threadIdx.x] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (finish_partials<32, ET>(part, gridDim.x, counter, red) && (int)threadIdx.x < 2 * k)
+        out[threadIdx.x] = red[threadIdx.x];
 }
 
 }  // namespace
@@ -238,7 +293,8 @@ gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normali
     // reduction partials, scalars
     int64_t nmax = 0;
     for (int l = 0; l < nlevels; ++l) nmax = levels[l]->n > nmax ? levels[l]->n : nmax;
-    const int RB = f->num_sms * 4;  // reduction blocks
+    int RB = f->num_sms * MG_BLOCKS;  // blocks of the reductions
+    if (RB > STATS_GROUP * STATS_MAX_GROUPS) RB = STATS_GROUP * STATS_MAX_GROUPS;
     size_t need = 0;
     auto add = [&](size_t bytes) {
         size_t off = need;
@@ -247,9 +303,9 @@ gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normali
     };
     const size_t o_Y0 = add(sizeof(double) * (size_t)nmax * k), o_Y1 = add(sizeof(double) * (size_t)nmax * k),
                  o_G = add(sizeof(double) * (size_t)nmax * k),
-                 o_V = add(sizeof(double) * (size_t)n0 * k), o_T = add(sizeof(double) * (size_t)n0),
-                 o_part = add(sizeof(double) * (size_t)RB), o_sc = add(sizeof(double) * 64),
-                 o_lam = add(sizeof(double) * 32), o_ctr = add(64);
+                 o_V = add(sizeof(double) * (size_t)n0 * k), o_sums = add(sizeof(double) * 32 * (size_t)k),
+                 o_part = add(sizeof(double) * 64 * (size_t)RB), o_sc = add(sizeof(double) * 64),
+                 o_lam = add(sizeof(double) * 32), o_ctr = add(STATS_COUNTER_BYTES);
     // Galerkin masses of every level: b_0 = 1 or D (degree 0 -> 1), then the
     // member sums level by level
     std::vector<size_t> o_mass;
@@ -261,12 +317,12 @@ gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normali
     double* Y[2] = {(double*)(Bp + o_Y0), (double*)(Bp + o_Y1)};
     double* gain = (double*)(Bp + o_G);
     double* V = (double*)(Bp + o_V);
-    double* T = (double*)(Bp + o_T);
+    double* sums = (double*)(Bp + o_sums);  // per step: the products of its column with those from it on
     double* part = (double*)(Bp + o_part);
     double* sc = (double*)(Bp + o_sc);
     double* lam = (double*)(Bp + o_lam);
     unsigned* ctr = (unsigned*)(Bp + o_ctr);
-    GR_TRY_CUDA(f, cudaMemsetAsync(ctr, 0, 64, s), "memset");
+    GR_TRY_CUDA(f, cudaMemsetAsync(ctr, 0, STATS_COUNTER_BYTES, s), "memset");
     // the diagonal mass of each level (NULL: B = I)
     std::vector<const double*> mass(nlevels, nullptr);
     if (galerkin_mass) {
@@ -324,46 +380,40 @@ gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normali
     }
 
     // 3) modified Gram-Schmidt over the columns (Alg. 5 step 11)
-    k_to_colmajor<<<blocks(n0 * k), ET, 0, s>>>(n0, k, Y[cur], V);
-    count_launch();
-    const unsigned rb = (unsigned)(RB < ceil_div(n0, ET) ? RB : ceil_div(n0 > 0 ? n0 : 1, ET));
-    for (int i = 0; i < k; ++i) {
-        double* ui = V + (int64_t)i * n0;
-        for (int j = 0; j < i; ++j) {
-            const double* uj = V + (int64_t)j * n0;
-            k_dot<<<rb, ET, 0, s>>>(n0, uj, ui, part, ctr, sc);
-            count_launch();
-            k_axpy<<<blocks(n0), ET, 0, s>>>(n0, sc, uj, ui);
-            count_launch();
+    const int64_t rbw = ceil_div(n0 > 0 ? n0 : 1, ET);
+    const unsigned rb = (unsigned)(RB < rbw ? RB : rbw);
+    for (int j = 0; j < k; ++j) {
+        const double* prev = j > 0 ? sums + (size_t)(j - 1) * 32 : nullptr;
+        double* Vj = V + (int64_t)j * n0;
+        const int left = k - j;
+#define GR_MGS(RR) k_mgs_step<RR><<<rb, ET, 0, s>>>(n0, left, Y[cur], Vj, prev, part, ctr, sums + (size_t)j * 32)
+        switch (left) {
+            case 1: GR_MGS(1); break;
+            case 2: GR_MGS(2); break;
+            case 3: GR_MGS(3); break;
+            case 4: GR_MGS(4); break;
+            case 5: GR_MGS(5); break;
+            case 6: GR_MGS(6); break;
+            case 7: GR_MGS(7); break;
+            case 8: GR_MGS(8); break;
+            default:
+                if (left <= 12) GR_MGS(12);
+                else if (left <= 16) GR_MGS(16);
+                else if (left <= 24) GR_MGS(24);
+                else GR_MGS(32);
         }
-        k_dot<<<rb, ET, 0, s>>>(n0, ui, ui, part, ctr, sc);
-        count_launch();
-        k_unit<<<blocks(n0), ET, 0, s>>>(n0, sc, ui);
+#undef GR_MGS
         count_launch();
     }
-    k_to_rowmajor<<<blocks(n0 * k), ET, 0, s>>>(n0, k, V, U_out);
+    k_mgs_take<<<rb, ET, 0, s>>>(n0, k, V, sums, 32, U_out);
     count_launch();
 
     // 4) Rayleigh quotients of the result, x' L x / x' B x
     if (rayleigh_out) {
-        const unsigned rbm = (unsigned)(RB < ceil_div(f->m, ET) ? RB : ceil_div(f->m > 0 ? f->m : 1, ET));
-        for (int i = 0; i < k; ++i) {
-            const double* ui = V + (int64_t)i * n0;
-            if (f->m > 0) {
-                k_edge_quad<<<rbm, ET, 0, s>>>(f->m, f->eu, f->ev, f->ew, ui, part, ctr, sc + 2 * i);
-                count_launch();
-            } else {
-                GR_TRY_CUDA(f, cudaMemsetAsync(sc + 2 * i, 0, sizeof(double), s), "memset");
-            }
-            const double* bu = ui;
-            if (normalized) {
-                k_scale_by<<<blocks(n0), ET, 0, s>>>(n0, ui, f->deg, T);
-                count_launch();
-                bu = T;
-            }
-            k_dot<<<rb, ET, 0, s>>>(n0, ui, bu, part, ctr, sc + 2 * i + 1);
-            count_launch();
-        }
+        const int64_t qbw = ceil_div(n0 > 0 ? n0 : 1, ET / k);
+        k_rayleigh<<<(unsigned)(RB < qbw ? RB : qbw), ET, 0, s>>>(n0, k, f->eptr, f->ev, f->ew,
+                                                                 normalized ? f->deg : nullptr, U_out, part, ctr, sc);
+        count_launch();
         int64_t* hs = host_scratch();
         if (!hs) return set_error(f, GR_ENOMEM, "eigensolve: pinned scratch unavailable");
         double* hq = (double*)hs;  // 64 B: up to 4 pairs at a time
