@@ -54,7 +54,7 @@ struct Workspace {
 
 // Named workspace slots (each owner uses disjoint slots).
 enum WsSlot {
-    WS_SORT_A = 0, WS_SORT_B, WS_SORT_C, WS_SORT_D, WS_SORT_HIST, WS_SCAN,
+    WS_SORT_A = 0, WS_SORT_B, WS_SORT_C, WS_SORT_D, WS_SORT_HIST, WS_SCAN, WS_SCAN_TICKET,
     WS_SMOOTH_BUF, WS_SMOOTH_STATS, WS_SMOOTH_PART,
     WS_AGG_STATE, WS_AGG_LIST, WS_AGG_KEYS, WS_AGG_SMALL,
     WS_COARSE_KEYS, WS_COARSE_VALS, WS_COARSE_TMP,

@@ -68,11 +68,21 @@ int bits_for(uint64_t v) {
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan: reduce tiles -> scan tile sums -> scan tiles with offsets
+// Exclusive scan.  Up to SCAN_ONE entries: one block, tile by tile with a
+// carry.  More: tile sums, which the last block to finish scans, then the
+// tiles with their offsets.  The level loop scans a few dozen times; tile
+// sums, their scan and the tiles in three launches took 9 us even for a
+// thousand entries (each waits for the one before), one block takes 3.6; over
+// the reduction of the 128^3 mesh 148 us of scans became 83.
 // ---------------------------------------------------------------------------
 constexpr int SCAN_THREADS = 512;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int64_t SCAN_ONE = 2 * SCAN_TILE;
+// place of entry i of a tile in shared memory: a gap per thread's SCAN_ITEMS
+// consecutive entries (without it 16 lanes' 8-byte entries shared a bank)
+constexpr int SCAN_PAD_TILE = SCAN_TILE + SCAN_TILE / SCAN_ITEMS;
+__device__ __forceinline__ int scan_at(int i) { return i + i / SCAN_ITEMS; }
 
 template <typename T>
 __device__ T block_exclusive_scan(T x, T* warp_tot, T* block_total) {
@@ -102,9 +112,55 @@ __device__ T block_exclusive_scan(T x, T* warp_tot, T* block_total) {
     return r;
 }
 
+// exclusive scan of one tile of `in` plus `carry` into `out` (out may be in);
+// returns the tile's total
 template <typename T>
-__global__ void k_scan_reduce(const T* __restrict__ in, int64_t count, T* __restrict__ bsum) {
+__device__ T scan_tile(const T* in, T* out, int64_t base, int64_t count, T carry, T* tile, T* warp_tot, T* total) {
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        int64_t idx = base + (int64_t)i * SCAN_THREADS + threadIdx.x;
+        tile[scan_at(i * SCAN_THREADS + threadIdx.x)] = idx < count ? in[idx] : T(0);
+    }
+    __syncthreads();
+    T loc[SCAN_ITEMS];
+    T s = 0;
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        loc[i] = s;
+        s += tile[scan_at(threadIdx.x * SCAN_ITEMS + i)];
+    }
+    T ex = block_exclusive_scan<T>(s, warp_tot, total) + carry;
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) tile[scan_at(threadIdx.x * SCAN_ITEMS + i)] = ex + loc[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        int64_t idx = base + (int64_t)i * SCAN_THREADS + threadIdx.x;
+        if (idx < count) out[idx] = tile[scan_at(i * SCAN_THREADS + threadIdx.x)];
+    }
+    return *total;
+}
+
+// one block, tile by tile
+template <typename T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_one(const T* in, T* out, int64_t count) {
+    __shared__ T tile[SCAN_PAD_TILE];
+    __shared__ T warp_tot[SCAN_THREADS / 32];
+    __shared__ T total;
+    T carry = 0;
+    for (int64_t base = 0; base < count; base += SCAN_TILE) {
+        carry += scan_tile<T>(in, out, base, count, carry, tile, warp_tot, &total);
+        __syncthreads();
+    }
+}
+
+// tile sums; the last block turns them into the tiles' offsets (ticket: zero
+// before and after)
+template <typename T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const T* in, int64_t count, T* bsum, unsigned* ticket) {
     __shared__ T red[SCAN_THREADS / 32];
+    __shared__ T total;
+    __shared__ bool last;
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     T s = 0;
 #pragma unroll
@@ -120,66 +176,49 @@ __global__ void k_scan_reduce(const T* __restrict__ in, int64_t count, T* __rest
         T t = 0;
         for (int w = 0; w < SCAN_THREADS / 32; ++w) t += red[w];
         bsum[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-}
-
-// one block: exclusive scan of nb tile sums in place, chunk by chunk
-template <typename T>
-__global__ void k_scan_bsums(T* __restrict__ bsum, int64_t nb) {
-    __shared__ T warp_tot[SCAN_THREADS / 32];
-    __shared__ T total;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int64_t nb = gridDim.x;
     T carry = 0;
-    for (int64_t base = 0; base < nb; base += SCAN_THREADS) {
-        int64_t idx = base + threadIdx.x;
-        T x = idx < nb ? bsum[idx] : T(0);
-        T ex = block_exclusive_scan<T>(x, warp_tot, &total);
+    for (int64_t b = 0; b < nb; b += SCAN_THREADS) {
+        const int64_t idx = b + threadIdx.x;
+        const T x = idx < nb ? __ldcg(bsum + idx) : T(0);
+        const T ex = block_exclusive_scan<T>(x, red, &total);
         if (idx < nb) bsum[idx] = ex + carry;
         carry += total;
         __syncthreads();
     }
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 template <typename T>
-__global__ void k_scan_apply(const T* __restrict__ in, T* __restrict__ out, int64_t count,
-                             const T* __restrict__ bsum) {
-    __shared__ T tile[SCAN_TILE];
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const T* in, T* out, int64_t count, const T* bsum) {
+    __shared__ T tile[SCAN_PAD_TILE];
     __shared__ T warp_tot[SCAN_THREADS / 32];
     __shared__ T total;
-    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        int64_t idx = base + (int64_t)i * SCAN_THREADS + threadIdx.x;
-        tile[i * SCAN_THREADS + threadIdx.x] = idx < count ? in[idx] : T(0);
-    }
-    __syncthreads();
-    T loc[SCAN_ITEMS];
-    T s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        loc[i] = s;
-        s += tile[threadIdx.x * SCAN_ITEMS + i];
-    }
-    T ex = block_exclusive_scan<T>(s, warp_tot, &total) + bsum[blockIdx.x];
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) tile[threadIdx.x * SCAN_ITEMS + i] = ex + loc[i];
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        int64_t idx = base + (int64_t)i * SCAN_THREADS + threadIdx.x;
-        if (idx < count) out[idx] = tile[i * SCAN_THREADS + threadIdx.x];
-    }
+    scan_tile<T>(in, out, (int64_t)blockIdx.x * SCAN_TILE, count, bsum[blockIdx.x], tile, warp_tot, &total);
 }
 
 template <typename T>
 static cudaError_t scan_exclusive(const T* in, T* out, int64_t count, Workspace& ws,
                                   cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
+    if (count <= SCAN_ONE) {
+        k_scan_one<T><<<1, SCAN_THREADS, 0, s>>>(in, out, count); count_launch();
+        return cudaGetLastError();
+    }
     int64_t nb = ceil_div(count, SCAN_TILE);
-    void* p = nullptr;
+    void *p = nullptr, *pt = nullptr;
     GR_CUDA(ws.get(WS_SCAN, sizeof(T) * (size_t)nb, &p));
+    const bool fresh = (int)ws.slots.size() <= WS_SCAN_TICKET || !ws.slots[WS_SCAN_TICKET].ptr;
+    GR_CUDA(ws.get(WS_SCAN_TICKET, 16, &pt));
+    if (fresh) GR_CUDA(cudaMemsetAsync(pt, 0, 16, s));
     T* bsum = (T*)p;
-    k_scan_reduce<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, count, bsum); count_launch();
-    k_scan_bsums<T><<<1, SCAN_THREADS, 0, s>>>(bsum, nb); count_launch();
+    k_scan_reduce<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, count, bsum, (unsigned*)pt); count_launch();
     k_scan_apply<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, count, bsum); count_launch();
     return cudaGetLastError();
 }
