@@ -416,6 +416,13 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
     constexpr int E = L::E, G = L::G, RB = L::RB;
     constexpr int RPW = 32 / G;
     constexpr bool F64 = sizeof(T) == 8;
+    // Row chunks to lanes.  FP32 and BF16: RPW whole rows a warp.  FP64 rows of
+    // 24 columns (12 chunks) would leave 8 of 32 lanes idle, and the FP64 pipe,
+    // which bounds the sweep, spends their time all the same: there the
+    // chunks go to the consumer threads in line, rows across warps (64^3
+    // mesh, K = 24, eight sweeps: 1,774 -> 1,301 us, with the shorter epilogue below).
+    constexpr bool LINE = F64 && 32 % G != 0;
+    static_assert(!LINE || BAND_CT % G == 0, "a thread keeps its chunk column");
     static_assert(L::CB == 16, "band rows are whole 16-byte chunks");
     extern __shared__ __align__(128) unsigned char bsm[];
     __shared__ __align__(8) uint64_t ld_bar[BAND_NS];
@@ -521,8 +528,8 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
         __syncwarp();
     } else {
         // ------------------------------------------------------------ consumers
-        const int seg = lane / G, q = lane % G;
-        const bool lane_ok = seg < RPW;
+        const int seg = LINE ? 0 : lane / G, q = LINE ? tid % G : lane % G;
+        const bool lane_ok = LINE || seg < RPW;
         const Acc omega = (Acc)a.omega, one_m = (Acc)(1.0 - a.omega);
         const T* Aq = a.Ain + q * E;
         const uint32_t rows_q = sbase + q * 16;
@@ -532,6 +539,16 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
         for (int e = 0; e < E; ++e) {
             mu[e] = st_sh[q * E + e];
             is[e] = st_sh[K + q * E + e];
+        }
+        // FP64: (1-w) x + w acc, centred and scaled, in two multiply-adds
+        Acc ca[E], cb[E], cc[E];
+        if constexpr (F64) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                ca[e] = one_m * is[e];
+                cb[e] = omega * is[e];
+                cc[e] = -mu[e] * is[e];
+            }
         }
         bool ok = true;
         for (int k = 0; ok && k < nb; ++k) {
@@ -549,7 +566,7 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
             // the low words of the row pointers give the local slot range
             const int* rp32 = reinterpret_cast<const int*>(S);
             const int s0lo = (int)M.s0a;
-            for (int lr0 = warp * RPW; lr0 < M.nrows; lr0 += BAND_CW * RPW) {
+            for (int lr0 = LINE ? tid / G : warp * RPW; lr0 < M.nrows; lr0 += LINE ? BAND_CT / G : BAND_CW * RPW) {
                 const int lr = lr0 + seg;
                 if (!lane_ok || lr >= M.nrows) continue;
                 const int r = M.r0 + lr;
@@ -591,8 +608,12 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
                 Acc y[E];
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    Acc z = isolated ? xi[e] : one_m * xi[e] + omega * acc[e];
-                    y[e] = (z - mu[e]) * is[e];
+                    if constexpr (F64) {
+                        y[e] = isolated ? fma(is[e], xi[e], cc[e]) : fma(ca[e], xi[e], fma(cb[e], acc[e], cc[e]));
+                    } else {
+                        Acc z = isolated ? xi[e] : one_m * xi[e] + omega * acc[e];
+                        y[e] = (z - mu[e]) * is[e];
+                    }
                 }
                 store_chunk<T, E>(a.Aout + (size_t)r * K + q * E, y);
 #pragma unroll
@@ -610,30 +631,46 @@ __global__ void __launch_bounds__(band_threads<T, K>(), 1) k_sweep_band(const __
     // rows); warps combined in FP64 in fixed order.  The pipeline's shared
     // memory is idle now and holds the per-warp sums.
     __syncthreads();
-    double* wst = reinterpret_cast<double*>(bsm);  // [BAND_CW][2K]
+    double* wst = reinterpret_cast<double*>(bsm);  // [BAND_CW][2K]; LINE: [2E][BAND_CT]
+    if constexpr (LINE) {
+        if (warp < BAND_CW) {
 #pragma unroll
-    for (int e = 0; e < E; ++e)
-#pragma unroll
-        for (int r = 1; r < RPW; ++r) {
-            const Acc t1 = __shfl_sync(0xffffffffu, s1[e], (lane + r * G) & 31);
-            const Acc t2 = __shfl_sync(0xffffffffu, s2[e], (lane + r * G) & 31);
-            if (lane < G) {
-                s1[e] += t1;
-                s2[e] += t2;
+            for (int e = 0; e < E; ++e) {
+                wst[e * BAND_CT + tid] = s1[e];
+                wst[(E + e) * BAND_CT + tid] = s2[e];
             }
         }
-    if (warp < BAND_CW && lane < G) {
+    } else {
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            wst[warp * 2 * K + lane * E + e] = (double)s1[e];
-            wst[warp * 2 * K + K + lane * E + e] = (double)s2[e];
+        for (int e = 0; e < E; ++e)
+#pragma unroll
+            for (int r = 1; r < RPW; ++r) {
+                const Acc t1 = __shfl_sync(0xffffffffu, s1[e], (lane + r * G) & 31);
+                const Acc t2 = __shfl_sync(0xffffffffu, s2[e], (lane + r * G) & 31);
+                if (lane < G) {
+                    s1[e] += t1;
+                    s2[e] += t2;
+                }
+            }
+        if (warp < BAND_CW && lane < G) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                wst[warp * 2 * K + lane * E + e] = to_f64(s1[e]);
+                wst[warp * 2 * K + K + lane * E + e] = to_f64(s2[e]);
+            }
         }
     }
     __syncthreads();
     if (abort_flag && tid == 0) atomicExch(a.err, 1);
     if (tid < 2 * K) {
-        double t = 0.0;
-        for (int w = 0; w < BAND_CW; ++w) t += wst[w * 2 * K + tid];
+        double t;
+        if constexpr (LINE) {
+            // column tid % K = q E + e: the threads q, q + G, ...
+            const int col = tid % K, q = col / E, e = col % E + (tid < K ? 0 : E);
+            t = sum_warps<BAND_CT / G, G>(wst + e * BAND_CT + q);
+        } else {
+            t = sum_warps<BAND_CW, 2 * K>(wst + tid);
+        }
         // a block that gave up leaves its rows unwritten: NaN partials make the
         // statistics, and so every later output, NaN
         a.part[(int64_t)blockIdx.x * 2 * K + tid] = abort_flag ? __longlong_as_double(0x7ff8000000000000ll) : t;
@@ -690,7 +727,8 @@ static bool band_plan(const gr_ctx* c, bool forced, BandPlan* bp) {
             size_t total = (size_t)off_stage + (size_t)BAND_NS * stage_bytes;
             if (total > (size_t)BAND_SMEM_MAX) continue;
             // the statistics' per-warp sums reuse the pipeline's shared memory
-            if (total < (size_t)BAND_CW * 2 * K * sizeof(double)) total = (size_t)BAND_CW * 2 * K * sizeof(double);
+            // (one set per consumer thread at most)
+            if (total < (size_t)BAND_CW * 64 * RowLayout<T, K>::E * sizeof(double)) total = (size_t)BAND_CW * 64 * RowLayout<T, K>::E * sizeof(double);
             bp->R = R;
             bp->H = H;
             bp->SC = SC;

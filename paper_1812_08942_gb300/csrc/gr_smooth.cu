@@ -42,15 +42,13 @@ __device__ void block_stats(Acc (&s1)[E], Acc (&s2)[E], double* __restrict__ par
     if (lane < G) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            wst[warp][lane * E + e] = (double)s1[e];
-            wst[warp][K + lane * E + e] = (double)s2[e];
+            wst[warp][lane * E + e] = to_f64(s1[e]);
+            wst[warp][K + lane * E + e] = to_f64(s2[e]);
         }
     }
     __syncthreads();
     if (threadIdx.x < 2 * K) {
-        double s = 0.0;
-        for (int w = 0; w < SM_WARPS; ++w) s += wst[w][threadIdx.x];
-        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = s;
+        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = sum_warps<SM_WARPS, 2 * K>(&wst[0][threadIdx.x]);
     }
     __threadfence();
     __syncthreads();
@@ -166,15 +164,13 @@ __device__ void block_stats_chunks(Acc (&s1)[E], Acc (&s2)[E], int q, double* __
     if (lane < G) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            wst[warp][q * E + e] = (double)s1[e];
-            wst[warp][K + q * E + e] = (double)s2[e];
+            wst[warp][q * E + e] = to_f64(s1[e]);
+            wst[warp][K + q * E + e] = to_f64(s2[e]);
         }
     }
     __syncthreads();
     if (threadIdx.x < 2 * K) {
-        double t = 0.0;
-        for (int w = 0; w < SM_WARPS; ++w) t += wst[w][threadIdx.x];
-        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = t;
+        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = sum_warps<SM_WARPS, 2 * K>(&wst[0][threadIdx.x]);
     }
     __threadfence();
     __syncthreads();
@@ -452,15 +448,13 @@ __device__ bool block_sums_rows(Acc (&s1)[E], Acc (&s2)[E], double* __restrict__
     if (lane < G) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            wst[warp][lane * E + e] = (double)s1[e];
-            wst[warp][K + lane * E + e] = (double)s2[e];
+            wst[warp][lane * E + e] = to_f64(s1[e]);
+            wst[warp][K + lane * E + e] = to_f64(s2[e]);
         }
     }
     __syncthreads();
     if (threadIdx.x < 2 * K) {
-        double t = 0.0;
-        for (int w = 0; w < SM_WARPS; ++w) t += wst[w][threadIdx.x];
-        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = t;
+        part[(int64_t)blockIdx.x * 2 * K + threadIdx.x] = sum_warps<SM_WARPS, 2 * K>(&wst[0][threadIdx.x]);
     }
     __threadfence();
     __syncthreads();
@@ -496,6 +490,17 @@ __device__ __forceinline__ void sweep_row_body(
     Acc s1[E], s2[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) s1[e] = s2[e] = Acc(0);
+    // FP64: (1-w) x + w acc, centred and scaled, in two multiply-adds (the
+    // FP64 pipe bounds that sweep; FP32 keeps its rounding)
+    Acc ca[E], cb[E], cc[E];
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            ca[e] = one_m * st_sh[K + q * E + e];
+            cb[e] = omega * st_sh[K + q * E + e];
+            cc[e] = -st_sh[q * E + e] * st_sh[K + q * E + e];
+        }
+    }
     const int stride = ((gridDim.x * blockDim.x) >> 5) * RPW;
     int row = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RPW + (lane_ok ? seg : 0);
     const T* Aq = Ain + q * E;
@@ -552,8 +557,13 @@ __device__ __forceinline__ void sweep_row_body(
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
                     const int k = q * E + e;
-                    Acc z = isolated ? xi[e] : one_m * xi[e] + omega * acc[e];
-                    y[e] = (z - st_sh[k]) * st_sh[K + k];
+                    if constexpr (sizeof(T) == 8) {
+                        y[e] = isolated ? fma(st_sh[K + k], xi[e], cc[e])
+                                        : fma(ca[e], xi[e], fma(cb[e], acc[e], cc[e]));
+                    } else {
+                        Acc z = isolated ? xi[e] : one_m * xi[e] + omega * acc[e];
+                        y[e] = (z - st_sh[k]) * st_sh[K + k];
+                    }
                 }
                 store_chunk<T, E>(Aout + (size_t)row * K + q * E, y);
                 add_sums<Acc, E>(s1, s2, y);
@@ -824,6 +834,10 @@ static cudaError_t launch_sweep_row(gr_ctx* c, const SweepPlan& P, const T* Ain,
                        (size_t)c->n * K * sizeof(T) <= ROW_DENSE_MAX_BYTES;
     int grid = c->num_sms * (dense ? bps4d : (four ? bps4 : bps2));
     if (grid > part_cap) grid = part_cap;
+    // no more blocks than rows ask for: idle blocks' partial sums would be
+    // waited for too (4,096 rows, FP64: 19 us a sweep with a full wave)
+    const int64_t want = ceil_div(c->n > 0 ? c->n : 1, (int64_t)(32 / RowLayout<T, K>::G) * SM_WARPS);
+    if (want < grid) grid = (int)want;
     const typename SlotOf<T>::type* slots;
     if constexpr (sizeof(T) == 8) slots = P.cw64;
     else slots = c->cw32;

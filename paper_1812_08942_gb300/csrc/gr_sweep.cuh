@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gr_vec.cuh"
+
 namespace gr {
 
 // Partials are combined in two levels: blocks form groups of STATS_GROUP
@@ -32,10 +34,32 @@ constexpr int STATS_GCOUNT_OFF = 16;
 // bytes of counter words that follow the statistics sets
 constexpr size_t STATS_COUNTER_BYTES = sizeof(unsigned) * (STATS_GCOUNT_OFF + STATS_MAX_GROUPS);
 
+// A lane's FP32 sum as FP64 (integer operations: the conversion unit is slow)
+__device__ __forceinline__ double to_f64(float x) { return f32_to_f64(x); }
+__device__ __forceinline__ double to_f64(double x) { return x; }
+
+// Sum of NW values STRIDE apart, in pairs: FP64 additions wait 64 cycles for
+// one another on this part, so a chain of eight costs three times the tree.
+template <int NW, int STRIDE>
+__device__ __forceinline__ double sum_warps(const double* v) {
+    if constexpr (NW > 16) {  // by halves, so as not to hold them all
+        constexpr int H = NW / 2;
+        return sum_warps<H, STRIDE>(v) + sum_warps<NW - H, STRIDE>(v + H * STRIDE);
+    }
+    double a[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) a[w] = v[w * STRIDE];
+#pragma unroll
+    for (int o = 1; o < NW; o <<= 1)
+#pragma unroll
+        for (int w = 0; w + o < NW; w += 2 * o) a[w] += a[w + o];
+    return a[0];
+}
+
 // red[s] = sum over r < nrows of base[r * rstride + s], s < 2K, in a fixed
 // order (each of the first PER * 2K threads sums every PER-th row with eight
 // interleaved accumulators, then the PER sums of a column are added in
-// order).  Every thread of the block must call it (block barriers).
+// pairs).  Every thread of the block must call it (block barriers).
 template <int K, int NT>
 __device__ __forceinline__ void sum_partial_rows(const double* base, int nrows, int64_t rstride,
                                                  double* red) {
@@ -59,11 +83,7 @@ __device__ __forceinline__ void sum_partial_rows(const double* base, int nrows, 
     }
     if (t < NT) red[t] = acc;
     __syncthreads();
-    if (t < NS) {
-        double s = 0.0;
-        for (int j = 0; j < PER; ++j) s += red[j * NS + t];
-        red[t] = s;  // row 0 of red is read only by its own thread above
-    }
+    if (t < NS) red[t] = sum_warps<PER, NS>(red + t);  // row 0 of red is read only by its own thread
     __syncthreads();
 }
 
