@@ -465,7 +465,29 @@ __global__ void k_gal_unpack(int64_t R, const unsigned long long* __restrict__ p
     eptr[i] = (int64_t)(p[i] & 0xffffffffull);
 }
 
-// Coarse CSR, row-scaled weights and canonical edge list from the rows.
+// D(A, A) of short rows, a thread per row: the weights in slot order
+// (= ascending edge id), the plain definition's order.  Four loads in flight.
+__global__ void __launch_bounds__(GT) k_gal_degree(int64_t nc, const RowMeta* __restrict__ meta,
+                                                   const double* __restrict__ uw, double* __restrict__ deg) {
+    const int64_t A = (int64_t)blockIdx.x * GT + threadIdx.x;
+    if (A >= nc) return;
+    const int4 m = __ldg(reinterpret_cast<const int4*>(meta) + A);
+    const double* w = uw + (uint32_t)m.x;
+    double s = 0.0;
+    for (int32_t i = 0; i < m.y; i += 4) {
+        double x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u < m.y) x[u] = __ldg(w + i + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u < m.y) s += x[u];
+    }
+    deg[A] = s;
+}
+
+// Coarse CSR, row-scaled weights and canonical edge list from the rows; long
+// rows (G = 32) also their degrees.
 // Lower entries (B < A) take the id of edge (B, A): A's position among B's
 // upper entries.
 template <int G>
@@ -481,13 +503,15 @@ __global__ void k_gal_fill(int64_t nc, const RowMeta* __restrict__ meta, const i
     const uint32_t base = (uint32_t)mA.x;
     const int32_t U = mA.y, low = U - mA.z;
     const int64_t r0 = rowptr[A], e0 = eptr[A];
-    // D(A, A): lane sums in slot order, combined by a fixed butterfly
     double dA = 0.0;
-    for (int32_t i = l; i < U; i += G) dA += uw[base + i];
-    const unsigned mask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << ((threadIdx.x & 31) / G * G);
+    if constexpr (G == 32) {  // lane sums in slot order, combined by a fixed butterfly
+        for (int32_t i = l; i < U; i += G) dA += uw[base + i];
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) dA += __shfl_xor_sync(mask, dA, o, G);
-    if (l == 0) deg[A] = dA;
+        for (int o = 16; o > 0; o >>= 1) dA += __shfl_xor_sync(0xffffffffu, dA, o);
+        if (l == 0) deg[A] = dA;
+    } else {
+        dA = deg[A];
+    }
     const double inv = dA > 0.0 ? 1.0 / dA : 0.0;
     for (int32_t i = l; i < U; i += G) {
         const int32_t B = ucol[base + i];
@@ -624,17 +648,18 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
     GR_TRY_CUDA(c, cudaMallocAsync(&cc->eid, sizeof(int32_t) * cs, s), "alloc");
     GR_TRY_CUDA(c, cudaMallocAsync(&cc->cw32, sizeof(int2) * cs, s), "alloc");
     GR_TRY_CUDA(c, cudaMallocAsync(&cc->wn64, sizeof(double) * cs, s), "alloc");
-    if (mc > 0) {
-        const int G = 2 * mc >= 32 * nc ? 32 : 4;
-        const unsigned grid = (unsigned)ceil_div(nc * G, GT);
-        if (G == 32)
-            k_gal_fill<32><<<grid, GT, 0, s>>>(nc, meta, ucol, uw, cc->deg, cc->rowptr, cc->eptr, cc->col, cc->eid,
-                                               cc->wn64, cc->cw32, cc->eu, cc->ev, cc->ew);
-        else
-            k_gal_fill<4><<<grid, GT, 0, s>>>(nc, meta, ucol, uw, cc->deg, cc->rowptr, cc->eptr, cc->col, cc->eid,
-                                              cc->wn64, cc->cw32, cc->eu, cc->ev, cc->ew);
+    const int G = 2 * mc >= 32 * nc ? 32 : 4;
+    const unsigned grid = (unsigned)ceil_div(nc * G, GT);
+    if (G == 32) {
+        k_gal_fill<32><<<grid, GT, 0, s>>>(nc, meta, ucol, uw, cc->deg, cc->rowptr, cc->eptr, cc->col, cc->eid,
+                                           cc->wn64, cc->cw32, cc->eu, cc->ev, cc->ew);
+    } else {
+        k_gal_degree<<<(unsigned)ceil_div(nc, GT), GT, 0, s>>>(nc, meta, uw, cc->deg);
         count_launch();
+        k_gal_fill<4><<<grid, GT, 0, s>>>(nc, meta, ucol, uw, cc->deg, cc->rowptr, cc->eptr, cc->col, cc->eid,
+                                          cc->wn64, cc->cw32, cc->eu, cc->ev, cc->ew);
     }
+    count_launch();
     GR_TRY_CUDA(c, cudaGetLastError(), "galerkin fill");
     return GR_OK;
 }
