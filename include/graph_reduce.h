@@ -130,7 +130,9 @@ gr_status graph_reduce_smooth_noalloc(gr_ctx* ctx, int K, int sweeps, double ome
  * slot order, so they agree within the rounding of the column statistics.
  *   GR_SWEEP_AUTO    (default) the streaming kernel when rows are long (a
  *                    warp's group of 32 / lanes-per-row rows would hold over
- *                    128 slots); else the band kernel when the graph has at
+ *                    128 slots; FP64 and BF16 blocks of a created graph
+ *                    whose rows hold at most 64 slots below and above the
+ *                    diagonal are excepted); else the band kernel when the graph has at
  *                    least 640 rows per SM (enough for a chunk of bands on
  *                    every SM) and is in a banded order: at least half of
  *                    its slots within a halo of at most 1,024 rows that fits

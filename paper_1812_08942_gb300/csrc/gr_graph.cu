@@ -166,16 +166,19 @@ constexpr int LOWER_WARP = 2048;   // up to this long: by a warp in shared memor
 constexpr int FW = 4;              // warps per block of the warp kernel
 
 // per edge: canonical-input check (when asked) and the lower count of v;
-// the block maximum of the counts reached goes to lmax
+// the block maximum of the counts reached goes to lmax; long_up is raised by
+// an upper part past ROW_PART_SHORT edges (u is sorted)
 __global__ void k_csr_count(int64_t n, int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
                             const double* __restrict__ w, int check, int32_t* __restrict__ lcnt,
-                            int32_t* __restrict__ bad, int32_t* __restrict__ lmax) {
+                            int32_t* __restrict__ bad, int32_t* __restrict__ lmax,
+                            int32_t* __restrict__ long_up) {
     __shared__ int32_t bmax;
     if (threadIdx.x == 0) bmax = 0;
     __syncthreads();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e < m) {
         const int32_t a = u[e], b = v[e];
+        if (e >= ROW_PART_SHORT && u[e - ROW_PART_SHORT] == a) *long_up = 1;
         if (check) {
             bool ok = a >= 0 && b < n && a < b && w[e] > 0.0 && isfinite(w[e]);
             if (e > 0) {
@@ -446,14 +449,14 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
     int32_t* lcnt = (int32_t*)p_i32;
     int32_t* lfill = lcnt + R;
     int32_t* list = lfill + R;
-    int32_t* flags = list + R;  // [0] not canonical, [1] longest lower part, [2] listed rows
+    int32_t* flags = list + R;  // [0] not canonical, [1] longest lower part, [2] listed rows, [3] long upper part
     int64_t* rowcnt = (int64_t*)p_i64;
 
     GR_TRY_CUDA(c, cudaMemsetAsync(lcnt, 0, sizeof(int32_t) * (2 * R), s), "memset");
     GR_TRY_CUDA(c, cudaMemsetAsync(flags, 0, 16, s), "memset");
     if (m > 0) {
         k_csr_count<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(n, m, c->eu, c->ev, c->ew, check ? 1 : 0, lcnt, flags,
-                                                            flags + 1);
+                                                            flags + 1, flags + 3);
         count_launch();
     }
     // dense graphs (mean degree 32 or more): the global sort of the lower
@@ -469,6 +472,7 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
             return set_error(c, GR_EINVAL, "csr: the edge list is not canonical");
         }
         lmax = hf[1];
+        c->short_rows = hf[1] <= ROW_PART_SHORT && !hf[3];
     }
     k_upper_ptr<<<(unsigned)ceil_div(m + 1, TB), TB, 0, s>>>(c->eu, m, n, c->eptr); count_launch();
     if (!sparse || lmax > LOWER_WARP) return build_csr_sorted(c, lcnt, rowcnt);

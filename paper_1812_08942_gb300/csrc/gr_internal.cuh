@@ -30,6 +30,9 @@ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 constexpr int64_t CSR_PAD_ROWS = 1;
 constexpr size_t CSR_PAD_SLOTS = 4;
 
+// longest lower and upper part of a row up to which gr_ctx::short_rows holds
+constexpr int ROW_PART_SHORT = 64;
+
 // Shape of the band sweep on one graph (gr_band.cu)
 struct BandPlan {
     int R = 0, H = 0;       // rows per band, halo rows on each side of a band
@@ -89,6 +92,7 @@ struct gr_ctx {
     int32_t* wpart = nullptr;
     int64_t wpart_W = 0;
     int4* cw64 = nullptr;       // 2m: (col, 0, w / deg_row as FP64), built on first FP64 sweep
+    bool short_rows = false;    // no row has more than ROW_PART_SHORT slots on either side of the diagonal (false: not known)
     // sweep kernel selection (gr_sweep_kernel)
     int sweep_kind = GR_SWEEP_AUTO;
     // locality profile for the band sweep: slots with |col - row| in

@@ -648,11 +648,18 @@ struct SweepScratch {
 };
 
 // Streaming sweep when a group of 32 / GP rows would hold more slots than
-// four ring batches (long rows).
+// four ring batches (long rows).  FP64 and BF16 blocks of graphs known to have
+// short rows keep the row-group kernel: streaming serves them for its balance
+// over hubs, and without hubs a warp per row of a dozen slots is half idle
+// (neighbour graph of 200,000 nodes, mean degree 11.6, BF16, K = 16: 37 us a
+// sweep against 75; FP64, K = 8, mean degree 17: 105 against 338; with hubs,
+// mean degree 20, BF16, K = 16: 256 against 107).  FP32 blocks keep the rule,
+// and with it the rounding of their column sums.
 template <typename T, int K>
 static bool stream_wide(const gr_ctx* c) {
     constexpr int GP = RowLayout<T, K>::GP;
     const double avg = c->n > 0 ? 2.0 * (double)c->m / (double)c->n : 0.0;
+    if (sizeof(T) != 4 && c->short_rows) return false;
     return GP < 32 && (32.0 / GP) * avg > 128.0;
 }
 
