@@ -3,6 +3,7 @@
 // memory (gr_galerkin.cu), or by a global sort + segmented sum when a coarse
 // row is too long for that.
 #include "gr_internal.cuh"
+#include "gr_vec.cuh"
 
 namespace gr {
 
@@ -11,27 +12,47 @@ constexpr int TB = 256;
 // ---------------------------------------------------------------------------
 // CSR construction from a canonical edge list
 // ---------------------------------------------------------------------------
+constexpr int PT = 4;  // list positions a thread of the per-edge kernels takes, their loads in flight together
+
 // eptr[p] = first edge with u >= p (u is sorted), for p in [0, n]
-__global__ void k_upper_ptr(const int32_t* __restrict__ eu, int64_t m, int64_t n,
-                            int64_t* __restrict__ eptr) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e > m) return;
-    int64_t prev = e == 0 ? -1 : (int64_t)eu[e - 1];
-    int64_t cur = e == m ? n : (int64_t)eu[e];
-    for (int64_t p = prev + 1; p <= cur; ++p) eptr[p] = e;
+__global__ void __launch_bounds__(TB) k_upper_ptr(const int32_t* __restrict__ eu, int64_t m, int64_t n,
+                                                  int64_t* __restrict__ eptr) {
+    const int64_t t0 = (int64_t)blockIdx.x * (TB * PT) + threadIdx.x;
+    int64_t prev[PT], cur[PT];
+#pragma unroll
+    for (int i = 0; i < PT; ++i) {
+        const int64_t e = t0 + i * TB;
+        prev[i] = e == 0 || e > m ? -1 : (int64_t)__ldg(eu + e - 1);
+        cur[i] = e == m ? n : e > m ? -1 : (int64_t)__ldg(eu + e);
+    }
+#pragma unroll
+    for (int i = 0; i < PT; ++i)
+        for (int64_t p = prev[i] + 1; p <= cur[i]; ++p) eptr[p] = t0 + i * TB;
 }
 
-// rowcnt[p] = lower count + upper count (entry n is 0); lc64 = lower count as int64
-__global__ void k_row_count(const int32_t* __restrict__ lcnt, const int64_t* __restrict__ eptr,
-                            int64_t n, int64_t* __restrict__ rowcnt, int64_t* __restrict__ lc64) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) {
-        rowcnt[p] = (int64_t)lcnt[p] + (eptr[p + 1] - eptr[p]);
-        lc64[p] = lcnt[p];
-    } else if (p == n) {
-        rowcnt[p] = 0;
-        lc64[p] = 0;
+// The lower parts from the edges sorted by v: lstart[p] = first position with
+// v >= p, for p in [0, n], and with the upper parts before it the row's start.
+// long_low (may be null) is raised by a lower part past ROW_PART_SHORT edges.
+__global__ void __launch_bounds__(TB) k_lower_ptr(const uint32_t* __restrict__ skey, int64_t m, int64_t n,
+                                                  const int64_t* __restrict__ eptr, int64_t* __restrict__ lstart,
+                                                  int64_t* __restrict__ rowptr, int32_t* __restrict__ long_low) {
+    const int64_t t0 = (int64_t)blockIdx.x * (TB * PT) + threadIdx.x;
+    int64_t prev[PT], cur[PT];
+    bool far = false;
+#pragma unroll
+    for (int i = 0; i < PT; ++i) {
+        const int64_t t = t0 + i * TB;
+        prev[i] = t == 0 || t > m ? -1 : (int64_t)__ldg(skey + t - 1);
+        cur[i] = t == m ? n : t > m ? -1 : (int64_t)__ldg(skey + t);
+        if (long_low && t >= ROW_PART_SHORT && t < m) far |= (int64_t)__ldg(skey + t - ROW_PART_SHORT) == cur[i];
     }
+#pragma unroll
+    for (int i = 0; i < PT; ++i)
+        for (int64_t p = prev[i] + 1; p <= cur[i]; ++p) {
+            lstart[p] = t0 + i * TB;
+            rowptr[p] = t0 + i * TB + eptr[p];
+        }
+    if (far) *long_low = 1;
 }
 
 __global__ void k_keys_from_v(const int32_t* __restrict__ ev, int64_t m, uint32_t* __restrict__ keys,
@@ -63,37 +84,182 @@ __global__ void k_fill_lower(const uint32_t* __restrict__ skey, const uint32_t* 
 // upper part of row p: edges (p, v), v > p, after the lower part
 __global__ void k_fill_upper(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                              const double* __restrict__ ew, int64_t m,
-                             const int64_t* __restrict__ eptr, const int32_t* __restrict__ lcnt,
-                             const int64_t* __restrict__ rowptr, int32_t* __restrict__ col,
-                             int32_t* __restrict__ eid, double* __restrict__ wslot) {
+                             const int64_t* __restrict__ eptr, const int64_t* __restrict__ rowptr,
+                             int32_t* __restrict__ col, int32_t* __restrict__ eid,
+                             double* __restrict__ wslot) {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m) return;
     int64_t p = eu[e];
-    int64_t slot = rowptr[p] + lcnt[p] + (e - eptr[p]);
+    int64_t slot = rowptr[p + 1] - (eptr[p + 1] - e);
     col[slot] = ev[e];
     eid[slot] = (int32_t)e;
     wslot[slot] = ew[e];
 }
 
-// warp per row: D(p,p) = sum of the row's weights (fixed shuffle-tree order),
-// then the row-scaled weights w / D(p,p) that D^-1 A uses.
-__global__ void k_degree_scale(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                               int64_t n, double* __restrict__ wn64, int2* __restrict__ cw32,
-                               double* __restrict__ deg) {
-    const int lane = threadIdx.x & 31;
-    int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (p >= n) return;
-    int64_t b = rowptr[p], e = rowptr[p + 1];
-    double s = 0.0;
-    for (int64_t j = b + lane; j < e; j += 32) s += wn64[j];
+// Warp per row of a dense graph, from the lower edge ids sorted by v: the
+// slots, D(p,p) = the lanes' sums in slot order combined by a fixed tree, and
+// the row-scaled weights w / D(p,p) that D^-1 A uses, in one pass.  A row of
+// up to 128 slots stays in registers; a longer one keeps its weights in the
+// slot array between its two passes.  Four slots in flight a lane (eight leave
+// four blocks an SM: 427 us against 373 below).
+// Bound by the waits for the two dependent gathers and by the FP64 pipe, which
+// takes an instruction of one lane as long as one of 32: the tree and the
+// division of eight rows are one warp's, a lane per pair and per row (a
+// shuffle tree and a division in every warp: 607 us).  434,000 rows, 32 M
+// slots: 966 us with separate fills of the two parts and a scaling pass, 373
+// now; 13,000 rows, 26 M slots: 446 and 315.
+constexpr int FIN_ROWS = TB / 32;
+constexpr int FIN_FLIGHT = 4;  // slots in flight a lane
+
+struct FinRow {
+    int64_t r0, l0, e0;
+    int low, len;
+};
+
+struct FinArrays {
+    const uint32_t* sval;
+    const int32_t *eu, *ev;
+    const double* ew;
+    int32_t *col, *eid;
+    double* wn64;
+    int2* cw32;
+};
+
+// sum of a row's lane sums, for the block's rows: every thread calls it
+__device__ __forceinline__ double fin_inverse(double s, double* __restrict__ deg, int64_t n) {
+    __shared__ double part[FIN_ROWS][32];
+    __shared__ double inv[FIN_ROWS];
+    static_assert(FIN_ROWS == 8, "the tree's first step is four pairs a lane");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) deg[p] = s;
-    double inv = s > 0.0 ? 1.0 / s : 0.0;
-    for (int64_t j = b + lane; j < e; j += 32) {
-        double x = wn64[j] * inv;
-        wn64[j] = x;
-        cw32[j] = make_int2(col[j], __float_as_int((float)x));
+        for (int o = 16; o > 0; o >>= 1) {  // lane l of a row takes l + o
+            double x[4];
+#pragma unroll
+            for (int i = 0; i < (o + 3) / 4; ++i) {
+                const int j = lane + 32 * i;
+                if (j < FIN_ROWS * o) x[i] = part[j / o][j % o] + part[j / o][j % o + o];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < (o + 3) / 4; ++i) {
+                const int j = lane + 32 * i;
+                if (j < FIN_ROWS * o) part[j / o][j % o] = x[i];
+            }
+            __syncwarp();
+        }
+        const int64_t p = (int64_t)blockIdx.x * FIN_ROWS + lane;
+        if (lane < FIN_ROWS) {
+            const double d = part[lane][0];
+            if (p < n) deg[p] = d;
+            inv[lane] = d > 0.0 ? 1.0 / d : 0.0;
+        }
+    }
+    __syncthreads();
+    return inv[warp];
+}
+
+template <int U, int N>
+__device__ __forceinline__ double fin_load(const FinArrays& A, const FinRow& R, int b, int32_t (&e)[N],
+                                           int32_t (&q)[N], double (&w)[N], double s) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int i = b + 32 * u;
+        if (i < R.len) e[u] = i < R.low ? (int32_t)__ldg(A.sval + R.l0 + i) : (int32_t)(R.e0 + (i - R.low));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (b + 32 * u < R.len) {
+            q[u] = __ldg((b + 32 * u < R.low ? A.eu : A.ev) + e[u]);
+            w[u] = __ldg(A.ew + e[u]);
+        }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (b + 32 * u < R.len) s += w[u];
+    return s;
+}
+
+template <int U, int N>
+__device__ __forceinline__ void fin_store(const FinArrays& A, const FinRow& R, int b, const int32_t (&e)[N],
+                                          const int32_t (&q)[N], const double (&w)[N], double inv) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (b + 32 * u < R.len) {
+            const int64_t j = R.r0 + b + 32 * u;
+            const double x = w[u] * inv;
+            A.col[j] = q[u];
+            A.eid[j] = e[u];
+            A.wn64[j] = x;
+            A.cw32[j] = make_int2(q[u], __float_as_int(f64_to_f32(x)));
+        }
+}
+
+__global__ void __launch_bounds__(TB, 5) k_row_finish_sorted(int64_t n, const int64_t* __restrict__ rowptr,
+                                                          const int64_t* __restrict__ lstart,
+                                                          const int64_t* __restrict__ eptr, FinArrays A,
+                                                          double* __restrict__ deg) {
+    const int lane = threadIdx.x & 31;
+    const int64_t p = (int64_t)blockIdx.x * FIN_ROWS + (threadIdx.x >> 5);
+    FinRow R{0, 0, 0, 0, 0};
+    if (p < n) {
+        R.r0 = rowptr[p];
+        R.l0 = lstart[p];
+        R.e0 = eptr[p];
+        R.low = (int)(lstart[p + 1] - R.l0);
+        R.len = (int)(rowptr[p + 1] - R.r0);
+    }
+    int32_t e[FIN_FLIGHT], q[FIN_FLIGHT];
+    double w[FIN_FLIGHT], s = 0.0;
+    const bool kept = R.len <= 32 * FIN_FLIGHT;
+    // by length, for an FP64 instruction whose lanes are all past the end
+    // takes the pipe like any other
+    if (R.len <= 32) {
+        s = fin_load<1>(A, R, lane, e, q, w, s);
+    } else if (R.len <= 64) {
+        s = fin_load<2>(A, R, lane, e, q, w, s);
+    } else if (kept) {
+        s = fin_load<4>(A, R, lane, e, q, w, s);
+    } else {
+        for (int b = lane; b < R.len; b += 32 * FIN_FLIGHT) {
+            int32_t ee[FIN_FLIGHT], qq[FIN_FLIGHT];
+            double ww[FIN_FLIGHT];
+            s = fin_load<FIN_FLIGHT>(A, R, b, ee, qq, ww, s);
+#pragma unroll
+            for (int u = 0; u < FIN_FLIGHT; ++u)
+                if (b + 32 * u < R.len) {
+                    const int64_t j = R.r0 + b + 32 * u;
+                    A.col[j] = qq[u];
+                    A.eid[j] = ee[u];
+                    A.wn64[j] = ww[u];
+                }
+        }
+    }
+    const double inv = fin_inverse(s, deg, n);
+    if (kept) {
+        if (R.len <= 32) fin_store<1>(A, R, lane, e, q, w, inv);
+        else if (R.len <= 64) fin_store<2>(A, R, lane, e, q, w, inv);
+        else fin_store<4>(A, R, lane, e, q, w, inv);
+        return;
+    }
+    // a lane reads back what it wrote itself
+    for (int b = lane; b < R.len; b += 32 * FIN_FLIGHT) {
+        int32_t qq[FIN_FLIGHT];
+        double ww[FIN_FLIGHT];
+#pragma unroll
+        for (int u = 0; u < FIN_FLIGHT; ++u)
+            if (b + 32 * u < R.len) {
+                ww[u] = A.wn64[R.r0 + b + 32 * u];
+                qq[u] = A.col[R.r0 + b + 32 * u];
+            }
+#pragma unroll
+        for (int u = 0; u < FIN_FLIGHT; ++u)
+            if (b + 32 * u < R.len) {
+                const double x = ww[u] * inv;
+                A.wn64[R.r0 + b + 32 * u] = x;
+                A.cw32[R.r0 + b + 32 * u] = make_int2(qq[u], __float_as_int(f64_to_f32(x)));
+            }
     }
 }
 
@@ -165,30 +331,54 @@ constexpr int LOWER_THREAD = 32;   // lower parts up to this long: sorted by the
 constexpr int LOWER_WARP = 2048;   // up to this long: by a warp in shared memory; longer: global sort
 constexpr int FW = 4;              // warps per block of the warp kernel
 
-// per edge: canonical-input check (when asked) and the lower count of v;
-// the block maximum of the counts reached goes to lmax; long_up is raised by
-// an upper part past ROW_PART_SHORT edges (u is sorted)
-__global__ void k_csr_count(int64_t n, int64_t m, const int32_t* __restrict__ u, const int32_t* __restrict__ v,
-                            const double* __restrict__ w, int check, int32_t* __restrict__ lcnt,
-                            int32_t* __restrict__ bad, int32_t* __restrict__ lmax,
-                            int32_t* __restrict__ long_up) {
+// per edge: canonical-input check (when asked) and, unless lcnt is null, the
+// lower count of v; the block maximum of the counts reached goes to lmax;
+// long_up is raised by an upper part past ROW_PART_SHORT edges (u is sorted)
+__global__ void __launch_bounds__(TB) k_csr_count(int64_t n, int64_t m, const int32_t* __restrict__ u,
+                                                  const int32_t* __restrict__ v, const double* __restrict__ w,
+                                                  int check, int32_t* __restrict__ lcnt, int32_t* __restrict__ bad,
+                                                  int32_t* __restrict__ lmax, int32_t* __restrict__ long_up) {
     __shared__ int32_t bmax;
     if (threadIdx.x == 0) bmax = 0;
     __syncthreads();
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < m) {
-        const int32_t a = u[e], b = v[e];
-        if (e >= ROW_PART_SHORT && u[e - ROW_PART_SHORT] == a) *long_up = 1;
-        if (check) {
-            bool ok = a >= 0 && b < n && a < b && w[e] > 0.0 && isfinite(w[e]);
-            if (e > 0) {
-                const int32_t pa = u[e - 1], pb = v[e - 1];
-                ok = ok && (pa < a || (pa == a && pb < b));
-            }
-            if (!ok) atomicExch(bad, 1);
-        }
-        if (b >= 0 && b < n) atomicMax(&bmax, atomicAdd(&lcnt[b], 1) + 1);
+    const int64_t t0 = (int64_t)blockIdx.x * (TB * PT) + threadIdx.x;
+    int32_t a[PT], b[PT], reached = 0;
+    bool far = false, wrong = false;
+#pragma unroll
+    for (int i = 0; i < PT; ++i) {
+        const int64_t e = t0 + i * TB;
+        a[i] = e < m ? __ldg(u + e) : -1;
+        b[i] = e < m ? __ldg(v + e) : -1;
+        if (e < m && e >= ROW_PART_SHORT) far |= __ldg(u + e - ROW_PART_SHORT) == a[i];
     }
+    if (check) {
+        // positive and finite, on the weight's bits: FP64 compares would take
+        // the FP64 pipe longer than the loads take
+        int64_t wb[PT];
+        int32_t pa[PT], pb[PT];
+#pragma unroll
+        for (int i = 0; i < PT; ++i) {
+            const int64_t e = t0 + i * TB;
+            wb[i] = e < m ? __ldg(reinterpret_cast<const long long*>(w) + e) : 1;
+            pa[i] = e > 0 && e < m ? __ldg(u + e - 1) : -1;
+            pb[i] = e > 0 && e < m ? __ldg(v + e - 1) : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < PT; ++i) {
+            const bool ok = a[i] >= 0 && b[i] < n && a[i] < b[i] && wb[i] > 0 && wb[i] < 0x7ff0000000000000ll &&
+                            (t0 + i * TB == 0 || pa[i] < a[i] || (pa[i] == a[i] && pb[i] < b[i]));
+            if (t0 + i * TB < m && !ok) wrong = true;
+        }
+    }
+    if (lcnt) {
+#pragma unroll
+        for (int i = 0; i < PT; ++i)
+            if (b[i] >= 0 && b[i] < n) reached = max(reached, atomicAdd(&lcnt[b[i]], 1) + 1);
+        reached = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)reached);
+        if ((threadIdx.x & 31) == 0 && reached) atomicMax(&bmax, reached);
+    }
+    if (far) *long_up = 1;
+    if (wrong) atomicExch(bad, 1);
     __syncthreads();
     if (threadIdx.x == 0 && bmax) atomicMax(lmax, bmax);
 }
@@ -441,27 +631,26 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
     GR_TRY_CUDA(c, cudaMallocAsync(&c->cw32, sizeof(int2) * slots, s), "alloc cw32");
     GR_TRY_CUDA(c, cudaMallocAsync(&c->wn64, sizeof(double) * slots, s), "alloc wn64");
 
-    // lcnt (n+1), lfill (n+1), list (n+1), flags (16 B); rowcnt (n+1, int64)
+    // lcnt (n+1), lfill (n+1), list (n+1), flags (16 B)
     void *p_i32, *p_i64;
     const size_t R = (size_t)(n + 1);
     GR_TRY_CUDA(c, c->ws.get(WS_COARSE_TMP, sizeof(int32_t) * (3 * R + 4), &p_i32), "ws");
-    GR_TRY_CUDA(c, c->ws.get(WS_SORT_C, sizeof(int64_t) * R * 3, &p_i64), "ws");
+    GR_TRY_CUDA(c, c->ws.get(WS_SORT_C, sizeof(int64_t) * R, &p_i64), "ws");
     int32_t* lcnt = (int32_t*)p_i32;
     int32_t* lfill = lcnt + R;
     int32_t* list = lfill + R;
-    int32_t* flags = list + R;  // [0] not canonical, [1] longest lower part, [2] listed rows, [3] long upper part
-    int64_t* rowcnt = (int64_t*)p_i64;
-
-    GR_TRY_CUDA(c, cudaMemsetAsync(lcnt, 0, sizeof(int32_t) * (2 * R), s), "memset");
+    int32_t* flags = list + R;  // [0] not canonical, [1] longest lower part, [2] listed rows, [3] long part
+    // dense graphs (mean degree 32 or more): the global sort of the lower
+    // parts beats per-row sorting of long lower parts, and gives their counts:
+    // counting by atomics took 200 to 280 us a level of 13 to 16 M edges
+    const bool sparse = 2 * m < 32 * n;
+    if (sparse) GR_TRY_CUDA(c, cudaMemsetAsync(lcnt, 0, sizeof(int32_t) * (2 * R), s), "memset");
     GR_TRY_CUDA(c, cudaMemsetAsync(flags, 0, 16, s), "memset");
-    if (m > 0) {
-        k_csr_count<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(n, m, c->eu, c->ev, c->ew, check ? 1 : 0, lcnt, flags,
-                                                            flags + 1, flags + 3);
+    if (m > 0 && (check || sparse)) {
+        k_csr_count<<<(unsigned)ceil_div(m, TB * PT), TB, 0, s>>>(n, m, c->eu, c->ev, c->ew, check ? 1 : 0,
+                                                            sparse ? lcnt : nullptr, flags, flags + 1, flags + 3);
         count_launch();
     }
-    // dense graphs (mean degree 32 or more): the global sort of the lower
-    // parts beats per-row sorting of long lower parts
-    const bool sparse = 2 * m < 32 * n;
     int32_t lmax = 0;
     if (check || sparse) {
         GR_TRY_CUDA(c, cudaMemcpyAsync(hs, flags, 16, cudaMemcpyDeviceToHost, s), "readback");
@@ -472,10 +661,18 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
             return set_error(c, GR_EINVAL, "csr: the edge list is not canonical");
         }
         lmax = hf[1];
-        c->short_rows = hf[1] <= ROW_PART_SHORT && !hf[3];
+        c->short_rows = sparse && lmax <= ROW_PART_SHORT && !hf[3];
     }
-    k_upper_ptr<<<(unsigned)ceil_div(m + 1, TB), TB, 0, s>>>(c->eu, m, n, c->eptr); count_launch();
-    if (!sparse || lmax > LOWER_WARP) return build_csr_sorted(c, lcnt, rowcnt);
+    k_upper_ptr<<<(unsigned)ceil_div(m + 1, TB * PT), TB, 0, s>>>(c->eu, m, n, c->eptr); count_launch();
+    if (!sparse || lmax > LOWER_WARP) {
+        const gr_status st = build_csr_sorted(c, check && !sparse ? flags + 3 : nullptr);
+        if (st != GR_OK || sparse || !check) return st;
+        GR_TRY_CUDA(c, cudaMemcpyAsync(hs, flags, 16, cudaMemcpyDeviceToHost, s), "readback");
+        GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
+        c->short_rows = !((const int32_t*)hs)[3];
+        return GR_OK;
+    }
+    int64_t* rowcnt = (int64_t*)p_i64;
     k_row_total<<<(unsigned)ceil_div(n + 1, TB), TB, 0, s>>>(lcnt, c->eptr, n, rowcnt); count_launch();
     GR_TRY_CUDA(c, scan_exclusive_i64(rowcnt, c->rowptr, n + 1, c->ws, s), "scan rowptr");
     if (m > 0) {
@@ -498,53 +695,46 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
     return GR_OK;
 }
 
-// Rows with a lower part too long for one warp's shared memory: a stable
-// radix sort of the edge ids by v lists every row's lower part in order.
-gr_status build_csr_sorted(gr_ctx* c, const int32_t* lcnt, int64_t* rowcnt) {
+// Dense graphs, and rows with a lower part too long for one warp's shared
+// memory: a stable radix sort of the edge ids by v lists every row's lower
+// part in order.
+gr_status build_csr_sorted(gr_ctx* c, int32_t* long_low) {
     const int64_t n = c->n, m = c->m;
     cudaStream_t s = c->stream;
-    int64_t* lc64 = rowcnt + (n + 1);
-    int64_t* lstart = lc64 + (n + 1);
-    k_row_count<<<(unsigned)ceil_div(n + 1, TB), TB, 0, s>>>(lcnt, c->eptr, n, rowcnt, lc64); count_launch();
-    GR_TRY_CUDA(c, scan_exclusive_i64(rowcnt, c->rowptr, n + 1, c->ws, s), "scan rowptr");
-    GR_TRY_CUDA(c, scan_exclusive_i64(lc64, lstart, n + 1, c->ws, s), "scan lstart");
+    void *p_start, *p_k0, *p_v0, *p_alt;
+    const size_t M = (size_t)(m > 0 ? m : 1);
+    GR_TRY_CUDA(c, c->ws.get(WS_SORT_C, sizeof(int64_t) * (size_t)(n + 1), &p_start), "ws");
+    GR_TRY_CUDA(c, c->ws.get(WS_SORT_A, sizeof(uint32_t) * M, &p_k0), "ws");
+    GR_TRY_CUDA(c, c->ws.get(WS_SORT_B, sizeof(uint32_t) * M, &p_v0), "ws");
+    GR_TRY_CUDA(c, c->ws.get(WS_SORT_D, sizeof(uint32_t) * M * 2, &p_alt), "ws");
+    int64_t* lstart = (int64_t*)p_start;
+    uint32_t *k0 = (uint32_t*)p_k0, *v0 = (uint32_t*)p_v0;
+    uint32_t *k1 = (uint32_t*)p_alt, *v1 = k1 + M;
+    int alt = 0;
     if (m > 0) {
-        void *p_k0, *p_v0, *p_alt;
-        GR_TRY_CUDA(c, c->ws.get(WS_SORT_A, sizeof(uint32_t) * (size_t)m, &p_k0), "ws");
-        GR_TRY_CUDA(c, c->ws.get(WS_SORT_B, sizeof(uint32_t) * (size_t)m, &p_v0), "ws");
-        GR_TRY_CUDA(c, c->ws.get(WS_SORT_D, sizeof(uint32_t) * (size_t)m * 2, &p_alt), "ws");
-        uint32_t* k0 = (uint32_t*)p_k0;
-        uint32_t* v0 = (uint32_t*)p_v0;
-        uint32_t* k1 = (uint32_t*)p_alt;
-        uint32_t* v1 = k1 + m;
         k_keys_from_v<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(c->ev, m, k0, v0); count_launch();
-        int alt = 0;
         GR_TRY_CUDA(c, radix_sort_u32(k0, v0, k1, v1, m, bits_for((uint64_t)(n - 1)), c->ws, s, &alt),
                     "sort by v");
-        const uint32_t* sk = alt ? k1 : k0;
-        const uint32_t* sv = alt ? v1 : v0;
+    }
+    const uint32_t* sk = alt ? k1 : k0;
+    const uint32_t* sv = alt ? v1 : v0;
+    k_lower_ptr<<<(unsigned)ceil_div(m + 1, TB * PT), TB, 0, s>>>(sk, m, n, c->eptr, lstart, c->rowptr, long_low);
+    count_launch();
+    if (m > 0 && 2 * m >= 32 * n) {
+        const FinArrays A{sv, c->eu, c->ev, c->ew, c->col, c->eid, c->wn64, c->cw32};
+        k_row_finish_sorted<<<(unsigned)ceil_div(n, FIN_ROWS), TB, 0, s>>>(n, c->rowptr, lstart, c->eptr, A, c->deg);
+        count_launch();
+    } else if (n > 0) {  // a few long rows among short ones
         k_fill_lower<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(sk, sv, m, lstart, c->rowptr, c->eu,
                                                               c->ew, c->col, c->eid, c->wn64); count_launch();
-        k_fill_upper<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(c->eu, c->ev, c->ew, m, c->eptr, lcnt,
-                                                              c->rowptr, c->col, c->eid, c->wn64); count_launch();
-    }
-    GR_TRY_CUDA(c, degree_scale(c), "degree scale");
-    return GR_OK;
-}
-
-cudaError_t degree_scale(gr_ctx* c) {
-    const int64_t n = c->n, m = c->m;
-    if (n > 0) {
-        if (2 * m < 32 * n) {  // mean degree below 32: a thread per row
-            k_degree_scale_rows<<<(unsigned)ceil_div(n, TB), TB, 0, c->stream>>>(c->rowptr, c->col, n, c->wn64,
-                                                                                 c->cw32, c->deg);
-        } else {
-            k_degree_scale<<<(unsigned)ceil_div(n * 32, TB), TB, 0, c->stream>>>(c->rowptr, c->col, n, c->wn64,
-                                                                                c->cw32, c->deg);
-        }
+        k_fill_upper<<<(unsigned)ceil_div(m, TB), TB, 0, s>>>(c->eu, c->ev, c->ew, m, c->eptr, c->rowptr,
+                                                              c->col, c->eid, c->wn64); count_launch();
+        k_degree_scale_rows<<<(unsigned)ceil_div(n, TB), TB, 0, s>>>(c->rowptr, c->col, n, c->wn64, c->cw32,
+                                                                     c->deg);
         count_launch();
     }
-    return cudaGetLastError();
+    GR_TRY_CUDA(c, cudaGetLastError(), "csr kernels");
+    return GR_OK;
 }
 
 // ---------------------------------------------------------------------------
