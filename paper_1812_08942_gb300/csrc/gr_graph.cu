@@ -55,19 +55,6 @@ __global__ void __launch_bounds__(TB) k_lower_ptr(const uint32_t* __restrict__ s
     if (far) *long_low = 1;
 }
 
-__global__ void __launch_bounds__(TB) k_keys_from_v(const int32_t* __restrict__ ev, int64_t m,
-                                                    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-    const int64_t t0 = (int64_t)blockIdx.x * (TB * PT) + threadIdx.x;
-#pragma unroll
-    for (int i = 0; i < PT; ++i) {
-        const int64_t e = t0 + i * TB;
-        if (e < m) {
-            keys[e] = (uint32_t)__ldg(ev + e);
-            vals[e] = (uint32_t)e;
-        }
-    }
-}
-
 // lower part of row p: edges (q, p), q < p, in ascending q (= ascending id);
 // position t of the stable sort by v holds the t-th such edge overall.
 __global__ void k_fill_lower(const uint32_t* __restrict__ skey, const uint32_t* __restrict__ sval,
@@ -716,8 +703,8 @@ gr_status build_csr_sorted(gr_ctx* c, int32_t* long_low) {
     uint32_t *k1 = (uint32_t*)p_alt, *v1 = k1 + M;
     int alt = 0;
     if (m > 0) {
-        k_keys_from_v<<<(unsigned)ceil_div(m, TB * PT), TB, 0, s>>>(c->ev, m, k0, v0); count_launch();
-        GR_TRY_CUDA(c, radix_sort_u32(k0, v0, k1, v1, m, bits_for((uint64_t)(n - 1)), c->ws, s, &alt),
+        GR_TRY_CUDA(c, radix_order_u32((const uint32_t*)c->ev, k0, v0, k1, v1, m, bits_for((uint64_t)(n - 1)), c->ws,
+                                       s, &alt),
                     "sort by v");
     }
     const uint32_t* sk = alt ? k1 : k0;
@@ -748,8 +735,7 @@ gr_status build_csr_sorted(gr_ctx* c, int32_t* long_low) {
 // inside one aggregate gets the sentinel, 2 kb ones: no pair, and after all.
 __global__ void __launch_bounds__(TB) k_galerkin_keys(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                                                       const int32_t* __restrict__ agg, int64_t m, int kb,
-                                                      uint64_t sentinel, uint64_t* __restrict__ keys,
-                                                      uint32_t* __restrict__ vals) {
+                                                      uint64_t sentinel, uint64_t* __restrict__ keys) {
     const int64_t t0 = (int64_t)blockIdx.x * (TB * PT) + threadIdx.x;
     int32_t a[PT], b[PT];
 #pragma unroll
@@ -769,7 +755,6 @@ __global__ void __launch_bounds__(TB) k_galerkin_keys(const int32_t* __restrict_
         if (e >= m) continue;
         const uint64_t lo = (uint32_t)min(a[i], b[i]), hi = (uint32_t)max(a[i], b[i]);
         keys[e] = lo == hi ? sentinel : lo << kb | hi;
-        vals[e] = (uint32_t)e;
     }
 }
 
@@ -905,10 +890,10 @@ gr_status coarsen_impl(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx** out) 
         int kb = bits_for((uint64_t)(nc - 1));
         if (kb < 1) kb = 1;
         const uint64_t sentinel = (1ull << (2 * kb)) - 1ull;
-        k_galerkin_keys<<<(unsigned)ceil_div(m, TB * PT), TB, 0, s>>>(c->eu, c->ev, agg, m, kb, sentinel, k0, v0);
+        k_galerkin_keys<<<(unsigned)ceil_div(m, TB * PT), TB, 0, s>>>(c->eu, c->ev, agg, m, kb, sentinel, k0);
         count_launch();
         int alt = 0;
-        GR_TRY_CUDA(c, radix_sort_u64(k0, v0, k1, v1, m, 2 * kb, c->ws, s, &alt), "sort keys");
+        GR_TRY_CUDA(c, radix_order_u64(k0, k0, v0, k1, v1, m, 2 * kb, c->ws, s, &alt), "sort keys");
         const uint64_t* sk = alt ? k1 : k0;
         const uint32_t* sv = alt ? v1 : v0;
         k_segment_count<<<(unsigned)tiles, TB, 0, s>>>(sk, m, sentinel, head); count_launch();

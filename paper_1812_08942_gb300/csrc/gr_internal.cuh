@@ -174,6 +174,14 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
 cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
                            cudaStream_t s, int* result_in_alt);
+// the same for the keys `in` (left as they are unless in == keys) with their
+// positions as values
+cudaError_t radix_order_u32(const uint32_t* in, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
+                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
+                            cudaStream_t s, int* result_in_alt);
+cudaError_t radix_order_u64(const uint64_t* in, uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
+                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
+                            cudaStream_t s, int* result_in_alt);
 int bits_for(uint64_t max_value_inclusive);
 // 64 bytes of pinned host memory owned by the calling thread, for small
 // readbacks inside one API call (never held across calls).

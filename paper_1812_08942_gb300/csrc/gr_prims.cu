@@ -359,7 +359,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter(
     uint32_t v[SORT_ITEMS];
 #pragma unroll
     for (int c = 0; c < SORT_ITEMS; ++c)
-        v[c] = w0 + c * 32 < total ? __ldg(vals + tbase + w0 + c * 32) : 0u;
+        v[c] = !vals ? (uint32_t)(tbase + w0 + c * 32)
+                     : w0 + c * 32 < total ? __ldg(vals + tbase + w0 + c * 32) : 0u;
     __syncthreads();
     int32_t g[SORT_ITEMS];
 #pragma unroll
@@ -392,19 +393,23 @@ static cudaError_t radix_scatter(const KT* keys, const uint32_t* vals, int64_t c
     return cudaGetLastError();
 }
 
+// in, vin: the input (keys and vals themselves, or other arrays, which stay as
+// they are; vin null: the values are the positions)
 template <typename KT>
-static cudaError_t radix_sort(KT* keys, uint32_t* vals, KT* keys_alt, uint32_t* vals_alt, int64_t count,
-                              int bits, Workspace& ws, cudaStream_t s, int* result_in_alt) {
+static cudaError_t radix_sort(const KT* in, const uint32_t* vin, KT* keys, uint32_t* vals, KT* keys_alt,
+                              uint32_t* vals_alt, int64_t count, int bits, Workspace& ws, cudaStream_t s, int* result_in_alt) {
     *result_in_alt = 0;
-    if (count <= 1 || bits <= 0) return cudaSuccess;
+    if (count <= 0 || bits <= 0) return cudaSuccess;
     const int passes = (bits + 9) / 10;
     const int width = (bits + passes - 1) / passes < 8 ? 8 : (bits + passes - 1) / passes;
     const int nb = (int)ceil_div(count, SORT_TILE);
     void* p = nullptr;
     GR_CUDA(ws.get(WS_SORT_HIST, (sizeof(int32_t) << width) * (size_t)nb, &p));
     int32_t* hist = (int32_t*)p;
-    KT *ki = keys, *ko = keys_alt;
-    uint32_t *vi = vals, *vo = vals_alt;
+    const KT* ki = in;
+    const uint32_t* vi = vin;
+    KT* ko = keys_alt;
+    uint32_t* vo = vals_alt;
     for (int i = 0; i < passes; ++i) {
         const int shift = i * width;
         k_radix_hist<KT><<<nb, SORT_THREADS, 0, s>>>(ki, count, shift, width, hist, nb); count_launch();
@@ -414,8 +419,10 @@ static cudaError_t radix_sort(KT* keys, uint32_t* vals, KT* keys_alt, uint32_t* 
             : width == 9 ? radix_scatter<KT, 9>(ki, vi, count, shift, hist, nb, ko, vo, s)
                          : radix_scatter<KT, 10>(ki, vi, count, shift, hist, nb, ko, vo, s);
         if (e != cudaSuccess) return e;
-        KT* tk = ki; ki = ko; ko = tk;
-        uint32_t* tv = vi; vi = vo; vo = tv;
+        ki = ko;
+        vi = vo;
+        ko = ko == keys ? keys_alt : keys;
+        vo = vo == vals ? vals_alt : vals;
     }
     *result_in_alt = passes & 1;
     return cudaSuccess;
@@ -424,12 +431,22 @@ static cudaError_t radix_sort(KT* keys, uint32_t* vals, KT* keys_alt, uint32_t* 
 cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
                            cudaStream_t s, int* result_in_alt) {
-    return radix_sort<uint32_t>(keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
+    return radix_sort<uint32_t>(keys, vals, keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
 }
 cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
                            cudaStream_t s, int* result_in_alt) {
-    return radix_sort<uint64_t>(keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
+    return radix_sort<uint64_t>(keys, vals, keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
+}
+cudaError_t radix_order_u32(const uint32_t* in, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
+                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
+                            cudaStream_t s, int* result_in_alt) {
+    return radix_sort<uint32_t>(in, nullptr, keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
+}
+cudaError_t radix_order_u64(const uint64_t* in, uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
+                            uint32_t* vals_alt, int64_t count, int bits, Workspace& ws,
+                            cudaStream_t s, int* result_in_alt) {
+    return radix_sort<uint64_t>(in, nullptr, keys, vals, keys_alt, vals_alt, count, bits, ws, s, result_in_alt);
 }
 
 }  // namespace gr
