@@ -419,8 +419,15 @@ __global__ void k_pairs_keys(int32_t npairs, const uint64_t* __restrict__ phi,
 constexpr int SELECT_THREADS = 1024;
 constexpr int32_t SELECT_MAX = 65536;  // larger sets take the radix sort
 
+// What the last pass may merge, from the counters (ctr[1] pairs, ctr[4..7]
+// error flags, ctr[9] pairs that a first pass merged on the device) and the
+// clusters known to the host: ctr[12] = 0 nothing (or too many pairs for one
+// block), 1 the pairs marked in keep, 2 all pairs.
+enum : int32_t { MERGE_NONE = 0, MERGE_KEPT = 1, MERGE_ALL = 2 };
+
 template <bool D64>
-__global__ void __launch_bounds__(SELECT_THREADS) k_select_smallest(int32_t npairs, int32_t allowed,
+__global__ void __launch_bounds__(SELECT_THREADS) k_select_smallest(int64_t n_cur, int deferred, int64_t target_nc,
+                                                                     int32_t* __restrict__ ctr,
                                                                      const uint64_t* __restrict__ phi,
                                                                      const uint32_t* __restrict__ plo,
                                                                      int32_t* __restrict__ keep) {
@@ -429,6 +436,15 @@ __global__ void __launch_bounds__(SELECT_THREADS) k_select_smallest(int32_t npai
     __shared__ uint32_t pre_lo;
     __shared__ int32_t rank;
     constexpr int NPASS = D64 ? 12 : 8;
+    const int32_t npairs = ctr[1];
+    const int64_t budget = n_cur - (deferred ? ctr[9] : 0) - target_nc;
+    const bool any = npairs > 0 && budget > 0 && !(ctr[4] | ctr[5] | ctr[6] | ctr[7]);
+    if (!any || npairs <= budget || npairs > SELECT_MAX) {
+        if (threadIdx.x == 0) ctr[12] = any && npairs <= budget ? MERGE_ALL : MERGE_NONE;
+        return;
+    }
+    if (threadIdx.x == 0) ctr[12] = MERGE_KEPT;
+    const int32_t allowed = (int32_t)budget;
     if (threadIdx.x == 0) {
         pre_hi = 0ull;
         pre_lo = 0u;
@@ -518,12 +534,17 @@ __global__ void k_merge(int32_t npairs, const int32_t* __restrict__ pc, const in
     tail[c] = tail[b];
 }
 
-// every pair merges (the pass cannot exceed its merge budget); pair count on the device
-__global__ void k_merge_all(const int32_t* __restrict__ npairs, const int32_t* __restrict__ pc,
+// pair count on the device: every pair merges (the pass cannot exceed its
+// merge budget), or, with keep, what *mode says
+__global__ void k_merge_all(const int32_t* __restrict__ npairs, const int32_t* __restrict__ mode,
+                            const int32_t* __restrict__ keep, const int32_t* __restrict__ pc,
                             const int32_t* __restrict__ pb, int32_t* __restrict__ cl, int32_t* __restrict__ nxt,
                             int32_t* __restrict__ tail) {
+    const int32_t md = keep ? *mode : MERGE_ALL;
+    if (md == MERGE_NONE) return;
     const int32_t cnt = *npairs;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
+        if (md == MERGE_KEPT && !keep[i]) continue;
         const int32_t c = pc[i], b = pb[i];
         for (int32_t p = b; p >= 0; p = nxt[p]) cl[p] = c;
         nxt[tail[c]] = b;
@@ -637,6 +658,15 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
     // matching has at most n/2 pairs), so it merges on the device without a
     // readback; its counts are checked at the next pass's readback.
     bool deferred = false;
+    // rank of each cluster head (= its smallest member), and their count
+    auto label = [&]() -> cudaError_t {
+        k_head_flags<<<gn, 256, 0, s>>>(n, S.cl, S.flags); count_launch();
+        const cudaError_t e = scan_exclusive_i32(S.flags, S.lab, n, c->ws, s);
+        if (e != cudaSuccess) return e;
+        k_labels<<<gn, 256, 0, s>>>(n, S.cl, S.lab, S.flags, agg, hs + 6); count_launch();
+        return cudaGetLastError();
+    };
+    bool labelled = false;
     for (int pass = 0; pass < passes; ++pass) {
         if (!deferred && n_cur <= target_nc) break;
         const bool first = pass == 0;
@@ -649,13 +679,32 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         else launch_suitor_lpc<false>(c, S, lpc, n_cur, d, chain_cap, first);
         GR_TRY_CUDA(c, cudaGetLastError(), "aggregate matching");
         if (first && passes > 1 && 2 * target_nc <= n_cur) {
-            k_merge_all<<<(unsigned)ceil_div(n / 2 > 0 ? n / 2 : 1, 256), 256, 0, s>>>(S.ctr + 1, S.pc, S.pb, S.cl,
-                                                                                     S.nxt, S.tail);
+            k_merge_all<<<(unsigned)ceil_div(n / 2 > 0 ? n / 2 : 1, 256), 256, 0, s>>>(
+                S.ctr + 1, nullptr, nullptr, S.pc, S.pb, S.cl, S.nxt, S.tail);
             count_launch();
             // keep this pass's heads, pairs and proposals for the next readback
             GR_TRY_CUDA(c, cudaMemcpyAsync(S.ctr + 8, S.ctr, 16, cudaMemcpyDeviceToDevice, s), "copy");
             deferred = true;
             continue;
+        }
+        // The last pass merges on the device and the labels follow, before the
+        // one readback: only more pairs than one block selects from are left
+        // to the host (a wait less a level: about 20 us of an idle GPU).
+        const bool last = pass == passes - 1;
+        const int64_t known = n_cur;
+        if (last) {
+            const unsigned gm = (unsigned)ceil_div(n_cur / 2 > 0 ? n_cur / 2 : 1, 256);
+            if (d_is_f64)
+                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, S.ctr, S.phi, S.plo,
+                                                                     S.keep);
+            else
+                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, S.ctr, S.phi, S.plo,
+                                                                      S.keep);
+            k_merge_all<<<gm, 256, 0, s>>>(S.ctr + 1, S.ctr + 12, S.keep, S.pc, S.pb, S.cl, S.nxt, S.tail);
+            count_launch();
+            count_launch();
+            GR_TRY_CUDA(c, label(), "labels");
+            labelled = true;
         }
         GR_TRY_CUDA(c, cudaMemcpyAsync(hctr, S.ctr, 48, cudaMemcpyDeviceToHost, s), "readback");
         GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
@@ -680,12 +729,17 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         const int32_t npairs = hctr[1];
         if (npairs == 0 || allowed <= 0) break;
         const unsigned gp = (unsigned)ceil_div(npairs, 256);
+        if (last && ((int64_t)npairs <= allowed || npairs <= SELECT_MAX)) {  // merged on the device
+            n_cur -= (int64_t)npairs <= allowed ? npairs : allowed;
+            break;
+        }
+        labelled = false;
         if ((int64_t)npairs > allowed && npairs <= SELECT_MAX) {
             // keep the `allowed` smallest keys: one block selects them
             if (d_is_f64) {
-                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(npairs, (int32_t)allowed, S.phi, S.plo, S.keep);
+                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, S.ctr, S.phi, S.plo, S.keep);
             } else {
-                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(npairs, (int32_t)allowed, S.phi, S.plo, S.keep);
+                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, S.ctr, S.phi, S.plo, S.keep);
             }
             count_launch();
             n_cur -= allowed;
@@ -724,13 +778,11 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         GR_TRY_CUDA(c, cudaGetLastError(), "aggregate merge");
     }
     if (deferred) return set_error(c, GR_ECUDA, "aggregate: internal pass bookkeeping");
-    // labels: rank of each cluster head (= its smallest member)
-    k_head_flags<<<gn, 256, 0, s>>>(n, S.cl, S.flags); count_launch();
-    GR_TRY_CUDA(c, scan_exclusive_i32(S.flags, S.lab, n, c->ws, s), "scan labels");
-    k_labels<<<gn, 256, 0, s>>>(n, S.cl, S.lab, S.flags, agg, hs + 2); count_launch();
-    GR_TRY_CUDA(c, cudaGetLastError(), "labels");
-    GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
-    *nc_out = hs[2];
+    if (!labelled) {
+        GR_TRY_CUDA(c, label(), "labels");
+        GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
+    }
+    *nc_out = hs[6];
     if (*nc_out != n_cur) return set_error(c, GR_ECUDA, "aggregate: internal count mismatch");
     if (proposals_out) *proposals_out = total_proposals;
     return GR_OK;

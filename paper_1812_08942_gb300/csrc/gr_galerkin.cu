@@ -630,9 +630,14 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
     GR_TRY_CUDA(c, cudaMemsetAsync(packed + nc, 0, 8, s), "memset");
     GR_TRY_CUDA(c, scan_exclusive_i64((const int64_t*)packed, (int64_t*)packed, (int64_t)R, c->ws, s), "scan rows");
     GR_TRY_CUDA(c, cudaMemcpyAsync(hs, packed + nc, 8, cudaMemcpyDeviceToHost, s), "readback");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->eptr, sizeof(int64_t) * R, s), "alloc eptr");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->rowptr, sizeof(int64_t) * (R + CSR_PAD_ROWS), s), "alloc rowptr");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->deg, sizeof(double) * (size_t)(nc > 0 ? nc : 1), s), "alloc");
+    SlabPlan rows;
+    const size_t o_eptr = rows.add(sizeof(int64_t) * R), o_row = rows.add(sizeof(int64_t) * (R + CSR_PAD_ROWS)),
+                 o_deg = rows.add(sizeof(double) * (size_t)(nc > 0 ? nc : 1));
+    GR_TRY_CUDA(c, cudaMallocAsync(&cc->slab[0], rows.need, s), "alloc rows");
+    char* b0 = (char*)cc->slab[0];
+    cc->eptr = (int64_t*)(b0 + o_eptr);
+    cc->rowptr = (int64_t*)(b0 + o_row);
+    cc->deg = (double*)(b0 + o_deg);
     k_gal_unpack<<<(unsigned)ceil_div((int64_t)R, GT), GT, 0, s>>>((int64_t)R, packed, cc->rowptr, cc->eptr);
     count_launch();
     GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
@@ -641,13 +646,20 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
         return set_error(c, GR_ECUDA, "coarsen: coarse rows are not symmetric");
     cc->m = mc;
     const size_t cs = (size_t)(2 * mc > 0 ? 2 * mc : 1) + CSR_PAD_SLOTS, ce = (size_t)(mc > 0 ? mc : 1);
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->eu, sizeof(int32_t) * ce, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->ev, sizeof(int32_t) * ce, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->ew, sizeof(double) * ce, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->col, sizeof(int32_t) * cs, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->eid, sizeof(int32_t) * cs, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->cw32, sizeof(int2) * cs, s), "alloc");
-    GR_TRY_CUDA(c, cudaMallocAsync(&cc->wn64, sizeof(double) * cs, s), "alloc");
+    SlabPlan ents;
+    const size_t o_eu = ents.add(sizeof(int32_t) * ce), o_ev = ents.add(sizeof(int32_t) * ce),
+                 o_ew = ents.add(sizeof(double) * ce), o_col = ents.add(sizeof(int32_t) * cs),
+                 o_eid = ents.add(sizeof(int32_t) * cs), o_cw = ents.add(sizeof(int2) * cs),
+                 o_wn = ents.add(sizeof(double) * cs);
+    GR_TRY_CUDA(c, cudaMallocAsync(&cc->slab[1], ents.need, s), "alloc entries");
+    char* b1 = (char*)cc->slab[1];
+    cc->eu = (int32_t*)(b1 + o_eu);
+    cc->ev = (int32_t*)(b1 + o_ev);
+    cc->ew = (double*)(b1 + o_ew);
+    cc->col = (int32_t*)(b1 + o_col);
+    cc->eid = (int32_t*)(b1 + o_eid);
+    cc->cw32 = (int2*)(b1 + o_cw);
+    cc->wn64 = (double*)(b1 + o_wn);
     const int G = 2 * mc >= 32 * nc ? 32 : 4;
     const unsigned grid = (unsigned)ceil_div(nc * G, GT);
     if (G == 32) {

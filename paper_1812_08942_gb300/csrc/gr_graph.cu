@@ -2,6 +2,8 @@
 // and Galerkin coarsening L_R = P^T L_G P (Sec. 3.2.2): row by row in shared
 // memory (gr_galerkin.cu), or by a global sort + segmented sum when a coarse
 // row is too long for that.
+#include <utility>
+
 #include "gr_internal.cuh"
 #include "gr_vec.cuh"
 
@@ -607,20 +609,45 @@ __global__ void __launch_bounds__(FW * 32) k_row_finish_warp(
     }
 }
 
+// the canonical edge list's arrays
+cudaError_t alloc_edges(gr_ctx* c, int64_t m) {
+    const size_t me = (size_t)(m > 0 ? m : 1);
+    SlabPlan sl;
+    const size_t o_u = sl.add(sizeof(int32_t) * me), o_v = sl.add(sizeof(int32_t) * me),
+                 o_w = sl.add(sizeof(double) * me);
+    const cudaError_t e = cudaMallocAsync(&c->slab[0], sl.need, c->stream);
+    if (e != cudaSuccess) {
+        c->slab[0] = nullptr;
+        return e;
+    }
+    c->eu = (int32_t*)((char*)c->slab[0] + o_u);
+    c->ev = (int32_t*)((char*)c->slab[0] + o_v);
+    c->ew = (double*)((char*)c->slab[0] + o_w);
+    return cudaSuccess;
+}
+
 gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
     const int64_t n = c->n, m = c->m;
     cudaStream_t s = c->stream;
     if (invalid) *invalid = false;
     int64_t* hs = host_scratch();
     if (!hs) return set_error(c, GR_ENOMEM, "csr: pinned scratch unavailable");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->eptr, sizeof(int64_t) * (n + 1), s), "alloc eptr");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->rowptr, sizeof(int64_t) * (n + 1 + CSR_PAD_ROWS), s), "alloc rowptr");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->deg, sizeof(double) * (n > 0 ? n : 1), s), "alloc deg");
-    size_t slots = (size_t)(2 * m > 0 ? 2 * m : 1) + CSR_PAD_SLOTS;
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->col, sizeof(int32_t) * slots, s), "alloc col");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->eid, sizeof(int32_t) * slots, s), "alloc eid");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->cw32, sizeof(int2) * slots, s), "alloc cw32");
-    GR_TRY_CUDA(c, cudaMallocAsync(&c->wn64, sizeof(double) * slots, s), "alloc wn64");
+    const size_t slots = (size_t)(2 * m > 0 ? 2 * m : 1) + CSR_PAD_SLOTS;
+    SlabPlan sl;
+    const size_t o_eptr = sl.add(sizeof(int64_t) * (size_t)(n + 1)),
+                 o_row = sl.add(sizeof(int64_t) * (size_t)(n + 1 + CSR_PAD_ROWS)),
+                 o_deg = sl.add(sizeof(double) * (size_t)(n > 0 ? n : 1)), o_col = sl.add(sizeof(int32_t) * slots),
+                 o_eid = sl.add(sizeof(int32_t) * slots), o_cw = sl.add(sizeof(int2) * slots),
+                 o_wn = sl.add(sizeof(double) * slots);
+    GR_TRY_CUDA(c, cudaMallocAsync(&c->slab[1], sl.need, s), "alloc csr");
+    char* base = (char*)c->slab[1];
+    c->eptr = (int64_t*)(base + o_eptr);
+    c->rowptr = (int64_t*)(base + o_row);
+    c->deg = (double*)(base + o_deg);
+    c->col = (int32_t*)(base + o_col);
+    c->eid = (int32_t*)(base + o_eid);
+    c->cw32 = (int2*)(base + o_cw);
+    c->wn64 = (double*)(base + o_wn);
 
     // lcnt (n+1), lfill (n+1), list (n+1), flags (16 B)
     void *p_i32, *p_i64;
@@ -903,10 +930,7 @@ gr_status coarsen_impl(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx** out) 
         GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
         mc = hs[0];
         cc->m = mc;
-        cudaError_t e1 = cudaMallocAsync(&cc->eu, sizeof(int32_t) * (size_t)(mc > 0 ? mc : 1), s);
-        cudaError_t e2 = cudaMallocAsync(&cc->ev, sizeof(int32_t) * (size_t)(mc > 0 ? mc : 1), s);
-        cudaError_t e3 = cudaMallocAsync(&cc->ew, sizeof(double) * (size_t)(mc > 0 ? mc : 1), s);
-        if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
+        if (alloc_edges(cc, mc) != cudaSuccess) {
             set_error(c, GR_ENOMEM, "coarsen: allocation failed");
             return fail(GR_ENOMEM);
         }
@@ -915,11 +939,15 @@ gr_status coarsen_impl(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx** out) 
         GR_TRY_CUDA(c, cudaGetLastError(), "segment sum");
     } else {
         cc->m = 0;
-        cudaMallocAsync(&cc->eu, 4, s);
-        cudaMallocAsync(&cc->ev, 4, s);
-        cudaMallocAsync(&cc->ew, 8, s);
+        if (alloc_edges(cc, 0) != cudaSuccess) {
+            set_error(c, GR_ENOMEM, "coarsen: allocation failed");
+            return fail(GR_ENOMEM);
+        }
     }
+    // in this graph's scratch: the coarse graph is smaller
+    std::swap(c->ws, cc->ws);
     gr_status st = build_csr(cc, false, nullptr);
+    std::swap(c->ws, cc->ws);
     if (st != GR_OK) {
         set_error(c, st, "coarsen: " + cc->last_error);
         return fail(st);

@@ -76,7 +76,9 @@ struct gr_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     int num_sms = 0;
-    // canonical edge list (owned)
+    // the arrays from eu to deg lie in these allocations
+    void* slab[2] = {nullptr, nullptr};
+    // canonical edge list
     int32_t* eu = nullptr;
     int32_t* ev = nullptr;
     double* ew = nullptr;
@@ -123,6 +125,17 @@ struct gr_ctx {
 };
 
 namespace gr {
+
+// Arrays laid out one after the other (256-byte steps) in one allocation: an
+// allocation and its release cost the host 1.3 us, a level has eleven arrays.
+struct SlabPlan {
+    size_t need = 0;
+    size_t add(size_t bytes) {
+        const size_t off = need;
+        need += (bytes + 255) & ~size_t(255);
+        return off;
+    }
+};
 
 // band sweep (gr_band.cu).  ensure_locality fills the context's locality
 // profile (one kernel and a readback into host memory; 264 bytes of device
@@ -194,6 +207,7 @@ uint64_t launch_count();
 
 // graph construction (gr_graph.cu).  build_csr checks that the edge list is
 // canonical when `check` is set (*invalid reports a failed check, GR_EINVAL).
+cudaError_t alloc_edges(gr_ctx* c, int64_t m);
 gr_status build_csr(gr_ctx* c, bool check, bool* invalid);
 // from a global sort by v; *long_low (device, may be null) is raised by a
 // lower part past ROW_PART_SHORT edges
