@@ -19,6 +19,7 @@
 // larger one (169k rows of 37 slots: 162 us; a thread each, with networks of
 // up to 64 keys, 176).  A sorting network costs O(s log^2 s)
 // per row, so graphs with longer rows use the global sort.
+#include "gr_ieee.cuh"
 #include "gr_internal.cuh"
 #include "gr_vec.cuh"
 
@@ -512,7 +513,7 @@ __global__ void k_gal_fill(int64_t nc, const RowMeta* __restrict__ meta, const i
     } else {
         dA = deg[A];
     }
-    const double inv = dA > 0.0 ? 1.0 / dA : 0.0;
+    const double inv = row_inverse(dA);
     for (int32_t i = l; i < U; i += G) {
         const int32_t B = ucol[base + i];
         const double w = uw[base + i];

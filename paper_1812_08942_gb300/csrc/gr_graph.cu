@@ -4,6 +4,7 @@
 // row is too long for that.
 #include <utility>
 
+#include "gr_ieee.cuh"
 #include "gr_internal.cuh"
 #include "gr_vec.cuh"
 
@@ -147,7 +148,7 @@ __device__ __forceinline__ double fin_inverse(double s, double* __restrict__ deg
         if (lane < FIN_ROWS) {
             const double d = part[lane][0];
             if (p < n) deg[p] = d;
-            inv[lane] = d > 0.0 ? 1.0 / d : 0.0;
+            inv[lane] = row_inverse(d);
         }
     }
     __syncthreads();
@@ -289,14 +290,14 @@ __global__ void __launch_bounds__(TB, 4) k_degree_scale_rows(const int64_t* __re
             double s = 0.0;
             for (int j = b; j < e; ++j) s += W[j];
             deg[p] = s;
-            const double inv = s > 0.0 ? 1.0 / s : 0.0;
+            const double inv = row_inverse(s);
             for (int j = b; j < e; ++j) W[j] = W[j] * inv;
         }
         __syncwarp();
         for (int j = lane; j < ns; j += 32) {
             const double x = W[j];
             wn64[R0 + j] = x;
-            cw32[R0 + j] = make_int2(C[j], __float_as_int((float)x));
+            cw32[R0 + j] = make_int2(C[j], __float_as_int(f64_to_f32(x)));
         }
         return;
     }
@@ -305,11 +306,11 @@ __global__ void __launch_bounds__(TB, 4) k_degree_scale_rows(const int64_t* __re
     double s = 0.0;
     for (int64_t j = b; j < e; ++j) s += wn64[j];
     deg[p] = s;
-    const double inv = s > 0.0 ? 1.0 / s : 0.0;
+    const double inv = row_inverse(s);
     for (int64_t j = b; j < e; ++j) {
         const double x = wn64[j] * inv;
         wn64[j] = x;
-        cw32[j] = make_int2(col[j], __float_as_int((float)x));
+        cw32[j] = make_int2(col[j], __float_as_int(f64_to_f32(x)));
     }
 }
 
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(TB, 4) k_row_finish_thread(int64_t n, const in
                 sum += w;
             }
             deg[p] = sum;
-            const double inv = sum > 0.0 ? 1.0 / sum : 0.0;
+            const double inv = row_inverse(sum);
             for (int i = 0; i < L + U; ++i) S_w[b + i] = S_w[b + i] * inv;
         }
         __syncwarp();
@@ -502,7 +503,7 @@ __global__ void __launch_bounds__(TB, 4) k_row_finish_thread(int64_t n, const in
             col[R0 + j] = cj;
             eid[R0 + j] = S_eid[j];
             wn64[R0 + j] = x;
-            cw32[R0 + j] = make_int2(cj, __float_as_int((float)x));
+            cw32[R0 + j] = make_int2(cj, __float_as_int(f64_to_f32(x)));
         }
         return;
     }
@@ -535,12 +536,12 @@ __global__ void __launch_bounds__(TB, 4) k_row_finish_thread(int64_t n, const in
         sum += w;
     }
     deg[p] = sum;
-    const double inv = sum > 0.0 ? 1.0 / sum : 0.0;
+    const double inv = row_inverse(sum);
     const int64_t r1 = r0 + L + (e1 - e0);
     for (int64_t j = r0; j < r1; ++j) {
         const double x = wn64[j] * inv;
         wn64[j] = x;
-        cw32[j] = make_int2(col[j], __float_as_int((float)x));
+        cw32[j] = make_int2(col[j], __float_as_int(f64_to_f32(x)));
     }
 }
 
@@ -599,11 +600,11 @@ __global__ void __launch_bounds__(FW * 32) k_row_finish_warp(
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0) deg[p] = sum;
-        const double inv = sum > 0.0 ? 1.0 / sum : 0.0;
+        const double inv = row_inverse(sum);
         for (int64_t i = lane; i < len; i += 32) {
             const double x = wn64[r0 + i] * inv;
             wn64[r0 + i] = x;
-            cw32[r0 + i] = make_int2(col[r0 + i], __float_as_int((float)x));
+            cw32[r0 + i] = make_int2(col[r0 + i], __float_as_int(f64_to_f32(x)));
         }
         __syncwarp();
     }
