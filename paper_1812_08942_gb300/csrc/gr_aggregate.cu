@@ -422,11 +422,14 @@ constexpr int32_t SELECT_MAX = 65536;  // larger sets take the radix sort
 // What the last pass may merge, from the counters (ctr[1] pairs, ctr[4..7]
 // error flags, ctr[9] pairs that a first pass merged on the device) and the
 // clusters known to the host: ctr[12] = 0 nothing (or too many pairs for one
-// block), 1 the pairs marked in keep, 2 all pairs.
+// block), 1 the pairs marked in keep, 2 all pairs; ctr[13] = 1 if the call is
+// to be refused (error flags, or proposals past a positive budget): then
+// nothing is merged and no label written.
 enum : int32_t { MERGE_NONE = 0, MERGE_KEPT = 1, MERGE_ALL = 2 };
 
 template <bool D64>
 __global__ void __launch_bounds__(SELECT_THREADS) k_select_smallest(int64_t n_cur, int deferred, int64_t target_nc,
+                                                                     int64_t max_proposals,
                                                                      int32_t* __restrict__ ctr,
                                                                      const uint64_t* __restrict__ phi,
                                                                      const uint32_t* __restrict__ plo,
@@ -438,7 +441,12 @@ __global__ void __launch_bounds__(SELECT_THREADS) k_select_smallest(int64_t n_cu
     constexpr int NPASS = D64 ? 12 : 8;
     const int32_t npairs = ctr[1];
     const int64_t budget = n_cur - (deferred ? ctr[9] : 0) - target_nc;
-    const bool any = npairs > 0 && budget > 0 && !(ctr[4] | ctr[5] | ctr[6] | ctr[7]);
+    const unsigned long long* proposals = reinterpret_cast<const unsigned long long*>(ctr);  // [1] this pass, [5] the first
+    const bool refused = (ctr[4] | ctr[5] | ctr[6] | ctr[7]) ||
+                         (max_proposals > 0 && ((int64_t)proposals[1] > max_proposals ||
+                                                (deferred && (int64_t)proposals[5] > max_proposals)));
+    if (threadIdx.x == 0 && refused) ctr[13] = 1;
+    const bool any = npairs > 0 && budget > 0 && !refused;
     if (!any || npairs <= budget || npairs > SELECT_MAX) {
         if (threadIdx.x == 0) ctr[12] = any && npairs <= budget ? MERGE_ALL : MERGE_NONE;
         return;
@@ -558,8 +566,9 @@ __global__ void k_head_flags(int64_t n, const int32_t* __restrict__ cl, int32_t*
 }
 
 __global__ void k_labels(int64_t n, const int32_t* __restrict__ cl, const int32_t* __restrict__ lab,
-                         const int32_t* __restrict__ flags, int32_t* __restrict__ agg,
-                         int64_t* __restrict__ nc_out) {
+                         const int32_t* __restrict__ flags, const int32_t* __restrict__ refused,
+                         int32_t* __restrict__ agg, int64_t* __restrict__ nc_out) {
+    if (*refused) return;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) agg[i] = lab[cl[i]];
     if (i == n - 1) *nc_out = (int64_t)lab[i] + flags[i];
@@ -663,7 +672,7 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         k_head_flags<<<gn, 256, 0, s>>>(n, S.cl, S.flags); count_launch();
         const cudaError_t e = scan_exclusive_i32(S.flags, S.lab, n, c->ws, s);
         if (e != cudaSuccess) return e;
-        k_labels<<<gn, 256, 0, s>>>(n, S.cl, S.lab, S.flags, agg, hs + 6); count_launch();
+        k_labels<<<gn, 256, 0, s>>>(n, S.cl, S.lab, S.flags, S.ctr + 13, agg, hs + 6); count_launch();
         return cudaGetLastError();
     };
     bool labelled = false;
@@ -695,11 +704,11 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         if (last) {
             const unsigned gm = (unsigned)ceil_div(n_cur / 2 > 0 ? n_cur / 2 : 1, 256);
             if (d_is_f64)
-                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, S.ctr, S.phi, S.plo,
-                                                                     S.keep);
+                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, max_proposals, S.ctr, S.phi,
+                                                                     S.plo, S.keep);
             else
-                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, S.ctr, S.phi, S.plo,
-                                                                      S.keep);
+                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(known, deferred, target_nc, max_proposals, S.ctr, S.phi,
+                                                                      S.plo, S.keep);
             k_merge_all<<<gm, 256, 0, s>>>(S.ctr + 1, S.ctr + 12, S.keep, S.pc, S.pb, S.cl, S.nxt, S.tail);
             count_launch();
             count_launch();
@@ -737,9 +746,11 @@ gr_status aggregate_impl(gr_ctx* c, const void* d, int d_is_f64, int64_t target_
         if ((int64_t)npairs > allowed && npairs <= SELECT_MAX) {
             // keep the `allowed` smallest keys: one block selects them
             if (d_is_f64) {
-                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, S.ctr, S.phi, S.plo, S.keep);
+                k_select_smallest<true><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, 0, S.ctr, S.phi, S.plo,
+                                                                     S.keep);
             } else {
-                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, S.ctr, S.phi, S.plo, S.keep);
+                k_select_smallest<false><<<1, SELECT_THREADS, 0, s>>>(n_cur, 0, target_nc, 0, S.ctr, S.phi, S.plo,
+                                                                     S.keep);
             }
             count_launch();
             n_cur -= allowed;
