@@ -126,8 +126,9 @@ __global__ void k_cf_values(int64_t n, const int64_t* __restrict__ rowptr, const
 // its slot values av and diagonal ad.  Short rows: W lanes per row (16 for
 // p <= 16, else a warp), lanes over columns, the row's products in slot order.
 // A filter step on a thousand rows is bound by its round trips: eight slots'
-// neighbour rows are fetched together (1,000 rows of 13 slots, p = 16: 5.9 us a
-// step; one slot at a time and a warp per row of 16 columns 6.8).
+// neighbour rows are fetched together (1,000 rows of 13 slots, p = 16, L2
+// emptied before: 7.8 us a step; one slot at a time and a warp per row of 16
+// columns 8.3; 5.9 with the step before it in L2).
 template <int W>
 __global__ void k_cf_apply(int64_t n, int p, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                            const double* __restrict__ av, const double* __restrict__ ad, double c1, double c2,
