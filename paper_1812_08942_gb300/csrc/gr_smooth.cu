@@ -1120,6 +1120,10 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_init(int64_t n, const int64_t
 // round reads was written before it.  Every node is handled once: rounds over
 // all nodes took 43 us each on a 101 x 89 x 75 mesh (18 rounds), with a host
 // wait after each; colouring and five sweeps of it went from 1,870 to 959 us.
+// A thread per node, or (L = 32, mean degree 32 and more) a warp: a thread
+// walking a hub's row holds its round up (100,000 nodes, 3 M edges: 70 ms a
+// colouring against 6.6).
+template <int L>
 __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restrict__ rowptr,
                                                          const int32_t* __restrict__ col,
                                                          const int32_t* __restrict__ list,
@@ -1139,7 +1143,9 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restri
     __syncthreads();
     const int32_t cnt = *count;
     int32_t top = -1;
-    for (int64_t t = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * JP_THREADS) {
+    const int l = threadIdx.x % L;
+    for (int64_t t = ((int64_t)blockIdx.x * JP_THREADS + threadIdx.x) / L; t < cnt;
+         t += (int64_t)gridDim.x * JP_THREADS / L) {
         const int32_t i = list[t];
         const int64_t b = rowptr[i], e = rowptr[i + 1];
         // the smallest colour not used by a coloured neighbour, 64 candidates
@@ -1147,24 +1153,27 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restri
         int32_t c = 0;
         for (int32_t base = 0;; base += 64) {
             unsigned long long used = 0;
-            for (int64_t j = b; j < e; j += 8) {
+            for (int64_t j = b + l; j < e; j += 8 * L) {
                 int32_t cq[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) cq[u] = j + u < e ? __ldcg(colour + col[j + u]) : -1;
+                for (int u = 0; u < 8; ++u) cq[u] = j + u * L < e ? __ldcg(colour + col[j + u * L]) : -1;
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
                     if (cq[u] >= base && cq[u] < base + 64) used |= 1ull << (cq[u] - base);
             }
+            if constexpr (L == 32)
+                used = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(used >> 32)) << 32 |
+                       __reduce_or_sync(0xffffffffu, (unsigned)used);
             if (~used) {
                 c = base + __ffsll((long long)~used) - 1;
                 break;
             }
         }
-        for (int64_t j = b; j < e; j += 8) {
+        for (int64_t j = b + l; j < e; j += 8 * L) {
             int32_t q[8], was[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                q[u] = j + u < e ? col[j + u] : -1;
+                q[u] = j + u * L < e ? col[j + u * L] : -1;
                 if (q[u] >= 0 && __ldcg(colour + q[u]) >= 0) q[u] = -1;
             }
 #pragma unroll
@@ -1177,7 +1186,7 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restri
                     else next[atomicAdd(next_count, 1)] = q[u];
                 }
         }
-        colour[i] = c;
+        if (l == 0) colour[i] = c;
         top = c > top ? c : top;
     }
     top = __reduce_max_sync(0xffffffffu, top);
@@ -1257,8 +1266,12 @@ static gr_status gs_prepare(gr_ctx* c, uint64_t colour_seed, int32_t* colour_out
     int cur = 0;
     while (left > 0) {
         for (int r = 0; r < BATCH; ++r) {
-            k_jp_round<<<gr, JP_THREADS, 0, s>>>(c->rowptr, c->col, lists[cur], ctr + r, colour, pending,
-                                                lists[cur ^ 1], ctr + r + 1, ctr + BATCH + 1);
+            if (2 * c->m >= 32 * n)
+                k_jp_round<32><<<gr, JP_THREADS, 0, s>>>(c->rowptr, c->col, lists[cur], ctr + r, colour, pending,
+                                                        lists[cur ^ 1], ctr + r + 1, ctr + BATCH + 1);
+            else
+                k_jp_round<1><<<gr, JP_THREADS, 0, s>>>(c->rowptr, c->col, lists[cur], ctr + r, colour, pending,
+                                                       lists[cur ^ 1], ctr + r + 1, ctr + BATCH + 1);
             count_launch();
             cur ^= 1;
         }
