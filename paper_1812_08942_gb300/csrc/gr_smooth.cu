@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 
 #include "gr_internal.cuh"
+#include "gr_slots.cuh"
 #include "gr_sweep.cuh"
 #include "gr_vec.cuh"
 
@@ -836,7 +837,9 @@ static cudaError_t launch_sweep_row(gr_ctx* c, const SweepPlan& P, const T* Ain,
         if (bps4 < 1) bps4 = 1;
         if (bps4d < 1) bps4d = 1;
     }
-    const bool four = sizeof(T) < 8 && c->n > 0 && 2.0 * (double)c->m / (double)c->n >= 10.0;
+    const bool four = sizeof(T) < 8 && c->n > 0 && 2.0 * (double)c->m / (double)c->n >= 10.0 &&
+                      slots_step_fits(2 * (unsigned long long)c->m, 4);
+    // (two at a time always fit: 2m <= 2^32 - 2)
     const bool dense = four && sizeof(T) == 4 && c->n >= ROW_DENSE_MIN_ROWS &&
                        (size_t)c->n * K * sizeof(T) <= ROW_DENSE_MAX_BYTES;
     int grid = c->num_sms * (dense ? bps4d : (four ? bps4 : bps2));
@@ -1354,18 +1357,18 @@ __global__ void __launch_bounds__(SM_THREADS) k_gs_class(int64_t cnt, const int3
     load_chunk_rw<T, E>(X + i * K + q * E, xi);
 #pragma unroll
     for (int t = 0; t < E; ++t) acc[t] = Acc(0);
-    for (unsigned j = b; j < e; j += U) {
+    for (SlotRun s(b, e); s.left; s.next(U)) {
         Slot v[U];
         Acc x[U][E];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j + u < e) v[u] = __ldg(slots + j + u);
+            if (s.has(u)) v[u] = __ldg(slots + s.at + u);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j + u < e) load_chunk_rw<T, E>(X + (int64_t)slot_col(v[u]) * K + q * E, x[u]);
+            if (s.has(u)) load_chunk_rw<T, E>(X + (int64_t)slot_col(v[u]) * K + q * E, x[u]);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j + u < e) {
+            if (s.has(u)) {
                 const Acc w = slot_w(v[u], Acc(0));
 #pragma unroll
                 for (int t = 0; t < E; ++t) acc[t] = fma(w, x[u][t], acc[t]);
