@@ -738,14 +738,20 @@ gr_status adjoint_pick(gr_ctx* cc, int S, double omega, const float* mass, const
 
 gr_status loss_fine(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, int K, float* y0, float* Rf,
                     float* mass, bool* bad) {
-    switch (K) {
-        case 4: return fine_k<4>(f, cc, agg, X, y0, Rf, mass, bad);
-        case 8: return fine_k<8>(f, cc, agg, X, y0, Rf, mass, bad);
-        case 16: return fine_k<16>(f, cc, agg, X, y0, Rf, mass, bad);
-        case 24: return fine_k<24>(f, cc, agg, X, y0, Rf, mass, bad);
-        case 32: return fine_k<32>(f, cc, agg, X, y0, Rf, mass, bad);
-    }
-    return set_error(f, GR_EINVAL, "loss: K must be 4, 8, 16, 24 or 32");
+    auto run = [&]() {
+        switch (K) {
+            case 4: return fine_k<4>(f, cc, agg, X, y0, Rf, mass, bad);
+            case 8: return fine_k<8>(f, cc, agg, X, y0, Rf, mass, bad);
+            case 16: return fine_k<16>(f, cc, agg, X, y0, Rf, mass, bad);
+            case 24: return fine_k<24>(f, cc, agg, X, y0, Rf, mass, bad);
+            case 32: return fine_k<32>(f, cc, agg, X, y0, Rf, mass, bad);
+        }
+        return set_error(f, GR_EINVAL, "loss: K must be 4, 8, 16, 24 or 32");
+    };
+    const gr_status st = run();
+    // a refused call leaves no kernel behind that reads X or writes R_f
+    if (st != GR_OK || *bad) cudaStreamSynchronize(f->stream);
+    return st;
 }
 
 gr_status loss_work(gr_ctx* cc, int K, int S, bool adjoint, LossWork* W) {

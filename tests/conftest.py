@@ -19,3 +19,15 @@ def oracle_mod():
 
     oracle.build()
     return oracle
+
+
+@pytest.fixture(scope="session")
+def gpu_lib():
+    """The package with its library built and loaded."""
+    from paper_1812_08942_gb300 import build
+
+    build.build()
+    import paper_1812_08942_gb300 as gr
+
+    gr.load()
+    return gr
