@@ -136,6 +136,14 @@ class Graph:
         self.m = int(m)
         self.device = device
         self.stream = stream
+        self._torch_stream = None
+
+    def torch_stream(self):
+        """The stream as torch's object (it stays its creator's)."""
+        if self._torch_stream is None:
+            self._torch_stream = (torch.cuda.ExternalStream(self.stream, self.device) if self.stream
+                                  else torch.cuda.default_stream(self.device))
+        return self._torch_stream
 
     def __del__(self):
         h = getattr(self, "handle", None)
@@ -147,11 +155,18 @@ class Graph:
         self.__del__()
 
 
-def _join(g):
-    """Calls that queue their last kernels without waiting: a caller on another
-    stream than g's gets its results, and may free its inputs, as after a wait."""
-    if g.stream != torch.cuda.current_stream(g.device).cuda_stream:
-        torch.cuda.synchronize(g.device)
+def _join(g, *tensors):
+    """After a call that queues its last kernels without waiting, before its
+    status is looked at: a caller on another stream than g's gets its results,
+    and may free ``tensors``, as after a wait; on g's stream, a tensor of a
+    third stream is not given out again before g's stream is done with it.
+    (Only device tensors can be held so; the call's host tensors are waited for.)"""
+    s = g.torch_stream()
+    if g.stream != torch.cuda.current_stream(g.device).cuda_stream or not all(t.is_cuda for t in tensors):
+        s.synchronize()
+    else:
+        for t in tensors:
+            t.record_stream(s)
 
 
 # ---------------------------------------------------------------------------
@@ -375,8 +390,8 @@ def graph_reduce_reduce_data(levels, F, mean=False):
     out = torch.empty(levels[-1].n, F.shape[1], dtype=F.dtype, device=F.device)
     st = load().graph_reduce_reduce_data(arr, len(levels), _ptr(F), int(F.shape[1]),
                                          1 if F.dtype == torch.float64 else 0, 1 if mean else 0, _ptr(out))
+    _join(levels[0], F)
     _check(st, levels[0].handle)
-    _join(levels[0])
     return out
 
 
@@ -403,12 +418,13 @@ def graph_reduce_loss_fwd(fine: Graph, coarse: Graph, agg, X, w_c, sweeps_c, ome
     K = int(X.shape[1])
     assert X.dtype == torch.float32 and w_c.dtype == torch.float32 and w_c.numel() == coarse.m
     loss = torch.empty(1, dtype=torch.float32, device=X.device)
+    given = (agg, X, w_c) if saved is None else (agg, X, w_c, saved)
     if saved is None:
         saved = torch.empty(loss_saved_numel(coarse.n, K), dtype=torch.float32, device=X.device)
     st = load().graph_reduce_loss_fwd(fine.handle, coarse.handle, _ptr(agg), _ptr(X), K, _ptr(w_c), int(sweeps_c),
                                       float(omega), _ptr(loss), _ptr(saved))
+    _join(fine, *given)
     _check(st, fine.handle)
-    _join(fine)
     return loss, saved
 
 
