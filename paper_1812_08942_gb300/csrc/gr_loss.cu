@@ -358,6 +358,7 @@ __device__ __forceinline__ void scale_control(const ScaleStep& st, float loss) {
         S.eta = (S.L_prev / S.L0) * st.eta_max;
     }
     S.inv_bound = 1.0 / (S.lam1 * st.bound_step);
+    *st.lam_next = ~0ull;
     *st.loss_hist = loss;
     S.L_prev = L;
     S.it += 1;

@@ -20,6 +20,7 @@ struct ScaleStep {
     ScaleState* state = nullptr;
     double eta_max = 0.0, eps = 0.0, bound_step = 0.0, alpha = 0.0;
     const unsigned long long* lam_prev = nullptr;  // bits of the last update's smallest ratio (NULL: first iteration)
+    unsigned long long* lam_next = nullptr;        // where this one's will be taken: emptied by the loop control
     float* loss_hist = nullptr;                    // entry of this iteration
     const double* dG = nullptr;
     const double* dP = nullptr;

@@ -12,17 +12,21 @@
 #include <math.h>
 #include <string.h>
 
-#include <vector>
-
 #include "gr_loss.cuh"
 
 namespace gr {
+
+// iterations whose loss and lambda_1 the device keeps before the host reads
+// them: scratch of a fixed size, since kmax may be any number ("until it
+// converges")
+constexpr int64_t SCALE_HIST = 1024;
 
 gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, const float* X, int K, int sweeps,
                            double omega, double alpha, double eta_max, double delta_bar, double eps, int kmax,
                            float* w, int32_t* iters_out, double* loss_hist, double* lam1_hist) {
     cudaStream_t s = fine->stream;
     const int64_t nc = coarse->n, mc = coarse->m;
+    const int64_t hist = kmax < SCALE_HIST ? kmax : SCALE_HIST;
     size_t need = 0;
     auto add = [&](size_t bytes) {
         size_t off = need;
@@ -31,7 +35,7 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
     };
     const size_t o_dG = add(8 * (size_t)nc), o_dP = add(8 * (size_t)nc), o_dw = add(4 * (size_t)mc),
                  o_y0 = add(4 * (size_t)nc * K), o_Rf = add(4 * (size_t)K), o_mass = add(4 * (size_t)nc),
-                 o_state = add(sizeof(ScaleState)), o_loss = add(4 * (size_t)kmax), o_lam = add(8 * (size_t)kmax);
+                 o_state = add(sizeof(ScaleState)), o_loss = add(4 * (size_t)hist), o_lam = add(8 * (size_t)hist);
     void* base;
     GR_TRY_CUDA(fine, fine->ws.get(WS_SCALE, need, &base), "scaling scratch");
     char* B = (char*)base;
@@ -43,7 +47,8 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
     float* mass = (float*)(B + o_mass);
     ScaleState* state = (ScaleState*)(B + o_state);
     float* lossd = (float*)(B + o_loss);
-    unsigned long long* lam = (unsigned long long*)(B + o_lam);  // per update: bits of the smallest d_G / d_P after it
+    // per update (k - 1 modulo hist): bits of the smallest d_G / d_P after it
+    unsigned long long* lam = (unsigned long long*)(B + o_lam);
     int64_t* hs = host_scratch();
     if (!hs) return set_error(fine, GR_ENOMEM, "scale_edges: pinned scratch unavailable");
 
@@ -57,7 +62,7 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
     GR_TRY_CUDA(fine, cudaMemcpyAsync(W.Y, y0, 4 * (size_t)nc * K, cudaMemcpyDeviceToDevice, s), "copy");
     GR_TRY_CUDA(fine, cudaMemsetAsync(dw, 0, 4 * (size_t)mc, s), "memset");
     GR_TRY_CUDA(fine, cudaMemsetAsync(state, 0, sizeof(ScaleState), s), "memset");
-    GR_TRY_CUDA(fine, cudaMemsetAsync(lam, 0xff, 8 * (size_t)kmax, s), "memset");
+    GR_TRY_CUDA(fine, cudaMemsetAsync(lam, 0xff, 8 * (size_t)hist, s), "memset");
 
     ScaleStep step;
     step.state = state;
@@ -71,6 +76,7 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
     step.w = w;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     auto done = [&](gr_status r) {
+        if (r != GR_OK) cudaStreamSynchronize(s);  // a failed call leaves no kernel that reads X
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
         return r;
@@ -79,9 +85,31 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
             return done(set_error(fine, GR_ECUDA, "scale_edges: event"));
     auto cuda = [&](cudaError_t e) { return e == cudaSuccess ? GR_OK : cuda_error(fine, e, "scale_edges"); };
+    // the histories of the updates done, from update `read` on, which begins the device's arrays
+    ScaleState now;
+    int64_t read = 0;
+    double lam1 = 1.0;
+    auto read_hist = [&](int64_t len) {
+        float hl[SCALE_HIST];
+        unsigned long long hm[SCALE_HIST];
+        gr_status r = cuda(cudaMemcpyAsync(&now, state, sizeof(now), cudaMemcpyDeviceToHost, s));
+        if (r == GR_OK) r = cuda(cudaMemcpyAsync(hl, lossd, 4 * (size_t)len, cudaMemcpyDeviceToHost, s));
+        if (r == GR_OK) r = cuda(cudaMemcpyAsync(hm, lam, 8 * (size_t)len, cudaMemcpyDeviceToHost, s));
+        const gr_status sync = cuda(cudaStreamSynchronize(s));
+        if (r == GR_OK) r = sync;
+        if (r != GR_OK) return r;
+        for (int64_t i = read; i < now.it && i < read + len; ++i) {
+            const unsigned long long b = hm[i - read];
+            if (b != ~0ull) memcpy(&lam1, &b, 8);
+            if (loss_hist) loss_hist[i] = (double)hl[i - read];
+            if (lam1_hist) lam1_hist[i] = lam1;
+        }
+        read += len;
+        return GR_OK;
+    };
     bool stopped = false;
-    for (int k = 1; k <= kmax; ++k) {
-        const int slot = k & 1;
+    for (int64_t k = 1; k <= kmax; ++k) {
+        const int slot = (int)(k & 1);
         if (k > 2) {  // has iteration k - 2 ended the loop?
             if ((st = cuda(cudaEventSynchronize(ev[slot]))) != GR_OK) return done(st);
             if (((const int32_t*)hs)[slot]) {
@@ -89,15 +117,18 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
                 break;
             }
         }
+        unsigned long long* prev = k > 1 ? lam + (k - 2) % hist : nullptr;
         if (k == 1) {
             st = loss_weights(coarse, w, W, dG, nullptr, nullptr);
             if (st == GR_OK) st = cuda(cudaMemcpyAsync(dP, dG, 8 * (size_t)nc, cudaMemcpyDeviceToDevice, s));
         } else {
-            st = loss_weights(coarse, w, W, dP, dG, lam + (k - 2));
+            st = loss_weights(coarse, w, W, dP, dG, prev);
         }
+        if (st == GR_OK && k > 1 && (k - 1) % hist == 0) st = read_hist(hist);
         if (st != GR_OK) return done(st);
-        step.lam_prev = k > 1 ? lam + (k - 2) : nullptr;
-        step.loss_hist = lossd + (k - 1);
+        step.lam_prev = prev;
+        step.lam_next = lam + (k - 1) % hist;
+        step.loss_hist = lossd + (k - 1) % hist;
         st = loss_coarse(coarse, K, sweeps, omega, W.Y, Rf, mass, W, true, nullptr, nullptr, step);
         if (st == GR_OK) st = loss_adjoint(coarse, K, sweeps, omega, mass, W, nullptr, step);
         if (st == GR_OK) st = cuda(cudaMemcpyAsync((int32_t*)hs + slot, &state->stop, 4, cudaMemcpyDeviceToHost, s));
@@ -105,23 +136,10 @@ gr_status scale_edges_impl(gr_ctx* fine, gr_ctx* coarse, const int32_t* agg, con
         if (st != GR_OK) return done(st);
     }
     // lambda_1 after the last update
-    if (!stopped) st = loss_weights(coarse, w, W, dP, dG, lam + (kmax - 1));
-    ScaleState end;
-    std::vector<float> hl((size_t)kmax);
-    std::vector<unsigned long long> hm((size_t)kmax);
-    if (st == GR_OK) st = cuda(cudaMemcpyAsync(&end, state, sizeof(end), cudaMemcpyDeviceToHost, s));
-    if (st == GR_OK) st = cuda(cudaMemcpyAsync(hl.data(), lossd, 4 * (size_t)kmax, cudaMemcpyDeviceToHost, s));
-    if (st == GR_OK) st = cuda(cudaMemcpyAsync(hm.data(), lam, 8 * (size_t)kmax, cudaMemcpyDeviceToHost, s));
-    const gr_status sync = cuda(cudaStreamSynchronize(s));
-    if (st == GR_OK) st = sync;
+    if (!stopped) st = loss_weights(coarse, w, W, dP, dG, lam + (kmax - 1) % hist);
+    if (st == GR_OK) st = read_hist(hist < kmax - read ? hist : kmax - read);
     if (st != GR_OK) return done(st);
-    double lam1 = 1.0;
-    for (int i = 0; i < end.it; ++i) {
-        if (hm[i] != ~0ull) memcpy(&lam1, &hm[i], 8);
-        if (loss_hist) loss_hist[i] = (double)hl[i];
-        if (lam1_hist) lam1_hist[i] = lam1;
-    }
-    if (iters_out) *iters_out = end.it;
+    if (iters_out) *iters_out = now.it;
     return done(cuda(cudaGetLastError()));
 }
 
