@@ -457,13 +457,19 @@ __global__ void __launch_bounds__(MEDIUM_WARPS * 32) k_gal_rows_medium(
     }
 }
 
-// row pointers and edge-id bases from the scanned pairs
-__global__ void k_gal_unpack(int64_t R, const unsigned long long* __restrict__ p, int64_t* __restrict__ rowptr,
+// row pointers and edge-id bases from the scanned pairs; p[R] is raised by a
+// row with more than ROW_PART_SHORT entries on a side of the diagonal
+__global__ void k_gal_unpack(int64_t R, unsigned long long* p, int64_t* __restrict__ rowptr,
                              int64_t* __restrict__ eptr) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= R) return;
-    rowptr[i] = (int64_t)(p[i] >> 32);
-    eptr[i] = (int64_t)(p[i] & 0xffffffffull);
+    const unsigned long long x = p[i];
+    rowptr[i] = (int64_t)(x >> 32);
+    eptr[i] = (int64_t)(x & 0xffffffffull);
+    if (i + 1 == R) return;
+    const unsigned long long d = p[i + 1] - x;  // (entries, entries past the row)
+    const unsigned all = (unsigned)(d >> 32), up = (unsigned)d;
+    if (up > ROW_PART_SHORT || all - up > ROW_PART_SHORT) p[R] = 1;
 }
 
 // D(A, A) of short rows, a thread per row: the weights in slot order
@@ -561,7 +567,7 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
     };
     const size_t R = (size_t)nc + 1;
     const size_t o_cnt = add(8 * R), o_flags = add(64), o_sptr = add(8 * R), o_place = add(4 * (size_t)n),
-                 o_med = add(4 * R), o_meta = add(sizeof(RowMeta) * R), o_pack = add(8 * R);
+                 o_med = add(4 * R), o_meta = add(sizeof(RowMeta) * R), o_pack = add(8 * (R + 1));
     void* pr;
     GR_TRY_CUDA(c, c->ws.get(WS_GAL_ROWS, need, &pr), "coarsen scratch");
     char* Bp = (char*)pr;
@@ -628,9 +634,8 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
     GR_TRY_CUDA(c, cudaGetLastError(), "galerkin rows");
 
     // coarse row pointers and edge-id bases: one scan of (entries, entries past the row)
-    GR_TRY_CUDA(c, cudaMemsetAsync(packed + nc, 0, 8, s), "memset");
+    GR_TRY_CUDA(c, cudaMemsetAsync(packed + nc, 0, 16, s), "memset");
     GR_TRY_CUDA(c, scan_exclusive_i64((const int64_t*)packed, (int64_t*)packed, (int64_t)R, c->ws, s), "scan rows");
-    GR_TRY_CUDA(c, cudaMemcpyAsync(hs, packed + nc, 8, cudaMemcpyDeviceToHost, s), "readback");
     SlabPlan rows;
     const size_t o_eptr = rows.add(sizeof(int64_t) * R), o_row = rows.add(sizeof(int64_t) * (R + CSR_PAD_ROWS)),
                  o_deg = rows.add(sizeof(double) * (size_t)(nc > 0 ? nc : 1));
@@ -641,7 +646,9 @@ gr_status galerkin_rows(gr_ctx* c, const int32_t* agg, int64_t nc, gr_ctx* cc, b
     cc->deg = (double*)(b0 + o_deg);
     k_gal_unpack<<<(unsigned)ceil_div((int64_t)R, GT), GT, 0, s>>>((int64_t)R, packed, cc->rowptr, cc->eptr);
     count_launch();
+    GR_TRY_CUDA(c, cudaMemcpyAsync(hs, packed + nc, 16, cudaMemcpyDeviceToHost, s), "readback");
     GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
+    cc->parts = hs[1] ? 0 : 1;
     const int64_t mc = (int64_t)((uint64_t)hs[0] & 0xffffffffull);
     if ((int64_t)((uint64_t)hs[0] >> 32) != 2 * mc)
         return set_error(c, GR_ECUDA, "coarsen: coarse rows are not symmetric");

@@ -681,6 +681,7 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
         }
         lmax = hf[1];
         c->short_rows = sparse && lmax <= ROW_PART_SHORT && !hf[3];
+        if (sparse) c->parts = c->short_rows ? 1 : 0;
     }
     k_upper_ptr<<<(unsigned)ceil_div(m + 1, TB * PT), TB, 0, s>>>(c->eu, m, n, c->eptr); count_launch();
     if (!sparse || lmax > LOWER_WARP) {
@@ -689,6 +690,7 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
         GR_TRY_CUDA(c, cudaMemcpyAsync(hs, flags, 16, cudaMemcpyDeviceToHost, s), "readback");
         GR_TRY_CUDA(c, cudaStreamSynchronize(s), "sync");
         c->short_rows = !((const int32_t*)hs)[3];
+        c->parts = c->short_rows ? 1 : 0;
         return GR_OK;
     }
     int64_t* rowcnt = (int64_t*)p_i64;
@@ -712,6 +714,35 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
     }
     GR_TRY_CUDA(c, cudaGetLastError(), "csr kernels");
     return GR_OK;
+}
+
+// *longer = 1 if a row has more than ROW_PART_SHORT slots on a side of the diagonal
+__global__ void k_row_parts(int64_t n, const int64_t* __restrict__ rowptr, const int64_t* __restrict__ eptr,
+                            int64_t* __restrict__ longer) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int64_t up = eptr[p + 1] - eptr[p], low = rowptr[p + 1] - rowptr[p] - up;
+    if (up > ROW_PART_SHORT || low > ROW_PART_SHORT) *longer = 1;
+}
+
+cudaError_t parts_short(gr_ctx* c, bool* yes) {
+    *yes = c->parts == 1;
+    if (c->parts >= 0) return cudaSuccess;
+    cudaStreamCaptureStatus cap;
+    GR_CUDA(cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return cudaSuccess;
+    int64_t* hs = host_scratch();
+    if (!hs) return cudaErrorMemoryAllocation;
+    hs[0] = 0;
+    if (c->n > 0) {
+        k_row_parts<<<(unsigned)ceil_div(c->n, TB), TB, 0, c->stream>>>(c->n, c->rowptr, c->eptr, hs);
+        count_launch();
+    }
+    GR_CUDA(cudaGetLastError());
+    GR_CUDA(cudaStreamSynchronize(c->stream));
+    c->parts = hs[0] ? 0 : 1;
+    *yes = c->parts == 1;
+    return cudaSuccess;
 }
 
 // Dense graphs, and rows with a lower part too long for one warp's shared

@@ -30,7 +30,8 @@ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 constexpr int64_t CSR_PAD_ROWS = 1;
 constexpr size_t CSR_PAD_SLOTS = 4;
 
-// longest lower and upper part of a row up to which gr_ctx::short_rows holds
+// longest lower and upper part of a row up to which parts_short and
+// gr_ctx::short_rows hold
 constexpr int ROW_PART_SHORT = 64;
 
 // Shape of the band sweep on one graph (gr_band.cu)
@@ -95,6 +96,7 @@ struct gr_ctx {
     int64_t wpart_W = 0;
     int4* cw64 = nullptr;       // 2m: (col, 0, w / deg_row as FP64), built on first FP64 sweep
     bool short_rows = false;    // no row has more than ROW_PART_SHORT slots on either side of the diagonal (false: not known)
+    int parts = -1;             // the same as known so far: 1, 0, or -1 not known (parts_short finds it out)
     // sweep kernel selection (gr_sweep_kernel)
     int sweep_kind = GR_SWEEP_AUTO;
     // locality profile for the band sweep: slots with |col - row| in
@@ -208,6 +210,11 @@ uint64_t launch_count();
 // graph construction (gr_graph.cu).  build_csr checks that the edge list is
 // canonical when `check` is set (*invalid reports a failed check, GR_EINVAL).
 cudaError_t alloc_edges(gr_ctx* c, int64_t m);
+// Whether no row of c has more than ROW_PART_SHORT slots on either side of the
+// diagonal.  Most graphs know from their construction; else one kernel and a
+// wait, once.  (While the stream is captured an unknown graph counts as having
+// such a row.)
+cudaError_t parts_short(gr_ctx* c, bool* yes);
 gr_status build_csr(gr_ctx* c, bool check, bool* invalid);
 // from a global sort by v; *long_low (device, may be null) is raised by a
 // lower part past ROW_PART_SHORT edges

@@ -9,12 +9,17 @@
 //   y_{s+1} = (1-w) y_s + w D_c^-1 A_c y_s          (isolated node: unchanged)
 //   R_c[k]  = y^T L_c y / sum_A M_A (y_A - mu_k)^2,  mu_k = sum M y / sum M
 //   loss    = (1/K) sum_k (R_c[k]/R_f[k] - 1)^2
-// Vectors are FP32; sums are FP32 per lane and FP64 from the warp level up, in
-// a fixed order.
+// Vectors are FP32.  A sum over all rows or edges runs in FP32 over some 64
+// terms a lane, those blocks and a warp's lanes are added in FP32, the rest in
+// FP64, in a fixed order: a lane's error stays that of a few dozen additions
+// whatever the size of the graph and the length of its rows.
 //
 // Layout.  Every pass over vectors is a pass over rows in which G = K / 4
 // lanes hold one row, a 16-byte chunk each (short rows: 32 / G rows a warp),
 // or a warp holds one row, its sub-groups taking slots in turn (long rows).
+// Sums over edges take the edges in blocks of 64 instead where a row may be
+// long (parts_short): a row pass left a hub of 1,000,000 edges to one lane's
+// chain (231 ms and a relative error of 5e-4 of R_f, K = 8; by edges 0.4 ms and 3e-8).
 // A thread per entry or per edge, reading K scalars 4 bytes at a time, took
 // 17 us for a sweep of the 32,768-node reduced mesh (K = 24) and 200 us for
 // the fine quotients of the 128^3 mesh.  The weights are put in slot order
@@ -23,7 +28,7 @@
 // block); one-block kernels adding 304 rows of partials took 49 us each,
 // eight per loss and gradient.  Loss and gradient of the 128^3 mesh (K = 24,
 // aggregates of about 64 nodes, 5 sweeps): 1,505 us before, 522 now, of which the fine
-// pass takes 136.
+// pass takes 139.
 #include "gr_loss.cuh"
 #include "gr_sweep.cuh"
 #include "gr_vec.cuh"
@@ -98,12 +103,49 @@ __device__ __forceinline__ void join_row(float4& a) {
     }
 }
 
+// Column sums of a lane, by blocks of SUM_BLOCK terms or a little more.  The
+// closed blocks' sums are in shared memory, an entry per thread: in registers
+// they cost the fine pass 68 bytes of spills, and loss and gradient of the
+// 128^3 mesh 540 us against 522 (518 in one chain).
+constexpr unsigned SUM_BLOCK = 64;
+struct LaneSum {
+    float4 open;
+    float4* closed;
+    __device__ explicit LaneSum(float4* shared) : open(make_float4(0.f, 0.f, 0.f, 0.f)), closed(shared + threadIdx.x) {
+        if (shared) *closed = open;  // (none: not used)
+    }
+    __device__ __forceinline__ void close() {
+        *closed = total();
+        open = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __device__ __forceinline__ float4 total() const {
+        const float4 c = *closed;
+        return make_float4(c.x + open.x, c.y + open.y, c.z + open.z, c.w + open.w);
+    }
+};
+struct LaneSums {
+    LaneSum a, b;
+    unsigned terms;
+    __device__ explicit LaneSums(float4 (*shared)[LT]) : a(shared[0]), b(shared[1]), terms(0) {}
+    __device__ __forceinline__ void close() {
+        a.close();
+        b.close();
+        terms = 0;
+    }
+    // t more terms have been added
+    __device__ __forceinline__ void count(unsigned t) {
+        terms += t;
+        if (terms >= SUM_BLOCK) close();
+    }
+};
+
 // Two column sums per lane (chunks s1, s2) into the block's partial row:
-// lanes of one chunk added in FP32, warps in FP64.  True in the last block,
+// lanes of one chunk added in FP32, warps in FP64.  COUNT: the first sum of s2
+// is the whole numbers `cnt` of the warp's lanes.  True in the last block,
 // with the totals in red (K of s1, then K of s2).
-template <int K, bool LONG>
+template <int K, bool LONG, bool COUNT = false>
 __device__ bool finish_cols(const RowLanes<K, LONG>& m, float4 s1, float4 s2, double* part, unsigned* counter,
-                            double* red) {
+                            double* red, unsigned cnt = 0) {
     using L = RowLanes<K, LONG>;
     __shared__ double ws[LW][2 * K];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -124,6 +166,10 @@ __device__ bool finish_cols(const RowLanes<K, LONG>& m, float4 s1, float4 s2, do
             ws[warp][K + lane * 4 + i] = (double)a[4 + i];
         }
     }
+    if constexpr (COUNT) {
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) ws[warp][K] = (double)cnt;
+    }
     __syncthreads();
     if (threadIdx.x < 2 * K) {
         double t = 0.0;
@@ -133,6 +179,61 @@ __device__ bool finish_cols(const RowLanes<K, LONG>& m, float4 s1, float4 s2, do
     __threadfence();
     __syncthreads();
     return finish_partials<K, LT>(part, gridDim.x, counter, red);
+}
+
+__device__ __forceinline__ void add_squares(float4& s, const float4& x) {
+    s.x = fmaf(x.x, x.x, s.x);
+    s.y = fmaf(x.y, x.y, s.y);
+    s.z = fmaf(x.z, x.z, s.z);
+    s.w = fmaf(x.w, x.w, s.w);
+}
+// s += w (x - y)^2
+__device__ __forceinline__ void add_edge(float4& s, float w, const float4& x, const float4& y) {
+    float t = x.x - y.x;
+    s.x = fmaf(w * t, t, s.x);
+    t = x.y - y.y;
+    s.y = fmaf(w * t, t, s.y);
+    t = x.z - y.z;
+    s.z = fmaf(w * t, t, s.z);
+    t = x.w - y.w;
+    s.w = fmaf(w * t, t, s.w);
+}
+
+// S.a += w(e) (x_u - x_v)^2 over blocks g, g + groups, ... of SUM_BLOCK edges
+// of the canonical list; Xq: the lane's chunk of row 0
+template <typename Wt>
+__device__ __forceinline__ void edge_blocks(int64_t m, int64_t g, int64_t groups, const int32_t* __restrict__ eu,
+                                            const int32_t* __restrict__ ev, const float* __restrict__ Xq, int K,
+                                            LaneSums& S, Wt weight) {
+    constexpr int U = 4;
+    static_assert(SUM_BLOCK % U == 0, "a block is whole rounds");
+    for (int64_t b = g * SUM_BLOCK; b < m; b += groups * SUM_BLOCK) {
+        const int64_t e = b + SUM_BLOCK < m ? b + SUM_BLOCK : m;
+        int32_t cur = -1;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t j = b; j < e; j += U) {
+            int32_t p[U], q[U];
+            float w[U];
+            float4 y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + u < e) {
+                    p[u] = __ldg(eu + j + u);
+                    q[u] = __ldg(ev + j + u);
+                    w[u] = weight(j + u);
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + u < e) y[u] = ld4(Xq + (int64_t)q[u] * K);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j + u < e) {
+                    if (p[u] != cur) x = ld4(Xq + (int64_t)(cur = p[u]) * K);
+                    add_edge(S.a.open, w[u], x, y[u]);
+                }
+        }
+        S.close();
+    }
 }
 
 // R_f: per column sum_e w (x_u - x_v)^2 over the edges (p, v) of row p and
@@ -145,7 +246,8 @@ __global__ void __launch_bounds__(LT, ROW_BLOCKS) k_fine_quotients(int64_t n, co
     __shared__ double red[LT];
     const RowLanes<K, LONG> m;
     constexpr int U = 2, TS = RowLanes<K, LONG>::TS, RPW = RowLanes<K, LONG>::RPW;
-    float4 num = make_float4(0.f, 0.f, 0.f, 0.f), den = num;
+    __shared__ float4 closed[2][LT];
+    LaneSums S(closed);  // numerator, denominator
     // 32-bit row and edge numbers (n, m < 2^31) keep the kernel at 4 blocks per SM or more
     const unsigned rows = (unsigned)n, stride = ((gridDim.x * LT) >> 5) * RPW;
     unsigned p = ((blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg;
@@ -169,12 +271,7 @@ __global__ void __launch_bounds__(LT, ROW_BLOCKS) k_fine_quotients(int64_t n, co
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(ew + b1));
             }
         }
-        if (m.t == 0) {
-            den.x = fmaf(x.x, x.x, den.x);
-            den.y = fmaf(x.y, x.y, den.y);
-            den.z = fmaf(x.z, x.z, den.z);
-            den.w = fmaf(x.w, x.w, den.w);
-        }
+        if (m.t == 0) add_squares(S.b.open, x);
         for (unsigned j = b + m.t; j < e; j += U * TS) {
             float w[U];
             float4 y[U];
@@ -186,19 +283,36 @@ __global__ void __launch_bounds__(LT, ROW_BLOCKS) k_fine_quotients(int64_t n, co
                 }
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u * TS < e) {
-                    float t = x.x - y[u].x;
-                    num.x = fmaf(w[u] * t, t, num.x);
-                    t = x.y - y[u].y;
-                    num.y = fmaf(w[u] * t, t, num.y);
-                    t = x.z - y[u].z;
-                    num.z = fmaf(w[u] * t, t, num.z);
-                    t = x.w - y[u].w;
-                    num.w = fmaf(w[u] * t, t, num.w);
-                }
+                if (j + u * TS < e) add_edge(S.a.open, w[u], x, y[u]);
         }
+        S.count(e - b + 1);
     }
-    if (finish_cols<K, LONG>(m, num, den, part, counter, red) && threadIdx.x < K)
+    if (finish_cols<K, LONG>(m, S.a.total(), S.b.total(), part, counter, red) && threadIdx.x < K)
+        Rf[threadIdx.x] = (float)(red[threadIdx.x] / red[K + threadIdx.x]);
+}
+
+// The same with the edges in blocks of SUM_BLOCK for graphs that may have long
+// rows: G lanes take a block of consecutive edges, four in flight; the first
+// end's row is loaded again only where it changes.
+template <int K>
+__global__ void __launch_bounds__(LT) k_fine_edges(int64_t n, int64_t m, const int32_t* __restrict__ eu,
+                                                   const int32_t* __restrict__ ev, const double* __restrict__ ew,
+                                                   const float* __restrict__ X, double* part, unsigned* counter,
+                                                   float* __restrict__ Rf) {
+    __shared__ double red[LT];
+    const RowLanes<K, false> L;
+    constexpr int RPW = RowLanes<K, false>::RPW;
+    __shared__ float4 closed[2][LT];
+    LaneSums S(closed);
+    const int64_t groups = (((int64_t)gridDim.x * LT) >> 5) * RPW;
+    const int64_t g = L.ok ? (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + L.seg : n + m;  // past both ends
+    const float* Xq = X + L.q * 4;
+    edge_blocks(m, g, groups, eu, ev, Xq, K, S, [&](int64_t e) { return f64_to_f32(__ldg(ew + e)); });
+    for (int64_t p = g; p < n; p += groups) {
+        add_squares(S.b.open, ld4(Xq + p * K));
+        S.count(1);
+    }
+    if (finish_cols<K, false>(L, S.a.total(), S.b.total(), part, counter, red) && threadIdx.x < K)
         Rf[threadIdx.x] = (float)(red[threadIdx.x] / red[K + threadIdx.x]);
 }
 
@@ -287,7 +401,7 @@ __global__ void __launch_bounds__(LT) k_param_slots(int64_t nc, const int64_t* _
 // y1 = (1-w) y + w z.  SWEEP false: y1 = y, nothing written.  MEAN: the
 // mass-weighted column means of y1 end in mu.
 template <int K, bool LONG, bool SWEEP, bool MEAN>
-__global__ void __launch_bounds__(LT) k_param_sweep(int64_t n, const int64_t* __restrict__ rowptr,
+__global__ void __launch_bounds__(LT, 3) k_param_sweep(int64_t n, const int64_t* __restrict__ rowptr,
                                                     const int2* __restrict__ cw, const float* __restrict__ D,
                                                     const float* __restrict__ y, float omega,
                                                     float* __restrict__ z_out, float* __restrict__ y1,
@@ -297,7 +411,9 @@ __global__ void __launch_bounds__(LT) k_param_sweep(int64_t n, const int64_t* __
     const RowLanes<K, LONG> m;
     constexpr int RPW = RowLanes<K, LONG>::RPW;
     const float zero = 0.f, one_m = 1.f - omega;
-    float4 sy = make_float4(zero, zero, zero, zero), sm = sy;
+    __shared__ float4 closed[MEAN ? LT : 1];
+    LaneSum S(MEAN ? closed : nullptr);
+    unsigned terms = 0, total = 0;  // sizes are whole numbers, n of them in all
     const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
     for (int64_t A = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg; A < n; A += stride) {
         float4 yi = make_float4(zero, zero, zero, zero);
@@ -325,17 +441,19 @@ __global__ void __launch_bounds__(LT) k_param_sweep(int64_t n, const int64_t* __
         if constexpr (MEAN) {
             if (m.writes()) {
                 const float M = mass[A];
-                sy.x = fmaf(M, yi.x, sy.x);
-                sy.y = fmaf(M, yi.y, sy.y);
-                sy.z = fmaf(M, yi.z, sy.z);
-                sy.w = fmaf(M, yi.w, sy.w);
-                sm.x += M;
+                S.open.x = fmaf(M, yi.x, S.open.x);
+                S.open.y = fmaf(M, yi.y, S.open.y);
+                S.open.z = fmaf(M, yi.z, S.open.z);
+                S.open.w = fmaf(M, yi.w, S.open.w);
+                if (m.q == 0) total += (unsigned)M;
+                if (++terms % SUM_BLOCK == 0) S.close();
             }
         }
     }
     if constexpr (MEAN) {
-        if (finish_cols<K, LONG>(m, sy, sm, part, counter, red) && threadIdx.x < K)
-            mu[threadIdx.x] = red[threadIdx.x] / red[K];  // chunk 0's first sum is the total mass
+        const float4 none = make_float4(zero, zero, zero, zero);
+        if (finish_cols<K, LONG, true>(m, S.total(), none, part, counter, red, total) && threadIdx.x < K)
+            mu[threadIdx.x] = red[threadIdx.x] / red[K];
     }
 }
 
@@ -368,10 +486,17 @@ __device__ __forceinline__ void scale_control(const ScaleStep& st, float loss) {
 // every row's slots (each edge twice), sum M (y - mu)^2; in the last block
 // the loss and the adjoint's coefficients
 //   coef[0..K) = 2 g / Q, [K..2K) = 2 g N / Q^2, [2K..3K) = g / Q, [3K..4K) = mu,
-// g = d loss / d R_c.  LY: L y is stored.
-template <int K, bool LONG, bool LY>
+// g = d loss / d R_c.  LY: L y is stored.  LISTED (graphs that may have long
+// rows): the squared differences come from the edge list and its weights w, in
+// blocks; only L y goes through the rows.
+struct EdgeList {
+    int64_t m = 0;
+    const int32_t *eu = nullptr, *ev = nullptr;
+    const float* w = nullptr;
+};
+template <int K, bool LONG, bool LY, bool LISTED>
 __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __restrict__ rowptr,
-                                                  const int2* __restrict__ cw, const float* __restrict__ y,
+                                                  const int2* __restrict__ cw, EdgeList E, const float* __restrict__ y,
                                                   const float* __restrict__ mass, const double* __restrict__ mu,
                                                   double* part, unsigned* counter, const float* __restrict__ Rf,
                                                   const float* __restrict__ grad_loss, float* __restrict__ loss_out,
@@ -380,29 +505,43 @@ __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __re
     const RowLanes<K, LONG> m;
     constexpr int RPW = RowLanes<K, LONG>::RPW;
     const float zero = 0.f;
-    float4 N = make_float4(zero, zero, zero, zero), Q = N, mk = N;
+    __shared__ float4 closed[2][LT];
+    LaneSums S(closed);
+    float4 mk = make_float4(zero, zero, zero, zero);
     if (m.ok) {
         const double* u = mu + m.q * 4;
         mk = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
     }
     const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
-    for (int64_t A = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg; A < n; A += stride) {
+    const int64_t first = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg;
+    if constexpr (LISTED) {
+        // a long row's sub-groups take blocks in turn
+        constexpr int TS = RowLanes<K, LONG>::TS;
+        if (m.ok)
+            edge_blocks(E.m, first * TS + m.t, stride * TS, E.eu, E.ev, y + m.q * 4, K, S,
+                        [&](int64_t e) { return __ldg(E.w + e); });
+    }
+    for (int64_t A = first; A < n; A += stride) {
         float4 ya = make_float4(zero, zero, zero, zero), l = ya;
         if (m.ok) ya = ld4(y + A * K + m.q * 4);
-        for_slots<K, LONG>(m, rowptr[A], rowptr[A + 1], cw, y, [&](float w, const float4& x) {
-            float d = ya.x - x.x, wd = w * d;
-            N.x = fmaf(wd, d, N.x);
-            l.x += wd;
-            d = ya.y - x.y, wd = w * d;
-            N.y = fmaf(wd, d, N.y);
-            l.y += wd;
-            d = ya.z - x.z, wd = w * d;
-            N.z = fmaf(wd, d, N.z);
-            l.z += wd;
-            d = ya.w - x.w, wd = w * d;
-            N.w = fmaf(wd, d, N.w);
-            l.w += wd;
-        });
+        if constexpr (LY || !LISTED) {
+            const int64_t b = rowptr[A], e = rowptr[A + 1];
+            for_slots<K, LONG>(m, b, e, cw, y, [&](float w, const float4& x) {
+                float d = ya.x - x.x, wd = w * d;
+                if (!LISTED) S.a.open.x = fmaf(wd, d, S.a.open.x);
+                l.x += wd;
+                d = ya.y - x.y, wd = w * d;
+                if (!LISTED) S.a.open.y = fmaf(wd, d, S.a.open.y);
+                l.y += wd;
+                d = ya.z - x.z, wd = w * d;
+                if (!LISTED) S.a.open.z = fmaf(wd, d, S.a.open.z);
+                l.z += wd;
+                d = ya.w - x.w, wd = w * d;
+                if (!LISTED) S.a.open.w = fmaf(wd, d, S.a.open.w);
+                l.w += wd;
+            });
+            if (!LISTED) S.terms += (unsigned)(e - b);
+        }
         if constexpr (LY) {
             join_row<K, LONG>(l);
             if (m.writes()) st4(ly_out + A * K + m.q * 4, l);
@@ -410,21 +549,22 @@ __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __re
         if (m.writes()) {
             const float M = mass[A];
             float t = ya.x - mk.x;
-            Q.x = fmaf(M * t, t, Q.x);
+            S.b.open.x = fmaf(M * t, t, S.b.open.x);
             t = ya.y - mk.y;
-            Q.y = fmaf(M * t, t, Q.y);
+            S.b.open.y = fmaf(M * t, t, S.b.open.y);
             t = ya.z - mk.z;
-            Q.z = fmaf(M * t, t, Q.z);
+            S.b.open.z = fmaf(M * t, t, S.b.open.z);
             t = ya.w - mk.w;
-            Q.w = fmaf(M * t, t, Q.w);
+            S.b.open.w = fmaf(M * t, t, S.b.open.w);
         }
+        S.count(1);
     }
-    if (!finish_cols<K, LONG>(m, N, Q, part, counter, red)) return;
+    if (!finish_cols<K, LONG>(m, S.a.total(), S.b.total(), part, counter, red)) return;
     const int k = threadIdx.x;
     if (k >= 32) return;  // the first warp: a column per lane
     double s = 0.0;
     if (k < K) {
-        const double Ns = 0.5 * red[k], Qs = red[K + k], f = (double)Rf[k];
+        const double Ns = LISTED ? red[k] : 0.5 * red[k], Qs = red[K + k], f = (double)Rf[k];
         const double Rc = Ns / Qs, r = Rc / f - 1.0;
         s = r * r;
         if (coef) {
@@ -606,6 +746,16 @@ gr_status fine_quotients(gr_ctx* f, const float* X, double* part, unsigned* coun
     return GR_OK;
 }
 
+template <int K>
+gr_status fine_edges(gr_ctx* f, const float* X, double* part, unsigned* counter, float* Rf) {
+    const int64_t blocks = ceil_div(f->m, SUM_BLOCK), work = blocks > f->n ? blocks : f->n;
+    k_fine_edges<K><<<row_grid<K, false>(f, work), LT, 0, f->stream>>>(f->n, f->m, f->eu, f->ev, f->ew, X, part,
+                                                                      counter, Rf);
+    count_launch();
+    GR_TRY_CUDA(f, cudaGetLastError(), "fine edges");
+    return GR_OK;
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <int K>
@@ -613,6 +763,8 @@ gr_status fine_k(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, floa
                  bool* bad) {
     cudaStream_t s = f->stream;
     const int64_t n = f->n, nc = cc->n;
+    bool short_parts;
+    GR_TRY_CUDA(f, parts_short(f, &short_parts), "row lengths");
     // rows are moved in 16-byte chunks: a block or result that does not start
     // on such a boundary goes through an aligned copy
     const bool cx = !aligned16(X), cy = !aligned16(y0);
@@ -637,8 +789,9 @@ gr_status fine_k(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, floa
     gr_status st = group_begin(cc, WS_LOSS_C, ch, n, nc, &job);
     if (st != GR_OK) return st;
     // upper edges per row: half the slots
-    st = long_rows(f, f->m) ? fine_quotients<K, true>(f, X, part, counter, Rf)
-                            : fine_quotients<K, false>(f, X, part, counter, Rf);
+    if (!short_parts) st = fine_edges<K>(f, X, part, counter, Rf);
+    else st = long_rows(f, f->m) ? fine_quotients<K, true>(f, X, part, counter, Rf)
+                                 : fine_quotients<K, false>(f, X, part, counter, Rf);
     if (st != GR_OK) return st;
     st = group_finish(cc, &job, bad);
     if (st != GR_OK || *bad) return st;
@@ -675,13 +828,19 @@ gr_status coarse_k(gr_ctx* cc, int S, double omega, const float* y0, const float
         count_launch();
         y = out;
     }
-    if (adjoint)
-        k_quotients<K, LONG, true><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, y, mass, W.mu, W.part, W.counter, Rf,
-                                                        grad_loss, loss_out, W.yb1, W.coef, st);
-    else
-        k_quotients<K, LONG, false><<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, y, mass, W.mu, W.part, W.counter, Rf,
-                                                         nullptr, loss_out, nullptr, nullptr, st);
-    count_launch();
+    EdgeList E;
+    E.m = cc->m;
+    E.eu = cc->eu;
+    E.ev = cc->ev;
+    E.w = W.w;
+    auto quotients = [&](auto kern) {
+        kern<<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, E, y, mass, W.mu, W.part, W.counter, Rf,
+                                 adjoint ? grad_loss : nullptr, loss_out, adjoint ? W.yb1 : nullptr,
+                                 adjoint ? W.coef : nullptr, st);
+        count_launch();
+    };
+    if (W.short_parts) adjoint ? quotients(k_quotients<K, LONG, true, false>) : quotients(k_quotients<K, LONG, false, false>);
+    else adjoint ? quotients(k_quotients<K, LONG, true, true>) : quotients(k_quotients<K, LONG, false, true>);
     GR_TRY_CUDA(cc, cudaGetLastError(), "loss");
     return GR_OK;
 }
@@ -769,6 +928,7 @@ gr_status loss_work(gr_ctx* cc, int K, int S, bool adjoint, LossWork* W) {
                  o_Y = add(4 * nK * (adjoint ? (size_t)S + 1 : 2)), o_Z = add(adjoint ? 4 * nK * (size_t)S : 0),
                  o_T = add(adjoint ? 4 * nK * (size_t)S : 0), o_b0 = add(adjoint ? 4 * nK : 0),
                  o_b1 = add(adjoint ? 4 * nK : 0);
+    GR_TRY_CUDA(cc, parts_short(cc, &W->short_parts), "row lengths");
     void* base;
     GR_TRY_CUDA(cc, cc->ws.get(WS_LOSS_B, need, &base), "ws");
     char* B = (char*)base;
@@ -787,16 +947,19 @@ gr_status loss_work(gr_ctx* cc, int K, int S, bool adjoint, LossWork* W) {
     return GR_OK;
 }
 
-gr_status loss_weights(gr_ctx* cc, const float* w, const LossWork& W, double* dP, const double* dG,
+gr_status loss_weights(gr_ctx* cc, const float* w, LossWork& W, double* dP, const double* dG,
                        unsigned long long* lam) {
     cudaStream_t s = cc->stream;
     const int64_t nc = cc->n;
+    W.w = w;
     auto run = [&](auto kern, int lanes) {
         kern<<<(unsigned)ceil_div(nc * lanes, LT), LT, 0, s>>>(nc, cc->rowptr, cc->col, cc->eid, w, W.cw, W.D, dP, dG,
                                                                 lam);
         count_launch();
     };
-    const bool lng = long_rows(cc, 2 * cc->m);
+    // a warp wherever a row may be long: its sum is FP32 (8 lanes on a hub of
+    // 62,500 slots took 5 ms)
+    const bool lng = long_rows(cc, 2 * cc->m) || !W.short_parts;
     if (dP) lng ? run(k_param_slots<32, true>, 32) : run(k_param_slots<8, true>, 8);
     else lng ? run(k_param_slots<32, false>, 32) : run(k_param_slots<8, false>, 8);
     GR_TRY_CUDA(cc, cudaGetLastError(), "parameter weights");

@@ -30,6 +30,8 @@ struct ScaleStep {
 
 // Device buffers of the reduced-graph part
 struct LossWork {
+    bool short_parts;   // of the reduced graph: see parts_short
+    const float* w;     // m: the weights that loss_weights took
     int2* cw;           // 2m: (column, weight) in slot order
     float* D;           // nc: weighted degrees
     double* part;       // per-block partial sums
@@ -49,7 +51,7 @@ gr_status loss_fine(gr_ctx* f, gr_ctx* cc, const int32_t* agg, const float* X, i
 gr_status loss_work(gr_ctx* cc, int K, int sweeps, bool adjoint, LossWork* W);
 // slot-order weights and degrees of w (and, for the edge scaling, FP64 row
 // sums dP and the smallest dG / dP as bits)
-gr_status loss_weights(gr_ctx* cc, const float* w, const LossWork& W, double* dP, const double* dG,
+gr_status loss_weights(gr_ctx* cc, const float* w, LossWork& W, double* dP, const double* dG,
                        unsigned long long* lam);
 // sweeps from W.Y, the quotients and the loss; adjoint: keeps what loss_adjoint reads
 gr_status loss_coarse(gr_ctx* cc, int K, int sweeps, double omega, const float* y0, const float* Rf, const float* mass,
