@@ -158,6 +158,7 @@ __global__ void k_base_mass(int64_t n, const double* __restrict__ deg, int norma
 // took 1,450 us, the passes and the final scaling take 550.
 // ---------------------------------------------------------------------------
 constexpr int MG_BLOCKS = 4;  // per SM
+constexpr int RQ_EDGES = 64;  // consecutive edges of a Rayleigh quotient a thread takes at a time
 
 // Step with R columns left, of which `left` (<= R) exist: V points at the first
 // of them, prev (NULL: step 0, the columns come from row-major Y) holds the
@@ -232,36 +233,52 @@ __global__ void __launch_bounds__(ET) k_mgs_take(int64_t n, int k, const double*
 // x' L x and x' B x of every column: thread per (row, column) over the row's
 // upper edges, w (x_u - x_v)^2, and b x^2 (b NULL: 1).  Column-wise passes
 // over the edge list gathered 8 bytes at a time.  Bound by the FP64 pipe
-// (three operations per edge and column).  out[2 c] and out[2 c + 1].
-__global__ void __launch_bounds__(ET) k_rayleigh(int64_t n, int k, const int64_t* __restrict__ eptr,
-                                                 const int32_t* __restrict__ ev, const double* __restrict__ ew,
-                                                 const double* __restrict__ b, const double* __restrict__ U,
-                                                 double* part, unsigned* counter, double* __restrict__ out) {
+// (three operations per edge and column).  LISTED (graphs that may have long
+// rows): the edges in blocks of 64 of the canonical list, the first end's
+// entry loaded again where it changes; by rows, a hub of 1,000,000 edges took
+// 344 ms.  out[2 c] and out[2 c + 1].
+template <bool LISTED>
+__global__ void __launch_bounds__(ET) k_rayleigh(int64_t n, int k, int64_t m, const int64_t* __restrict__ eptr,
+                                                 const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+                                                 const double* __restrict__ ew, const double* __restrict__ b,
+                                                 const double* __restrict__ U, double* part, unsigned* counter,
+                                                 double* __restrict__ out) {
     __shared__ double red[ET], s1[ET], s2[ET];
     const int rpb = ET / k, c = threadIdx.x % k, rt = threadIdx.x / k;
     double num = 0.0, den = 0.0;
-    if (rt < rpb)
-        for (int64_t r = (int64_t)blockIdx.x * rpb + rt; r < n; r += (int64_t)gridDim.x * rpb) {
+    // edges [e0, e1), four in flight; `cur` is the node whose entry is x
+    auto edges = [&](int64_t e0, int64_t e1, int32_t cur, double x) {
+        constexpr int W = 4;
+        for (int64_t e = e0; e < e1; e += W) {
+            int32_t p[W];
+            double y[W], w[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u)
+                if (e + u < e1) {
+                    if (LISTED) p[u] = __ldg(eu + e + u);
+                    y[u] = U[(int64_t)__ldg(ev + e + u) * k + c];
+                    w[u] = __ldg(ew + e + u);
+                }
+#pragma unroll
+            for (int u = 0; u < W; ++u)
+                if (e + u < e1) {
+                    if (LISTED && p[u] != cur) x = U[(int64_t)(cur = p[u]) * k + c];
+                    const double d = x - y[u];
+                    num = fma(w[u] * d, d, num);
+                }
+        }
+    };
+    if (rt < rpb) {
+        const int64_t first = (int64_t)blockIdx.x * rpb + rt, stride = (int64_t)gridDim.x * rpb;
+        if constexpr (LISTED)
+            for (int64_t e = first * RQ_EDGES; e < m; e += stride * RQ_EDGES)
+                edges(e, e + RQ_EDGES < m ? e + RQ_EDGES : m, -1, 0.0);
+        for (int64_t r = first; r < n; r += stride) {
             const double x = U[r * k + c];
-            const int64_t e1 = eptr[r + 1];
-            constexpr int W = 4;
-            for (int64_t e = eptr[r]; e < e1; e += W) {
-                double y[W], w[W];
-#pragma unroll
-                for (int u = 0; u < W; ++u)
-                    if (e + u < e1) {
-                        y[u] = U[(int64_t)__ldg(ev + e + u) * k + c];
-                        w[u] = __ldg(ew + e + u);
-                    }
-#pragma unroll
-                for (int u = 0; u < W; ++u)
-                    if (e + u < e1) {
-                        const double d = x - y[u];
-                        num = fma(w[u] * d, d, num);
-                    }
-            }
+            if constexpr (!LISTED) edges(eptr[r], eptr[r + 1], (int32_t)r, x);
             den = fma(b ? b[r] * x : x, x, den);
         }
+    }
     s1[threadIdx.x] = num;
     s2[threadIdx.x] = den;
     __syncthreads();
@@ -410,9 +427,15 @@ gr_status eigensolve_impl(gr_ctx* const* levels, int nlevels, int k, int normali
 
     // 4) Rayleigh quotients of the result, x' L x / x' B x
     if (rayleigh_out) {
-        const int64_t qbw = ceil_div(n0 > 0 ? n0 : 1, ET / k);
-        k_rayleigh<<<(unsigned)(RB < qbw ? RB : qbw), ET, 0, s>>>(n0, k, f->eptr, f->ev, f->ew,
-                                                                 normalized ? f->deg : nullptr, U_out, part, ctr, sc);
+        bool short_parts;
+        GR_TRY_CUDA(f, parts_short(f, &short_parts), "row lengths");
+        const int64_t items = !short_parts && ceil_div(f->m, RQ_EDGES) > n0 ? ceil_div(f->m, RQ_EDGES) : n0;
+        const int64_t qbw = ceil_div(items > 0 ? items : 1, ET / k);
+        auto rayleigh = [&](auto kern) {
+            kern<<<(unsigned)(RB < qbw ? RB : qbw), ET, 0, s>>>(n0, k, f->m, f->eptr, f->eu, f->ev, f->ew,
+                                                                normalized ? f->deg : nullptr, U_out, part, ctr, sc);
+        };
+        short_parts ? rayleigh(k_rayleigh<false>) : rayleigh(k_rayleigh<true>);
         count_launch();
         int64_t* hs = host_scratch();
         if (!hs) return set_error(f, GR_ENOMEM, "eigensolve: pinned scratch unavailable");

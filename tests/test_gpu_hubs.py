@@ -73,3 +73,26 @@ def test_loss_and_gradient_of_a_reduced_hub(gpu_lib, oracle_mod, K, S, at, mean)
     grad = gr.graph_reduce_loss_bwd(C, saved, K, w, S, 0.7, torch.ones(1, device=DEV)).double().cpu().numpy()
     assert abs(loss.item() - L_ref) <= 1e-4 * abs(L_ref) + 1e-7
     assert np.linalg.norm(grad - g_ref) <= 1e-4 * np.linalg.norm(g_ref)
+
+
+@pytest.mark.parametrize("k,normalized", [(1, False), (5, True), (8, False), (32, True)])
+@pytest.mark.parametrize("hub_deg,mean,at", [(64, 1, "first"), (65, 1, "first"), (15000, 6, "first"), (15000, 90, "last")])
+def test_rayleigh_quotients(gpu_lib, k, normalized, hub_deg, mean, at):
+    """x' L x / x' B x of the returned columns, FP64 in another order of the
+    sums: 1e-11 relative (2 x 10^5 nodes or a million edges at 2^-53 each)."""
+    gr = gpu_lib
+    n = 20000
+    g = _hubs(n, mean, 2, hub_deg, 11, at)
+    levels = [gr.graph_reduce_create(n, g.u, g.v, g.w)]
+    for r in (10, 10):
+        q = levels[-1].n
+        agg = torch.from_numpy((np.arange(q) // r).astype(np.int32)).to(DEV)
+        levels.append(gr.graph_reduce_coarsen(levels[-1], agg, -(-q // r)))
+    U, lam, rq = gr.graph_reduce_eigensolve(levels, k, normalized=normalized, galerkin_mass=True, iters=3)
+    u, v, w = (torch.from_numpy(x).to(DEV) for x in (g.u, g.v, g.w))
+    u, v = u.long(), v.long()
+    num = (w[:, None] * (U[u] - U[v]) ** 2).sum(0)
+    B = torch.zeros(n, dtype=torch.float64, device=DEV).index_add_(0, u, w).index_add_(0, v, w)
+    den = ((B[:, None] if normalized else 1.0) * U * U).sum(0)
+    want = (num / den).cpu().numpy()
+    assert np.all(np.isfinite(want)) and np.abs(rq / want - 1).max() <= 1e-11
