@@ -1090,25 +1090,44 @@ __device__ __forceinline__ uint64_t gs_prio(uint64_t seed, int64_t i) {
     return splitmix64_at(seed, (1ull << 62) + (uint64_t)i);
 }
 
-// Nodes with no higher-priority neighbour start the first round's list; the
-// others count theirs.
 constexpr int JP_THREADS = 256;
 constexpr int JP_READY = 1024;
+// A thread walks a node's row up to this many slots; a longer one is its warp's
+constexpr int JP_LONG = 128;
+
+// number of row entries from b + l on, in steps of L, with a higher priority than node i
+template <int L>
+__device__ __forceinline__ int32_t jp_above(int64_t i, int64_t b, int64_t e, int l, const int32_t* __restrict__ col,
+                                            uint64_t seed) {
+    const uint64_t pi = gs_prio(seed, i);
+    int32_t above = 0;
+    for (int64_t j = b + l; j < e; j += L) {
+        const int32_t q = col[j];
+        const uint64_t pq = gs_prio(seed, q);
+        above += (pq > pi || (pq == pi && q > i)) ? 1 : 0;
+    }
+    return above;
+}
+
+// Nodes with no higher-priority neighbour start the first round's list; the
+// others count theirs.
 __global__ void __launch_bounds__(JP_THREADS) k_jp_init(int64_t n, const int64_t* __restrict__ rowptr,
                                                         const int32_t* __restrict__ col, uint64_t seed,
                                                         int32_t* __restrict__ colour, int32_t* __restrict__ pending,
                                                         int32_t* __restrict__ list, int32_t* __restrict__ count) {
     const int64_t i = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x;
-    int32_t above = -1;
+    const int lane = threadIdx.x & 31;
+    const int64_t b = i < n ? rowptr[i] : 0, e = i < n ? rowptr[i + 1] : 0;
+    const bool far = e - b > JP_LONG;
+    int32_t above = i < n ? 0 : -1;
+    if (i < n && !far) above = jp_above<1>(i, b, e, 0, col, seed);
+    for (unsigned todo = __ballot_sync(0xffffffffu, far); todo; todo &= todo - 1) {
+        const int o = __ffs(todo) - 1;
+        const int64_t ob = __shfl_sync(0xffffffffu, b, o), oe = __shfl_sync(0xffffffffu, e, o);
+        const int32_t t = __reduce_add_sync(0xffffffffu, jp_above<32>(i - lane + o, ob, oe, lane, col, seed));
+        if (lane == o) above = t;
+    }
     if (i < n) {
-        const uint64_t pi = gs_prio(seed, i);
-        const int64_t e = rowptr[i + 1];
-        above = 0;
-        for (int64_t j = rowptr[i]; j < e; ++j) {
-            const int32_t q = col[j];
-            const uint64_t pq = gs_prio(seed, q);
-            above += (pq > pi || (pq == pi && q > i)) ? 1 : 0;
-        }
         colour[i] = -1;
         pending[i] = above;
     }
@@ -1116,16 +1135,65 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_init(int64_t n, const int64_t
     if (s >= 0) list[s] = (int32_t)i;
 }
 
-// One round over its list: the smallest colour the coloured (= higher-
-// priority) neighbours leave free, then one neighbour fewer to wait for at
-// every uncoloured (= lower-priority) one; those that wait for none form the
-// next round's list.  Two adjacent nodes are never in one list, so what a
+// Node i of a round's list, its row [b, e) walked by L lanes: the smallest
+// colour the coloured (= higher-priority) neighbours leave free, 64 candidates
+// at a time, then one neighbour fewer to wait for at every uncoloured one;
+// eight neighbours' colours, then eight counts in flight.
+template <int L>
+__device__ __forceinline__ int32_t jp_node(int32_t i, int64_t b, int64_t e, int l, const int32_t* __restrict__ col,
+                                           int32_t* colour, int32_t* __restrict__ pending, int32_t* ready,
+                                           int32_t* nready, int32_t* __restrict__ next,
+                                           int32_t* __restrict__ next_count) {
+    int32_t c = 0;
+    for (int32_t base = 0;; base += 64) {
+        unsigned long long used = 0;
+        for (int64_t j = b + l; j < e; j += 8 * L) {
+            int32_t cq[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) cq[u] = j + u * L < e ? __ldcg(colour + col[j + u * L]) : -1;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (cq[u] >= base && cq[u] < base + 64) used |= 1ull << (cq[u] - base);
+        }
+        if constexpr (L == 32)
+            used = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(used >> 32)) << 32 |
+                   __reduce_or_sync(0xffffffffu, (unsigned)used);
+        if (~used) {
+            c = base + __ffsll((long long)~used) - 1;
+            break;
+        }
+    }
+    for (int64_t j = b + l; j < e; j += 8 * L) {
+        int32_t q[8], was[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            q[u] = j + u * L < e ? col[j + u * L] : -1;
+            if (q[u] >= 0 && __ldcg(colour + q[u]) >= 0) q[u] = -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) was[u] = q[u] >= 0 ? atomicSub(&pending[q[u]], 1) : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (was[u] == 1) {
+                const int32_t k = atomicAdd(nready, 1);
+                if (k < JP_READY) ready[k] = q[u];
+                else next[atomicAdd(next_count, 1)] = q[u];
+            }
+    }
+    if (l == 0) colour[i] = c;
+    return c;
+}
+
+// One round over its list; nodes that wait for no neighbour any more form the
+// next round's.  Two adjacent nodes are never in one list, so what a
 // round reads was written before it.  Every node is handled once: rounds over
 // all nodes took 43 us each on a 101 x 89 x 75 mesh (18 rounds), with a host
 // wait after each; colouring and five sweeps of it went from 1,870 to 959 us.
-// A thread per node, or (L = 32, mean degree 32 and more) a warp: a thread
-// walking a hub's row holds its round up (100,000 nodes, 3 M edges: 70 ms a
-// colouring against 6.6).
+// A thread per node, with rows past JP_LONG left to the warp (a star of
+// 1,000,000 leaves: 392 ms a colouring with a thread per row, 37 with the
+// warp; mean degree 13 with hubs of 88,000: 115 and 10), or
+// (L = 32, mean degree 32 and more) a warp per node (100,000 nodes, 3 M edges,
+// with hubs: 70 ms a colouring with a thread per row against 6.6).
 template <int L>
 __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restrict__ rowptr,
                                                          const int32_t* __restrict__ col,
@@ -1146,51 +1214,34 @@ __global__ void __launch_bounds__(JP_THREADS) k_jp_round(const int64_t* __restri
     __syncthreads();
     const int32_t cnt = *count;
     int32_t top = -1;
-    const int l = threadIdx.x % L;
-    for (int64_t t = ((int64_t)blockIdx.x * JP_THREADS + threadIdx.x) / L; t < cnt;
-         t += (int64_t)gridDim.x * JP_THREADS / L) {
-        const int32_t i = list[t];
-        const int64_t b = rowptr[i], e = rowptr[i + 1];
-        // the smallest colour not used by a coloured neighbour, 64 candidates
-        // at a time; eight neighbours' colours, then eight counts in flight
-        int32_t c = 0;
-        for (int32_t base = 0;; base += 64) {
-            unsigned long long used = 0;
-            for (int64_t j = b + l; j < e; j += 8 * L) {
-                int32_t cq[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) cq[u] = j + u * L < e ? __ldcg(colour + col[j + u * L]) : -1;
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (cq[u] >= base && cq[u] < base + 64) used |= 1ull << (cq[u] - base);
+    const int lane = threadIdx.x & 31;
+    if constexpr (L == 32) {
+        for (int64_t t = ((int64_t)blockIdx.x * JP_THREADS + threadIdx.x) / 32; t < cnt;
+             t += (int64_t)gridDim.x * JP_THREADS / 32) {
+            const int32_t i = list[t];
+            const int32_t c = jp_node<32>(i, rowptr[i], rowptr[i + 1], lane, col, colour, pending, ready, &nready, next,
+                                          next_count);
+            top = c > top ? c : top;
+        }
+    } else {
+        for (int64_t t0 = (int64_t)blockIdx.x * JP_THREADS + threadIdx.x - lane; t0 < cnt;
+             t0 += (int64_t)gridDim.x * JP_THREADS) {
+            const bool in = t0 + lane < cnt;
+            const int32_t i = in ? list[t0 + lane] : 0;
+            const int64_t b = in ? rowptr[i] : 0, e = in ? rowptr[i + 1] : 0;
+            const bool far = e - b > JP_LONG;
+            if (in && !far) {
+                const int32_t c = jp_node<1>(i, b, e, 0, col, colour, pending, ready, &nready, next, next_count);
+                top = c > top ? c : top;
             }
-            if constexpr (L == 32)
-                used = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(used >> 32)) << 32 |
-                       __reduce_or_sync(0xffffffffu, (unsigned)used);
-            if (~used) {
-                c = base + __ffsll((long long)~used) - 1;
-                break;
+            for (unsigned todo = __ballot_sync(0xffffffffu, far); todo; todo &= todo - 1) {
+                const int o = __ffs(todo) - 1;
+                const int32_t c = jp_node<32>(__shfl_sync(0xffffffffu, i, o), __shfl_sync(0xffffffffu, b, o),
+                                              __shfl_sync(0xffffffffu, e, o), lane, col, colour, pending, ready,
+                                              &nready, next, next_count);
+                top = c > top ? c : top;
             }
         }
-        for (int64_t j = b + l; j < e; j += 8 * L) {
-            int32_t q[8], was[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                q[u] = j + u * L < e ? col[j + u * L] : -1;
-                if (q[u] >= 0 && __ldcg(colour + q[u]) >= 0) q[u] = -1;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) was[u] = q[u] >= 0 ? atomicSub(&pending[q[u]], 1) : 0;
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (was[u] == 1) {
-                    const int32_t k = atomicAdd(&nready, 1);
-                    if (k < JP_READY) ready[k] = q[u];
-                    else next[atomicAdd(next_count, 1)] = q[u];
-                }
-        }
-        if (l == 0) colour[i] = c;
-        top = c > top ? c : top;
     }
     top = __reduce_max_sync(0xffffffffu, top);
     if ((threadIdx.x & 31) == 0 && top >= 0) atomicMax(&top_s, top);

@@ -96,3 +96,30 @@ def test_rayleigh_quotients(gpu_lib, k, normalized, hub_deg, mean, at):
     den = ((B[:, None] if normalized else 1.0) * U * U).sum(0)
     want = (num / den).cpu().numpy()
     assert np.all(np.isfinite(want)) and np.abs(rq / want - 1).max() <= 1e-11
+
+
+@pytest.mark.parametrize("hub_deg,mean,at", [(125, 1, "first"), (128, 1, "last"), (129, 1, "first"), (8000, 4, "first"),
+                                             (8000, 30, "last"), (8000, 40, "first")])
+def test_colouring(gpu_lib, oracle_mod, hub_deg, mean, at):
+    """Rows on both sides of the length that a thread walks, bit for bit."""
+    gr = gpu_lib
+    n = 9000
+    g = _hubs(n, mean, 3, hub_deg, 13, at)
+    G = gr.graph_reduce_create(n, g.u, g.v, g.w)
+    for seed in (0, 5):
+        col, nc = gr.graph_reduce_colour(G, seed)
+        ref, rnc = oracle_mod.colour(n, g.u, g.v, seed)
+        assert nc == rnc and np.array_equal(col.cpu().numpy(), ref)
+
+
+def test_colouring_of_many_leaves(gpu_lib, oracle_mod):
+    """A star: more leaves become ready at once than a block lists in shared memory."""
+    gr = gpu_lib
+    n = 100000
+    u, v = np.full(n - 1, 777, np.int32), np.setdiff1d(np.arange(n, dtype=np.int32), [777])
+    u, v, w = W.canonicalize(n, u, v, np.ones(n - 1))
+    G = gr.graph_reduce_create(n, u, v, w)
+    for seed in (0, 5, 6):
+        col, nc = gr.graph_reduce_colour(G, seed)
+        ref, rnc = oracle_mod.colour(n, u, v, seed)
+        assert nc == rnc and np.array_equal(col.cpu().numpy(), ref)
