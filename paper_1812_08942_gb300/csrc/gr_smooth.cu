@@ -503,7 +503,9 @@ __device__ __forceinline__ void sweep_row_body(
         }
     }
     const int stride = ((gridDim.x * blockDim.x) >> 5) * RPW;
-    int row = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RPW + (lane_ok ? seg : 0);
+    // (eight slots in flight: fewer rows than lanes, spread over the blocks)
+    const int wid = U == 8 ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    int row = wid * RPW + (lane_ok ? seg : 0);
     const T* Aq = Ain + q * E;
     auto rp = [&](int r, unsigned& b, unsigned& e) {
         if (r < n && lane_ok) {
@@ -649,19 +651,39 @@ struct SweepScratch {
 };
 
 // Streaming sweep when a group of 32 / GP rows would hold more slots than
-// four ring batches (long rows).  FP64 and BF16 blocks of graphs known to have
-// short rows keep the row-group kernel: streaming serves them for its balance
-// over hubs, and without hubs a warp per row of a dozen slots is half idle
-// (neighbour graph of 200,000 nodes, mean degree 11.6, BF16, K = 16: 37 us a
-// sweep against 75; FP64, K = 8, mean degree 17: 105 against 338; with hubs,
-// mean degree 20, BF16, K = 16: 256 against 107).  FP32 blocks keep the rule,
-// and with it the rounding of their column sums.
+// four ring batches (long rows).  FP64 and BF16 blocks of created graphs known
+// to have short rows keep the row-group kernel: streaming serves them for its
+// balance over hubs, and without hubs a warp per row of a dozen slots is half
+// idle (neighbour graph of 200,000 nodes, mean degree 11.6, BF16, K = 16: 37 us
+// a sweep against 75; FP64, K = 8, mean degree 17: 105 against 338; with hubs,
+// mean degree 20, BF16, K = 16: 256 against 107).  But a graph must have rows
+// for every SM, the more the longer they are: a row is one lane group's, slot
+// after slot.  Regular graphs of degree 12 to 124, row-group and streaming, us:
+//   300,000 rows   FP64  K = 8   degree 60   298 | 618    120   549 | 882
+//                  BF16  K = 16  degree 60   129 | 204    120   211 | 341
+//   20,000 rows    FP64  K = 8   degree 60    37 | 60     124    57 | 76
+//                  BF16  K = 8   degree 60    21 | 24      80    27 | 25
+//   5,000 rows     FP64  K = 4   degree 40  20.5 | 20.6    60  24.7 | 21.7
+//                  BF16  K = 8   degree 40  16.4 | 14.8    80  20.5 | 16.5
+//   1,000 rows     FP64  K = 4   degree 40  20.5 | 14.4   100  30.9 | 15.5
+//                  BF16  K = 8   degree 40  16.0 | 14.5   100  21.6 | 14.5
+// The line: a mean degree of 1.5 (FP64) or 0.5 (BF16) times the rows per SM,
+// and up to 45 in any case for K of 8 and more, where at most 4 us are lost.
+// FP32 blocks keep the rule by degree alone, and with it the rounding of their
+// column sums.
 template <typename T, int K>
-static bool stream_wide(const gr_ctx* c) {
+static bool mean_long(const gr_ctx* c) {
     constexpr int GP = RowLayout<T, K>::GP;
     const double avg = c->n > 0 ? 2.0 * (double)c->m / (double)c->n : 0.0;
-    if (sizeof(T) != 4 && c->short_rows) return false;
     return GP < 32 && (32.0 / GP) * avg > 128.0;
+}
+template <typename T, int K>
+static bool stream_wide(const gr_ctx* c) {
+    if (!mean_long<T, K>(c)) return false;
+    if (sizeof(T) == 4 || !c->short_rows) return true;
+    const double avg = 2.0 * (double)c->m / (double)c->n;
+    const double filled = (sizeof(T) == 8 ? 1.5 : 0.5) * (double)c->n / c->num_sms;
+    return avg > filled && !(K >= 8 && avg <= 45.0);
 }
 
 template <typename T>
@@ -851,6 +873,28 @@ static cudaError_t launch_sweep_row(gr_ctx* c, const SweepPlan& P, const T* Ain,
     const typename SlotOf<T>::type* slots;
     if constexpr (sizeof(T) == 8) slots = P.cw64;
     else slots = c->cw32;
+    // Rows of a dozen slots and more that leave the chip half empty: eight
+    // slots in flight, and one warp a block while there are blocks for it
+    // (2,000 rows of 40 slots, FP64, K = 8: 22 us with two slots and full blocks,
+    // 18.5 now; streaming 16.4).
+    if constexpr (sizeof(T) != 4) {
+        static int bps8 = 0;
+        if (!bps8) {
+            GR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps8, k_sweep_row<T, K, 8>, SM_THREADS, 0));
+            if (bps8 < 1) bps8 = 1;
+        }
+        if (mean_long<T, K>(c) && want <= (int64_t)c->num_sms * bps8 && slots_step_fits(2 * (unsigned long long)c->m, 8)) {
+            if (want < c->num_sms) {
+                const int64_t warps = ceil_div(c->n, (int64_t)(32 / RowLayout<T, K>::G));
+                grid = (int)(warps < c->num_sms ? warps : c->num_sms);
+                if (grid > part_cap) grid = part_cap;
+            }
+            k_sweep_row<T, K, 8><<<grid, SM_THREADS, 0, c->stream>>>(c->n, c->rowptr, slots, Ain, Aout, omega, st_in,
+                                                                     part, counter, st_out);
+            count_launch();
+            return cudaGetLastError();
+        }
+    }
     if constexpr (sizeof(T) == 4) {
         if (dense) {
             k_sweep_row_fit4<T, K><<<grid, SM_THREADS, 0, c->stream>>>(c->n, c->rowptr, slots, Ain, Aout, omega,
