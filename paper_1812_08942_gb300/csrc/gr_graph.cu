@@ -680,8 +680,8 @@ gr_status build_csr(gr_ctx* c, bool check, bool* invalid) {
             return set_error(c, GR_EINVAL, "csr: the edge list is not canonical");
         }
         lmax = hf[1];
-        c->short_rows = sparse && lmax <= ROW_PART_SHORT && !hf[3];
-        if (sparse) c->parts = c->short_rows ? 1 : 0;
+        if (sparse) c->parts = lmax <= ROW_PART_SHORT && !hf[3] ? 1 : 0;
+        c->short_rows = check && c->parts == 1;
     }
     k_upper_ptr<<<(unsigned)ceil_div(m + 1, TB * PT), TB, 0, s>>>(c->eu, m, n, c->eptr); count_launch();
     if (!sparse || lmax > LOWER_WARP) {

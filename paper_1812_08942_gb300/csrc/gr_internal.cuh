@@ -95,8 +95,10 @@ struct gr_ctx {
     int32_t* wpart = nullptr;
     int64_t wpart_W = 0;
     int4* cw64 = nullptr;       // 2m: (col, 0, w / deg_row as FP64), built on first FP64 sweep
-    bool short_rows = false;    // no row has more than ROW_PART_SHORT slots on either side of the diagonal (false: not known)
-    int parts = -1;             // the same as known so far: 1, 0, or -1 not known (parts_short finds it out)
+    // no row has more than ROW_PART_SHORT slots on either side of the diagonal:
+    // 1, 0, or -1 not known (parts_short finds it out)
+    int parts = -1;
+    bool short_rows = false;    // parts == 1 of a created graph: what the choice of the sweep kernel goes by
     // sweep kernel selection (gr_sweep_kernel)
     int sweep_kind = GR_SWEEP_AUTO;
     // locality profile for the band sweep: slots with |col - row| in
