@@ -11,9 +11,9 @@
 // last-block finish), so results are reproducible.
 #include <vector>
 
+#include "gr_ieee.cuh"
 #include "gr_internal.cuh"
 #include "gr_sweep.cuh"
-#include "gr_vec.cuh"
 
 namespace gr {
 
@@ -41,21 +41,9 @@ __global__ void k_prolong(int64_t n, int k, const int32_t* __restrict__ map, con
 //   y <- (1 - w) y + g (D^-1 A y)_r:
 // FP64 runs at a small fraction of the FP32 rate on this part, and the
 // division, taken per entry and iteration, cost more than the row's
-// products.  The keep test reads the sign bit of g with an integer compare
-// (a floating compare would take the FP64 pipe too).
-// a / b for b > 0 to within an ulp or so: an FP32 reciprocal refined by one
-// Newton step, and the quotient corrected by its residual -- five FP64
-// operations where the division takes about ten (388 -> 251 us over the
-// hierarchy of a 128^3 mesh, k = 8); b outside FP32's range divides.  The range test is on the exponent: a floating compare is an FP64
-// operation too.
-__device__ __forceinline__ double quotient(double a, double b) {
-    if ((unsigned)((__double2hiint(b) >> 20) - 923) > 200u) return a / b;  // b in [2^-100, 2^101)
-    double y = f32_to_f64(1.0f / f64_to_f32(b));
-    y = fma(y, fma(-b, y, 1.0), y);
-    const double q = a * y;
-    return fma(fma(-b, q, a), y, q);
-}
-
+// products.  The division of the gains runs on the integer pipe, bit for bit
+// the same; both tests of a sign are integer compares (a floating compare
+// would take the FP64 pipe too).
 __global__ void k_shift_gain(int64_t n, int k, const double* __restrict__ deg, const double* __restrict__ lam,
                              const double* __restrict__ b, double omega, double* __restrict__ g) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -64,7 +52,8 @@ __global__ void k_shift_gain(int64_t n, int k, const double* __restrict__ deg, c
     const int c = (int)(idx % k);
     const double D = deg[r];
     const double diag = D - lam[c] * (b ? b[r] : 1.0);
-    g[idx] = __double2hiint(diag) > 0 ? quotient(omega * D, diag) : (diag > 0.0 ? omega * D / diag : -1.0);
+    const bool positive = ieee_bits(diag) - 1 < 0x7ff0000000000000ull;  // and not NaN
+    g[idx] = positive ? ieee_div(omega * D, diag) : -1.0;
 }
 
 // One iteration, thread per (row, column).
