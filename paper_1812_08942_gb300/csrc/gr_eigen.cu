@@ -209,14 +209,15 @@ __global__ void __launch_bounds__(ET, R <= 8 ? MG_BLOCKS : 1) k_mgs_step(int64_t
 }
 
 // U (row-major) = the finished columns over their norms: the first sum of a
-// column's step is its squared norm
+// column's step is its squared norm.  One rounding an entry: the division runs
+// on the integer pipe (times a reciprocal, rounded twice: the same time).
 __global__ void __launch_bounds__(ET) k_mgs_take(int64_t n, int k, const double* __restrict__ V,
                                                  const double* __restrict__ sums, int ld, double* __restrict__ U) {
-    __shared__ double inv[32];
-    if ((int)threadIdx.x < k) inv[threadIdx.x] = 1.0 / sqrt(sums[threadIdx.x * ld]);
+    __shared__ double norm[32];
+    if ((int)threadIdx.x < k) norm[threadIdx.x] = sqrt(sums[threadIdx.x * ld]);
     __syncthreads();
     for (int64_t r = (int64_t)blockIdx.x * ET + threadIdx.x; r < n; r += (int64_t)gridDim.x * ET)
-        for (int i = 0; i < k; ++i) U[r * k + i] = V[(int64_t)i * n + r] * inv[i];
+        for (int i = 0; i < k; ++i) U[r * k + i] = ieee_div(V[(int64_t)i * n + r], norm[i]);
 }
 
 // x' L x and x' B x of every column: thread per (row, column) over the row's
