@@ -6,47 +6,14 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "gr_convert.cuh"
+
 namespace gr {
 
 template <typename T>
 struct AccOf { using type = float; };
 template <>
 struct AccOf<double> { using type = double; };
-
-// FP64 <-> FP32 conversions on the integer pipe.  The conversion unit runs at
-// the FP64 pipe's rate (measured: 626 G a second against 530 G FP64
-// operations and about 20 T integer ones), and a conversion in a branch costs
-// its time even where no lane takes the branch, so every range is handled
-// with integer operations.  Results are the hardware's, bit for bit (NaN: some NaN).
-// To nearest even: the 53-bit significand is cut to FP32's 24 bits (fewer for
-// a subnormal result) and the remainder's carry added.
-__device__ __forceinline__ float f64_to_f32(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned ex = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
-    unsigned b;
-    if (ex - 897u <= 253u) {
-        b = ((ex - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-        b += ((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29;
-    } else if (ex > 896u) {  // too large, infinite or NaN
-        b = 0x7f800000u | ((ex == 0x7ffu && ((hi & 0xfffffu) | lo)) ? 0x400000u : 0u);
-    } else if (ex >= 872u) {  // subnormal result: the significand in units of 2^-149
-        const unsigned long long m = (1ull << 52) | ((unsigned long long)(hi & 0xfffffu) << 32) | lo;
-        const int sh = 29 + (int)(897u - ex);  // 30 .. 54
-        const unsigned long long rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-        b = (unsigned)(m >> sh);
-        b += (rem > half || (rem == half && (b & 1u))) ? 1u : 0u;
-    } else {
-        b = 0u;
-    }
-    return __int_as_float((int)(b | sign));
-}
-// exact: the exponent rebiased, a subnormal number scaled to a normal one first
-__device__ __forceinline__ double f32_to_f64(float x) {
-    const unsigned bx = (unsigned)__float_as_int(x), ex = (bx >> 23) & 0xffu, sign = bx & 0x80000000u;
-    const unsigned b = (ex ? bx : (unsigned)__float_as_int(x * 0x1p64f)) & 0x7fffffffu;
-    const unsigned bias = ex ? (ex == 0xffu ? 0x70000000u : 0x38000000u) : 0x34000000u;
-    return __hiloint2double((int)(sign | (b ? (b >> 3) + bias : 0u)), (int)(b << 29));
-}
 
 constexpr int next_pow2_c(int x) { return x <= 1 ? 1 : 2 * next_pow2_c((x + 1) / 2); }
 
