@@ -192,7 +192,7 @@ __device__ __forceinline__ int32_t other_end(int32_t e, int32_t b, const int32_t
 }
 
 // Best eligible neighbour over the slots [jb, je) of one member, one thread:
-// eight slots at a time, their suitor keys fetched together (fewer
+// four slots at a time, their suitor keys fetched together (fewer
 // dependent round trips than fetching only for improving slots).
 template <bool D64, bool FIRST_PASS>
 __device__ __forceinline__ void scan_slots_thread(int64_t jb, int64_t je, int32_t cur, const int32_t* __restrict__ col,

@@ -137,9 +137,11 @@ __global__ void k_base_mass(int64_t n, const double* __restrict__ deg, int norma
 // Modified Gram-Schmidt in column order, right-looking: step j finishes
 // column j, whose products with the columns after it are then known, and step
 // j + 1 subtracts its share from all of them in the same pass that makes the
-// next products.  The same operations on the same numbers as column-by-column
-// MGS (each column loses its parts along 0, 1, ... in that order), in k passes
-// instead of k (k + 1) / 2 pairs of them.  A thread holds a row, columns are
+// next products: k passes instead of k (k + 1) / 2 pairs of them.  Column-by-
+// column MGS (each column loses its parts along 0, 1, ... in that order) with
+// the normalisation put off: columns stay as they are, their products are
+// divided by the squared norm, and the last pass scales; the results are equal
+// up to rounding.  A thread holds a row, columns are
 // stored one after the other (coalesced; the first pass reads the row-major
 // block and the last writes it), and only the columns that are left are
 // touched.  Bound by the FP64 pipe, k (k + 1) multiply-adds a row (2,097,152 x
