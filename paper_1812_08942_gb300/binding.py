@@ -137,12 +137,15 @@ class Graph:
         self.device = device
         self.stream = stream
         self._torch_stream = None
+        self._index = None
 
     def torch_stream(self):
         """The stream as torch's object (it stays its creator's)."""
         if self._torch_stream is None:
-            self._torch_stream = (torch.cuda.ExternalStream(self.stream, self.device) if self.stream
-                                  else torch.cuda.default_stream(self.device))
+            dev = torch.device(self.device)
+            self._index = torch.cuda.current_device() if dev.index is None else dev.index
+            self._torch_stream = (torch.cuda.ExternalStream(self.stream, self._index) if self.stream
+                                  else torch.cuda.default_stream(self._index))
         return self._torch_stream
 
     def __del__(self):
@@ -161,12 +164,15 @@ def _join(g, *tensors):
     and may free ``tensors``, as after a wait; on g's stream, a tensor of a
     third stream is not given out again before g's stream is done with it.
     (Only device tensors can be held so; the call's host tensors are waited for.)"""
-    s = g.torch_stream()
-    if g.stream != torch.cuda.current_stream(g.device).cuda_stream or not all(t.is_cuda for t in tensors):
-        s.synchronize()
-    else:
-        for t in tensors:
+    s = g._torch_stream or g.torch_stream()
+    if torch._C._cuda_getCurrentRawStream(g._index) != g.stream:
+        s.synchronize() if g.stream is not None else torch.cuda.synchronize(g.device)
+        return
+    for t in tensors:
+        if t.is_cuda:
             t.record_stream(s)
+        else:
+            s.synchronize()
 
 
 # ---------------------------------------------------------------------------
