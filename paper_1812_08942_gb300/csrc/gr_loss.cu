@@ -66,12 +66,16 @@ struct RowLanes {
 __device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
 
+struct NoStep {
+    __device__ void operator()() const {}
+};
 // f(w, x) for every slot of the lane's share of [b, e): x the chunk of the
 // slot's column in src; eight slots in flight (a reduced mesh's row of 14 in
-// two round trips), in slot order per lane
-template <int K, bool LONG, typename F>
+// two round trips), in slot order per lane; step() after each round of eight
+template <int K, bool LONG, typename F, typename Step = NoStep>
 __device__ __forceinline__ void for_slots(const RowLanes<K, LONG>& m, int64_t b, int64_t e,
-                                          const int2* __restrict__ cw, const float* __restrict__ src, F f) {
+                                          const int2* __restrict__ cw, const float* __restrict__ src, F f,
+                                          Step step = Step()) {
     constexpr int U = 8, TS = RowLanes<K, LONG>::TS;
     if (!m.ok) return;
     for (int64_t j = b + m.t; j < e; j += U * TS) {
@@ -86,6 +90,7 @@ __device__ __forceinline__ void for_slots(const RowLanes<K, LONG>& m, int64_t b,
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (j + u * TS < e) f(__int_as_float(v[u].y), x[u]);
+        step();
     }
 }
 
@@ -199,35 +204,40 @@ __device__ __forceinline__ void add_edge(float4& s, float w, const float4& x, co
     s.w = fmaf(w * t, t, s.w);
 }
 
-// S.a += w(e) (x_u - x_v)^2 over blocks g, g + groups, ... of SUM_BLOCK edges
-// of the canonical list; Xq: the lane's chunk of row 0
-template <typename Wt>
-__device__ __forceinline__ void edge_blocks(int64_t m, int64_t g, int64_t groups, const int32_t* __restrict__ eu,
-                                            const int32_t* __restrict__ ev, const float* __restrict__ Xq, int K,
-                                            LaneSums& S, Wt weight) {
+// S.a += w(e) (x_u - x_v)^2 over the canonical list: a warp takes SUM_BLOCK R
+// consecutive edges at a time, each of its R lane groups every R-th of them,
+// four in flight (a block of consecutive edges per group, whose loads lie 64
+// edges apart: forward pass without sweeps on 16 M edges of a power-law graph,
+// 8 columns, 690 us; so 515).  The first end's chunk is loaded again only
+// where the node changes.  Xq: the lane's chunk of row 0.
+template <int R, typename Wt>
+__device__ __forceinline__ void edge_blocks(int64_t m, int64_t warp, int64_t warps, int group,
+                                            const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+                                            const float* __restrict__ Xq, int K, LaneSums& S, Wt weight) {
     constexpr int U = 4;
     static_assert(SUM_BLOCK % U == 0, "a block is whole rounds");
-    for (int64_t b = g * SUM_BLOCK; b < m; b += groups * SUM_BLOCK) {
-        const int64_t e = b + SUM_BLOCK < m ? b + SUM_BLOCK : m;
+    constexpr int64_t STEP = (int64_t)SUM_BLOCK * R;
+    for (int64_t b = warp * STEP; b < m; b += warps * STEP) {
+        const int64_t e = b + STEP < m ? b + STEP : m;
         int32_t cur = -1;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int64_t j = b; j < e; j += U) {
+        for (int64_t j = b + group; j < e; j += U * R) {
             int32_t p[U], q[U];
             float w[U];
             float4 y[U];
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u < e) {
-                    p[u] = __ldg(eu + j + u);
-                    q[u] = __ldg(ev + j + u);
-                    w[u] = weight(j + u);
+                if (j + u * R < e) {
+                    p[u] = __ldg(eu + j + u * R);
+                    q[u] = __ldg(ev + j + u * R);
+                    w[u] = weight(j + u * R);
                 }
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u < e) y[u] = ld4(Xq + (int64_t)q[u] * K);
+                if (j + u * R < e) y[u] = ld4(Xq + (int64_t)q[u] * K);
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (j + u < e) {
+                if (j + u * R < e) {
                     if (p[u] != cur) x = ld4(Xq + (int64_t)(cur = p[u]) * K);
                     add_edge(S.a.open, w[u], x, y[u]);
                 }
@@ -291,9 +301,7 @@ __global__ void __launch_bounds__(LT, ROW_BLOCKS) k_fine_quotients(int64_t n, co
         Rf[threadIdx.x] = (float)(red[threadIdx.x] / red[K + threadIdx.x]);
 }
 
-// The same with the edges in blocks of SUM_BLOCK for graphs that may have long
-// rows: G lanes take a block of consecutive edges, four in flight; the first
-// end's row is loaded again only where it changes.
+// The same with the edges in blocks for graphs that may have long rows
 template <int K>
 __global__ void __launch_bounds__(LT) k_fine_edges(int64_t n, int64_t m, const int32_t* __restrict__ eu,
                                                    const int32_t* __restrict__ ev, const double* __restrict__ ew,
@@ -304,13 +312,14 @@ __global__ void __launch_bounds__(LT) k_fine_edges(int64_t n, int64_t m, const i
     constexpr int RPW = RowLanes<K, false>::RPW;
     __shared__ float4 closed[2][LT];
     LaneSums S(closed);
-    const int64_t groups = (((int64_t)gridDim.x * LT) >> 5) * RPW;
-    const int64_t g = L.ok ? (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + L.seg : n + m;  // past both ends
+    const int64_t warp = ((int64_t)blockIdx.x * LT + threadIdx.x) >> 5, warps = ((int64_t)gridDim.x * LT) >> 5;
     const float* Xq = X + L.q * 4;
-    edge_blocks(m, g, groups, eu, ev, Xq, K, S, [&](int64_t e) { return f64_to_f32(__ldg(ew + e)); });
-    for (int64_t p = g; p < n; p += groups) {
-        add_squares(S.b.open, ld4(Xq + p * K));
-        S.count(1);
+    if (L.ok) {
+        edge_blocks<RPW>(m, warp, warps, L.seg, eu, ev, Xq, K, S, [&](int64_t e) { return f64_to_f32(__ldg(ew + e)); });
+        for (int64_t p = warp * RPW + L.seg; p < n; p += warps * RPW) {
+            add_squares(S.b.open, ld4(Xq + p * K));
+            S.count(1);
+        }
     }
     if (finish_cols<K, false>(L, S.a.total(), S.b.total(), part, counter, red) && threadIdx.x < K)
         Rf[threadIdx.x] = (float)(red[threadIdx.x] / red[K + threadIdx.x]);
@@ -486,15 +495,19 @@ __device__ __forceinline__ void scale_control(const ScaleStep& st, float loss) {
 // every row's slots (each edge twice), sum M (y - mu)^2; in the last block
 // the loss and the adjoint's coefficients
 //   coef[0..K) = 2 g / Q, [K..2K) = 2 g N / Q^2, [2K..3K) = g / Q, [3K..4K) = mu,
-// g = d loss / d R_c.  LY: L y is stored.  LISTED (graphs that may have long
-// rows): the squared differences come from the edge list and its weights w, in
-// blocks; only L y goes through the rows.
+// g = d loss / d R_c.  LY: L y is stored.  Where rows may be long, blocks are
+// closed within the rows (CLOSED_ROWS, with L y, which walks them anyway: a pass
+// over the edges beside it cost the gradient on a reduced graph of 13,152 nodes
+// and 14.6 M edges, 16 columns, 4,335 us for 3,620), or the squared differences
+// come from the edge list and its weights w in blocks (EDGE_LIST: no row is one
+// group's).
+enum QuotientMode { SHORT_ROWS, CLOSED_ROWS, EDGE_LIST };
 struct EdgeList {
     int64_t m = 0;
     const int32_t *eu = nullptr, *ev = nullptr;
     const float* w = nullptr;
 };
-template <int K, bool LONG, bool LY, bool LISTED>
+template <int K, bool LONG, bool LY, QuotientMode MODE>
 __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __restrict__ rowptr,
                                                   const int2* __restrict__ cw, EdgeList E, const float* __restrict__ y,
                                                   const float* __restrict__ mass, const double* __restrict__ mu,
@@ -514,33 +527,35 @@ __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __re
     }
     const int64_t stride = (((int64_t)gridDim.x * LT) >> 5) * RPW;
     const int64_t first = (((int64_t)blockIdx.x * LT + threadIdx.x) >> 5) * RPW + m.seg;
-    if constexpr (LISTED) {
-        // a long row's sub-groups take blocks in turn
-        constexpr int TS = RowLanes<K, LONG>::TS;
+    if constexpr (MODE == EDGE_LIST) {
+        // (a long row's sub-groups are groups here)
+        constexpr int R = RPW * RowLanes<K, LONG>::TS;
         if (m.ok)
-            edge_blocks(E.m, first * TS + m.t, stride * TS, E.eu, E.ev, y + m.q * 4, K, S,
-                        [&](int64_t e) { return __ldg(E.w + e); });
+            edge_blocks<R>(E.m, first / RPW, stride / RPW, m.seg + m.t, E.eu, E.ev, y + m.q * 4, K, S,
+                           [&](int64_t e) { return __ldg(E.w + e); });
     }
     for (int64_t A = first; A < n; A += stride) {
         float4 ya = make_float4(zero, zero, zero, zero), l = ya;
         if (m.ok) ya = ld4(y + A * K + m.q * 4);
-        if constexpr (LY || !LISTED) {
+        if constexpr (LY || MODE != EDGE_LIST) {
             const int64_t b = rowptr[A], e = rowptr[A + 1];
             for_slots<K, LONG>(m, b, e, cw, y, [&](float w, const float4& x) {
                 float d = ya.x - x.x, wd = w * d;
-                if (!LISTED) S.a.open.x = fmaf(wd, d, S.a.open.x);
+                if (MODE != EDGE_LIST) S.a.open.x = fmaf(wd, d, S.a.open.x);
                 l.x += wd;
                 d = ya.y - x.y, wd = w * d;
-                if (!LISTED) S.a.open.y = fmaf(wd, d, S.a.open.y);
+                if (MODE != EDGE_LIST) S.a.open.y = fmaf(wd, d, S.a.open.y);
                 l.y += wd;
                 d = ya.z - x.z, wd = w * d;
-                if (!LISTED) S.a.open.z = fmaf(wd, d, S.a.open.z);
+                if (MODE != EDGE_LIST) S.a.open.z = fmaf(wd, d, S.a.open.z);
                 l.z += wd;
                 d = ya.w - x.w, wd = w * d;
-                if (!LISTED) S.a.open.w = fmaf(wd, d, S.a.open.w);
+                if (MODE != EDGE_LIST) S.a.open.w = fmaf(wd, d, S.a.open.w);
                 l.w += wd;
+            }, [&] {
+                if (MODE == CLOSED_ROWS) S.count(8);  // for_slots' round
             });
-            if (!LISTED) S.terms += (unsigned)(e - b);
+            if (MODE == SHORT_ROWS) S.terms += (unsigned)(e - b);
         }
         if constexpr (LY) {
             join_row<K, LONG>(l);
@@ -564,7 +579,7 @@ __global__ void __launch_bounds__(LT) k_quotients(int64_t n, const int64_t* __re
     if (k >= 32) return;  // the first warp: a column per lane
     double s = 0.0;
     if (k < K) {
-        const double Ns = LISTED ? red[k] : 0.5 * red[k], Qs = red[K + k], f = (double)Rf[k];
+        const double Ns = MODE == EDGE_LIST ? red[k] : 0.5 * red[k], Qs = red[K + k], f = (double)Rf[k];
         const double Rc = Ns / Qs, r = Rc / f - 1.0;
         s = r * r;
         if (coef) {
@@ -839,8 +854,8 @@ gr_status coarse_k(gr_ctx* cc, int S, double omega, const float* y0, const float
                                  adjoint ? W.coef : nullptr, st);
         count_launch();
     };
-    if (W.short_parts) adjoint ? quotients(k_quotients<K, LONG, true, false>) : quotients(k_quotients<K, LONG, false, false>);
-    else adjoint ? quotients(k_quotients<K, LONG, true, true>) : quotients(k_quotients<K, LONG, false, true>);
+    if (W.short_parts) adjoint ? quotients(k_quotients<K, LONG, true, SHORT_ROWS>) : quotients(k_quotients<K, LONG, false, SHORT_ROWS>);
+    else adjoint ? quotients(k_quotients<K, LONG, true, CLOSED_ROWS>) : quotients(k_quotients<K, LONG, false, EDGE_LIST>);
     GR_TRY_CUDA(cc, cudaGetLastError(), "loss");
     return GR_OK;
 }
