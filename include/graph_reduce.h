@@ -132,10 +132,11 @@ gr_status graph_reduce_smooth_noalloc(gr_ctx* ctx, int K, int sweeps, double ome
  *                    warp's group of 32 / lanes-per-row rows would hold over
  *                    128 slots; FP64 and BF16 blocks of a created graph
  *                    whose rows hold at most 64 slots below and above the
- *                    diagonal are excepted, unless it has too few rows for
- *                    its mean degree to fill the SMs: more than 1.5, BF16
- *                    0.5, times the rows per SM, and for K >= 8 more than
- *                    45); else the band kernel when the graph has at
+ *                    diagonal are excepted, unless its rows are too few to
+ *                    fill the SMs at its mean degree: more than 0.7, BF16
+ *                    0.6, times the 16-byte row chunks per SM (at most 4
+ *                    times the rows), and for K >= 8 more than 45); else the
+ *                    band kernel when the graph has at
  *                    least 640 rows per SM (enough for a chunk of bands on
  *                    every SM) and is in a banded order: at least half of
  *                    its slots within a halo of at most 1,024 rows that fits

@@ -503,7 +503,7 @@ __device__ __forceinline__ void sweep_row_body(
         }
     }
     const int stride = ((gridDim.x * blockDim.x) >> 5) * RPW;
-    // (eight slots in flight: fewer rows than lanes, spread over the blocks)
+    // (eight slots in flight: few rows, a block's warps far apart)
     const int wid = U == 8 ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int row = wid * RPW + (lane_ok ? seg : 0);
     const T* Aq = Ain + q * E;
@@ -663,12 +663,15 @@ struct SweepScratch {
 //                  BF16  K = 16  degree 60   129 | 204    120   211 | 341
 //   20,000 rows    FP64  K = 8   degree 60    37 | 60     124    57 | 76
 //                  BF16  K = 8   degree 60    21 | 24      80    27 | 25
+//                  BF16  K = 24  degree 60    27 | 31     100    35 | 41
 //   5,000 rows     FP64  K = 4   degree 40  20.5 | 20.6    60  24.7 | 21.7
 //                  BF16  K = 8   degree 40  16.4 | 14.8    80  20.5 | 16.5
+//                  BF16  K = 24  degree 40  14.5 | 16.6    80  18.5 | 19.6
 //   1,000 rows     FP64  K = 4   degree 40  20.5 | 14.4   100  30.9 | 15.5
 //                  BF16  K = 8   degree 40  16.0 | 14.5   100  21.6 | 14.5
-// The line: a mean degree of 1.5 (FP64) or 0.5 (BF16) times the rows per SM,
-// and up to 45 in any case for K of 8 and more, where at most 4 us are lost.
+// The line: a mean degree of 0.7 (FP64) or 0.6 (BF16) times the row chunks per
+// SM (at most 4 times the rows), and up to 45 in any case for K of 8 and more,
+// where at most 4 us are lost.
 // FP32 blocks keep the rule by degree alone, and with it the rounding of their
 // column sums.
 template <typename T, int K>
@@ -682,7 +685,8 @@ static bool stream_wide(const gr_ctx* c) {
     if (!mean_long<T, K>(c)) return false;
     if (sizeof(T) == 4 || !c->short_rows) return true;
     const double avg = 2.0 * (double)c->m / (double)c->n;
-    const double filled = (sizeof(T) == 8 ? 1.5 : 0.5) * (double)c->n / c->num_sms;
+    constexpr double PER = (sizeof(T) == 8 ? 0.7 : 0.6) * RowLayout<T, K>::G;
+    const double filled = (PER < 4.0 ? PER : 4.0) * (double)c->n / c->num_sms;
     return avg > filled && !(K >= 8 && avg <= 45.0);
 }
 
@@ -873,22 +877,15 @@ static cudaError_t launch_sweep_row(gr_ctx* c, const SweepPlan& P, const T* Ain,
     const typename SlotOf<T>::type* slots;
     if constexpr (sizeof(T) == 8) slots = P.cw64;
     else slots = c->cw32;
-    // Rows of a dozen slots and more that leave the chip half empty: eight
-    // slots in flight, and one warp a block while there are blocks for it
-    // (2,000 rows of 40 slots, FP64, K = 8: 22 us with two slots and full blocks,
-    // 18.5 now; streaming 16.4).
+    // Rows of a dozen slots and more, too few for a block on every SM: eight
+    // slots in flight and the warps spread over the SMs (2,000 rows of 40
+    // slots, FP64, K = 8: 22 us with two slots and full blocks, 18.5 so;
+    // streaming 16.4).
     if constexpr (sizeof(T) != 4) {
-        static int bps8 = 0;
-        if (!bps8) {
-            GR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps8, k_sweep_row<T, K, 8>, SM_THREADS, 0));
-            if (bps8 < 1) bps8 = 1;
-        }
-        if (mean_long<T, K>(c) && want <= (int64_t)c->num_sms * bps8 && slots_step_fits(2 * (unsigned long long)c->m, 8)) {
-            if (want < c->num_sms) {
-                const int64_t warps = ceil_div(c->n, (int64_t)(32 / RowLayout<T, K>::G));
-                grid = (int)(warps < c->num_sms ? warps : c->num_sms);
-                if (grid > part_cap) grid = part_cap;
-            }
+        if (mean_long<T, K>(c) && want < c->num_sms && slots_step_fits(2 * (unsigned long long)c->m, 8)) {
+            const int64_t warps = ceil_div(c->n > 0 ? c->n : 1, (int64_t)(32 / RowLayout<T, K>::G));
+            grid = (int)(warps < c->num_sms ? warps : c->num_sms);
+            if (grid > part_cap) grid = part_cap;
             k_sweep_row<T, K, 8><<<grid, SM_THREADS, 0, c->stream>>>(c->n, c->rowptr, slots, Ain, Aout, omega, st_in,
                                                                      part, counter, st_out);
             count_launch();
