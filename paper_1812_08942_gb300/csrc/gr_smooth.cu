@@ -1425,7 +1425,10 @@ __device__ __forceinline__ void load_chunk_rw(const T* p, typename AccOf<T>::typ
 // each; the neighbours have other colours and are not written by this launch.
 // Bound by the gathers' round trips: four slots in flight (colouring and five
 // sweeps of a 101 x 89 x 75 mesh, K = 16: 959 us with four, 979 with two,
-// 1,042 with eight, whose registers cost resident warps).  (Column sums ended
+// 1,042 with eight, whose registers cost resident warps).  FP64 two: a multiply-
+// add of a slot past the row's end takes the FP64 pipe like any other (three
+// sweeps of a path of 500,000 nodes, K = 16: 668 us with four, 582 with two; the
+// same mesh 1,191 and 1,057; rows of 100 slots 2,800 and 2,613).  (Column sums ended
 // in these launches too: 8 us of finish for each of the six colours of a mesh,
 // where a pass of its own takes 21 once.)
 template <typename T, int K>
@@ -1436,7 +1439,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_gs_class(int64_t cnt, const int3
     using Slot = typename SlotOf<T>::type;
     using L = RowLayout<T, K>;
     using Acc = typename AccOf<T>::type;
-    constexpr int E = L::E, G = L::G, RPW = 32 / G, U = 4;
+    constexpr int E = L::E, G = L::G, RPW = 32 / G, U = sizeof(T) == 8 ? 2 : 4;
     const int lane = threadIdx.x & 31, seg = lane / G, q = lane % G;
     if (seg >= RPW) return;
     const int64_t r = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RPW + seg;
