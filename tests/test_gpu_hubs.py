@@ -123,3 +123,22 @@ def test_colouring_of_many_leaves(gpu_lib, oracle_mod):
         col, nc = gr.graph_reduce_colour(G, seed)
         ref, rnc = oracle_mod.colour(n, u, v, seed)
         assert nc == rnc and np.array_equal(col.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("hub_deg", [2100, 8000])
+@pytest.mark.parametrize("at", ["first", "last"])
+def test_csr_rows(gpu_lib, oracle_mod, hub_deg, at):
+    """Degrees and row weights of hubs on a sparse graph, seen through FP64
+    sweeps: 1e-12, the bar of the smoothing parity tests."""
+    gr = gpu_lib
+    n, K, S = 9001, 8, 3
+    g = _hubs(n, 4, 2, hub_deg, 17, at)
+    G = gr.graph_reduce_create(n, g.u, g.v, g.w)
+    X = torch.empty(n, K, dtype=torch.float64, device=DEV)
+    gr.graph_reduce_smooth(G, X, S)
+    ref = oracle_mod.smooth(n, g.u, g.v, g.w, K, S)
+    assert (np.linalg.norm(X.cpu().numpy() - ref, axis=0) / np.linalg.norm(ref, axis=0)).max() <= 1e-12
+    agg = torch.from_numpy((np.arange(n) // 3).astype(np.int32)).to(DEV)
+    u, v, w = gr.graph_reduce_get_edges(gr.graph_reduce_coarsen(G, agg, -(-n // 3)), on_host=True)
+    ur, vr, wr = oracle_mod.coarsen(n, g.u, g.v, g.w, agg.cpu().numpy(), -(-n // 3))
+    assert np.array_equal(u.numpy(), ur) and np.array_equal(v.numpy(), vr) and np.array_equal(w.numpy(), wr)
