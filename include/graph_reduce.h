@@ -135,8 +135,8 @@ gr_status graph_reduce_smooth_noalloc(gr_ctx* ctx, int K, int sweeps, double ome
  *                    diagonal are excepted, unless its rows are too few to
  *                    fill the SMs at its mean degree: more than 0.7, BF16
  *                    0.6, times the 16-byte row chunks per SM (at most 4
- *                    times the rows), and for K >= 8 more than 45); else the
- *                    band kernel when the graph has at
+ *                    times the rows), and, but for FP64 with K = 4, more
+ *                    than 45); else the band kernel when the graph has at
  *                    least 640 rows per SM (enough for a chunk of bands on
  *                    every SM) and is in a banded order: at least half of
  *                    its slots within a halo of at most 1,024 rows that fits

@@ -670,8 +670,8 @@ struct SweepScratch {
 //   1,000 rows     FP64  K = 4   degree 40  20.5 | 14.4   100  30.9 | 15.5
 //                  BF16  K = 8   degree 40  16.0 | 14.5   100  21.6 | 14.5
 // The line: a mean degree of 0.7 (FP64) or 0.6 (BF16) times the row chunks per
-// SM (at most 4 times the rows), and up to 45 in any case for K of 8 and more,
-// where at most 4 us are lost.
+// SM (at most 4 times the rows), and up to 45 in any case but FP64 with K = 4:
+// at most 4 us are lost there.
 // FP32 blocks keep the rule by degree alone, and with it the rounding of their
 // column sums.
 template <typename T, int K>
@@ -687,7 +687,7 @@ static bool stream_wide(const gr_ctx* c) {
     const double avg = 2.0 * (double)c->m / (double)c->n;
     constexpr double PER = (sizeof(T) == 8 ? 0.7 : 0.6) * RowLayout<T, K>::G;
     const double filled = (PER < 4.0 ? PER : 4.0) * (double)c->n / c->num_sms;
-    return avg > filled && !(K >= 8 && avg <= 45.0);
+    return avg > filled && !((K >= 8 || sizeof(T) == 2) && avg <= 45.0);
 }
 
 template <typename T>

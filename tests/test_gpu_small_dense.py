@@ -20,7 +20,7 @@ def _band(n, half, seed=0):
 
 
 @pytest.mark.parametrize("n,half,K,row64,row16", [(1000, 50, 8, False, False), (1000, 20, 8, True, True),
-                                                  (1000, 20, 4, False, False), (12000, 40, 8, True, False),
+                                                  (1000, 20, 4, False, True), (12000, 40, 8, True, False),
                                                   (60000, 60, 16, True, True)])
 def test_rows_for_every_sm(gpu_lib, n, half, K, row64, row16):
     gr = gpu_lib
