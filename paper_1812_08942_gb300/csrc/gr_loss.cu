@@ -206,22 +206,26 @@ __device__ __forceinline__ void add_edge(float4& s, float w, const float4& x, co
 
 // S.a += w(e) (x_u - x_v)^2 over the canonical list: a warp takes SUM_BLOCK R
 // consecutive edges at a time, each of its R lane groups every R-th of them,
-// four in flight (a block of consecutive edges per group, whose loads lie 64
+// EDGE_FLIGHT in flight (a block of consecutive edges per group, whose loads lie 64
 // edges apart: forward pass without sweeps on 16 M edges of a power-law graph,
 // 8 columns, 690 us; so 515).  The first end's chunk is loaded again only
 // where the node changes.  Xq: the lane's chunk of row 0.
+constexpr int EDGE_FLIGHT = 4;
 template <int R, typename Wt>
 __device__ __forceinline__ void edge_blocks(int64_t m, int64_t warp, int64_t warps, int group,
                                             const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
                                             const float* __restrict__ Xq, int K, LaneSums& S, Wt weight) {
-    constexpr int U = 4;
+    constexpr unsigned U = EDGE_FLIGHT;
     static_assert(SUM_BLOCK % U == 0, "a block is whole rounds");
-    constexpr int64_t STEP = (int64_t)SUM_BLOCK * R;
+    // shorter blocks where there are too few edges for all warps (m < 2^31)
+    unsigned per = (unsigned)((m + warps * R - 1) / (unsigned)(warps * R));
+    per = (per + U - 1) / U * U;
+    const int64_t STEP = (int64_t)(per < SUM_BLOCK ? per : SUM_BLOCK) * R;
     for (int64_t b = warp * STEP; b < m; b += warps * STEP) {
         const int64_t e = b + STEP < m ? b + STEP : m;
         int32_t cur = -1;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int64_t j = b + group; j < e; j += U * R) {
+        for (int64_t j = b + group; j < e; j += (int64_t)U * R) {
             int32_t p[U], q[U];
             float w[U];
             float4 y[U];
@@ -763,7 +767,7 @@ gr_status fine_quotients(gr_ctx* f, const float* X, double* part, unsigned* coun
 
 template <int K>
 gr_status fine_edges(gr_ctx* f, const float* X, double* part, unsigned* counter, float* Rf) {
-    const int64_t blocks = ceil_div(f->m, SUM_BLOCK), work = blocks > f->n ? blocks : f->n;
+    const int64_t rounds = ceil_div(f->m, EDGE_FLIGHT), work = rounds > f->n ? rounds : f->n;
     k_fine_edges<K><<<row_grid<K, false>(f, work), LT, 0, f->stream>>>(f->n, f->m, f->eu, f->ev, f->ew, X, part,
                                                                       counter, Rf);
     count_launch();
@@ -848,14 +852,21 @@ gr_status coarse_k(gr_ctx* cc, int S, double omega, const float* y0, const float
     E.eu = cc->eu;
     E.ev = cc->ev;
     E.w = W.w;
-    auto quotients = [&](auto kern) {
-        kern<<<grid, LT, 0, s>>>(nc, cc->rowptr, W.cw, E, y, mass, W.mu, W.part, W.counter, Rf,
-                                 adjoint ? grad_loss : nullptr, loss_out, adjoint ? W.yb1 : nullptr,
-                                 adjoint ? W.coef : nullptr, st);
+    auto quotients = [&](auto kern, unsigned blocks) {
+        kern<<<blocks, LT, 0, s>>>(nc, cc->rowptr, W.cw, E, y, mass, W.mu, W.part, W.counter, Rf,
+                                   adjoint ? grad_loss : nullptr, loss_out, adjoint ? W.yb1 : nullptr,
+                                   adjoint ? W.coef : nullptr, st);
         count_launch();
     };
-    if (W.short_parts) adjoint ? quotients(k_quotients<K, LONG, true, SHORT_ROWS>) : quotients(k_quotients<K, LONG, false, SHORT_ROWS>);
-    else adjoint ? quotients(k_quotients<K, LONG, true, CLOSED_ROWS>) : quotients(k_quotients<K, LONG, false, EDGE_LIST>);
+    if (W.short_parts) {
+        adjoint ? quotients(k_quotients<K, LONG, true, SHORT_ROWS>, grid)
+                : quotients(k_quotients<K, LONG, false, SHORT_ROWS>, grid);
+    } else if (adjoint) {
+        quotients(k_quotients<K, LONG, true, CLOSED_ROWS>, grid);
+    } else {  // a round of edges for every warp, if there are as many
+        const int64_t rounds = ceil_div(cc->m, EDGE_FLIGHT * RowLanes<K, LONG>::TS);
+        quotients(k_quotients<K, LONG, false, EDGE_LIST>, row_grid<K, LONG>(cc, rounds > nc ? rounds : nc));
+    }
     GR_TRY_CUDA(cc, cudaGetLastError(), "loss");
     return GR_OK;
 }
